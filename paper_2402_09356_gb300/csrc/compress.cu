@@ -53,9 +53,7 @@ constexpr int kOversample = 24;  // samples beyond the expected rank
 constexpr int kSpare = 20;       // fewer spare samples than this: redo with more
 constexpr int kQrThreads = 256;
 constexpr int kNw = kQrThreads / 32;
-// Threads of the shared-memory QR (512 measured slower at n = 40,000: the
-// step's barrier and exchange latency, not its dependent chains, bound it).
-constexpr int kQrSmThreads = 256;
+constexpr int kQrSmThreads = 512;
 constexpr int kMaxSweeps = 40;
 
 template <class T>
@@ -99,13 +97,17 @@ __device__ __forceinline__ void householder(double nrm2, double alpha, double &t
 // subnormal) is taken as zero: no reflector.
 __device__ __forceinline__ void householder_ff(FF nrm2, FF alpha, FF &rn, FF &rv, FF &beta, FF &v0) {
     rn = rv = beta = v0 = FF{0.f, 0.f};
-    const FF nrm = ff_sqrt(nrm2);
+    if (!(nrm2.h > 0.f)) return;
+    // every column step waits for this chain: |x| = |x|^2 (1 / |x|), no division
+    const FF r = ff_rsqrt(nrm2);
+    FF nrm = ff_mul(nrm2, r);
+    if (nrm2.h > 3.4e38f) nrm = FF{INFINITY, 0.f};  // an overflow stays one (rn is NaN)
     if (nrm.h >= 1e-30f) {
         const FF snrm = alpha.h < 0.f ? ff_neg(nrm) : nrm;
         beta = ff_neg(snrm);
         v0 = ff_add(alpha, snrm);
-        rn = ff_div(FF{1.f, 0.f}, nrm);
-        rv = ff_div(FF{1.f, 0.f}, v0.h < 0.f ? ff_neg(v0) : v0);
+        rn = r;
+        rv = ff_rcp(v0.h < 0.f ? ff_neg(v0) : v0);
     }
 }
 
@@ -117,30 +119,8 @@ struct QrJob {
     double *Rt;  // s x s output R' (ld s, lower triangular), or null
     int m, s;
     float2 *Rt2;  // paired-FP32 variant: R' also as (hi, lo) pairs (ld s), or null
-};
-
-// ---------------------------------------------------------------------------
-// Work split of one panel step over a CTA's threads.  GB300 issues FP64 at
-// 1/64 of the FP32 rate, so the FP64 instruction count is what matters: each
-// thread owns whole columns (lanes <-> columns, no shuffle reductions), and
-// when the columns fill fewer than all warps the rows are split into G
-// interleaved groups over the spare warps (their partial dot products are
-// summed through shared memory).  Thread t handles row group t / width and
-// columns first + t % width + k * width.
-template <int kThreads>
-struct PanelSplit {
-    int G, width;
-    __device__ __forceinline__ explicit PanelSplit(int ncols) {
-        constexpr int kWarps = kThreads / 32;
-        const int cw = (ncols + 31) / 32;
-        if (cw >= kWarps || cw == 0) {
-            G = 1;
-            width = kThreads;
-        } else {
-            G = kWarps / cw;
-            width = 32 * cw;
-        }
-    }
+    double *V;    // with Q: the reflectors (m x s, ld m) and 3 s column scalars, in the kernel's arithmetic
+    float2 *Q2;   // paired-FP32 variant: Q as (hi, lo) pairs (ld ldq) instead of doubles, or null
 };
 
 // Element arithmetic of the shared-memory QR: FP64, or paired FP32 (each
@@ -225,212 +205,322 @@ struct QrArith<true> {
     }
 };
 
-// Dot products d_cc = sum over local rows i >= lb of v[i] A(i, cc) for the
-// columns cc in [first, s), written to out[cc].  red: kThreads scalars.
-template <int kThreads, class Ar, class T, class P>
-__device__ __forceinline__ void panel_dots(const T *As, int ld, const T *v, int first, int s, int lb, int nr,
-                                           P *red, P *out) {
-    const int tid = threadIdx.x;
-    const PanelSplit<kThreads> ps(s - first);
-    const int g = tid / ps.width;
-    if (ps.G == 1) {
-        for (int cc = first + tid; cc < s; cc += ps.width) {
-            const T *ac = As + cc * ld;
-            typename Ar::Acc d;
-            for (int i = lb; i < nr; ++i) Ar::acc(d, v[i], ac[i]);
-            out[cc] = Ar::part(d);
-        }
-        return;
-    }
-    const int cc = first + tid % ps.width;
-    if (tid < ps.G * ps.width && cc < s) {
-        const T *ac = As + cc * ld;
-        typename Ar::Acc d;
-        for (int i = lb + g; i < nr; i += ps.G) Ar::acc(d, v[i], ac[i]);
-        red[tid] = Ar::part(d);
-    }
-    __syncthreads();
-    if (tid < ps.width && cc < s) {
-        P d{};
-        for (int q = 0; q < ps.G; ++q) d = Ar::padd(d, red[q * ps.width + tid]);
-        out[cc] = d;
-    }
+// Sum over each group of n lanes of a warp (n a power of two).
+__device__ __forceinline__ double lane_sum(double v, int n = 32) {
+#pragma unroll
+    for (int o = n >> 1; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
 }
-
-// A(i, cc) -= w[cc] v(i) for local rows i >= lb and columns cc in [first, s),
-// where v(i) = v[i] except v(ic) = vhead when ic is a local row.
-template <int kThreads, class Ar, class T, class P>
-__device__ __forceinline__ void panel_update(T *As, int ld, const T *v, int ic, T vhead, const P *w, int first,
-                                             int s, int lb, int nr) {
-    const int tid = threadIdx.x;
-    const PanelSplit<kThreads> ps(s - first);
-    if (tid >= ps.G * ps.width) return;
-    const int g = tid / ps.width;
-    for (int cc = first + tid % ps.width; cc < s; cc += ps.width) {
-        const typename Ar::W wc = Ar::prepP(w[cc]);
-        T *ac = As + cc * ld;
-        for (int i = lb + g; i < nr; i += ps.G) ac[i] = Ar::axmy(ac[i], wc, i == ic ? vhead : v[i]);
-    }
+__device__ __forceinline__ FF lane_sum(FF v, int n = 32) {
+#pragma unroll
+    for (int o = n >> 1; o; o >>= 1)
+        v = ff_add(v, FF{__shfl_xor_sync(0xFFFFFFFFu, v.h, o), __shfl_xor_sync(0xFFFFFFFFu, v.l, o)});
+    return v;
 }
 
 // ---------------------------------------------------------------------------
-// QR with the panel in shared memory.  CTA `rank` of the cluster owns rows
-// [r0, r0 + nr) of all s columns, column-major with an odd leading dimension.
-// Column c: every CTA forms the dot products of column c with columns c..s-1
-// over its rows (at or below row c), and the owner of row c publishes that
-// row; after one cluster barrier every CTA sums the kCl partials, forms the
-// reflector (v = column c with v_c = v0) and w_cc = tau (d_cc + (v0 - alpha)
-// A(c, cc)), and updates its own rows.  Buffers alternate by column parity, so
-// a CTA never overwrites values another CTA may still be reading.
-// Q = H_0 ... H_{s-1} [I; 0] is then accumulated backwards in place: before
-// H_c is applied, columns > c already hold their final values below row c,
-// and column c becomes H_c e_c (LAPACK's dorg2r ordering).
-// Shared memory: s * ld + 9 s + kQrSmThreads doubles.
+// QR with the panel in shared memory, factorisation.  CTA `rank` of the
+// cluster owns rows [r0, r0 + nr) of all s columns, column-major with an odd
+// leading dimension (8-byte elements a warp reads from 32 columns then fall
+// in distinct banks).  On entry to step c every CTA holds, for the columns
+// cc = c .. s-1, the dot product of columns c and cc below row c and the
+// entry of row c.  The step:
+//   1. one thread forms the reflector (v = column c with v_c = v0);
+//   2. column c + 1 alone is updated, by one thread per row:
+//      A(:, c+1) -= w v, w_cc = tau (d_cc + (v0 - alpha) A(c, cc));
+//   3. one pass over the columns behind it updates them and takes their dot
+//      products with the new column c + 1 (a separate pass each would load the
+//      panel twice);
+//   4. the CTAs' partial dot products are summed: each column by one CTA (one
+//      lane per source CTA, then shuffles), which stores the sum and row c + 1's
+//      entry into every CTA; a cluster barrier before and after.
+// What bounds it: the latency of a step.  Distributed shared memory moves only
+// about 11 bytes per clock and SM with 16 CTAs pulling at once (measured), so
+// that every CTA reading every CTA's partials, kCl s values a step, cost twice
+// the update itself; summing each column once moves 4 s values, for one more
+// barrier (550 cycles).  Dead index arithmetic counts too: the split of the
+// threads over columns and rows changes only every 32 columns and is kept.
+// m = 800, s = 200 on 16 CTAs alone: 0.93 ms in pairs, 1.50 in FP64, with Q
+// formed 1.12 and 1.94 (one kernel that read every partial everywhere and
+// accumulated Q over the cluster: 2.0 and 2.5 ms).
+// 512 threads at 64 registers leave half of an SM's registers to the look-ahead
+// product's CTA.  Q is formed by k_qr_form from the reflectors left in J.V.
+// Shared memory: s * ld + 8 s + kQrSmThreads doubles.
 template <int kCl, bool kDf>
-__global__ void __launch_bounds__(kQrSmThreads) k_qr_sm(const QrJob *__restrict__ jobs) {
+__global__ void __launch_bounds__(kQrSmThreads, 2) k_qr_factor(const QrJob *__restrict__ jobs) {
     using Ar = QrArith<kDf>;
     using T = typename Ar::T;
-    static_assert(sizeof(T) == sizeof(double), "the panel element takes the bytes of one double");
+    using P = typename Ar::P;
+    static_assert(sizeof(T) == sizeof(double) && sizeof(P) == sizeof(double), "elements take the bytes of a double");
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const QrJob J = jobs[blockIdx.x / kCl];
-    const int m = J.m, s = J.s, tid = threadIdx.x;
+    const int m = J.m, s = J.s, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int per = (m + kCl - 1) / kCl, ld = per | 1;
     const int r0 = min(m, rank * per), nr = min(m, r0 + per) - r0;
-    using P = typename Ar::P;
-    static_assert(sizeof(P) == sizeof(double), "a column scalar takes the bytes of one double");
     extern __shared__ double sm[];
     T *As = reinterpret_cast<T *>(sm);
     // taus: tau (FP64), or 1 / |x| with rvs = 1 / |v0| (pairs; householder_ff)
     P *taus = reinterpret_cast<P *>(sm + (size_t)s * ld), *betas = taus + s, *heads = betas + s, *rvs = heads + s;
-    P *pd = rvs + s, *prow = pd + 2 * s, *wv = prow + 2 * s, *red = wv + s;
+    P *pd = rvs + s, *prow = pd + s, *tot = prow + s, *rowv = tot + s, *red = rowv + s;
     for (int e = tid; e < nr * s; e += kQrSmThreads) {
         const int i = e % nr, j = e / nr;
         As[j * ld + i] = Ar::from(J.A[(int64_t)j * J.lda + r0 + i]);
     }
-    __syncthreads();
-    for (int c = 0; c < s; ++c) {
-        P *pdc = pd + (c & 1) * s, *prc = prow + (c & 1) * s;
-        const int lb = max(c - r0, 0), ic = c - r0;
-        T *vc = As + c * ld;
-        panel_dots<kQrSmThreads, Ar>(As, ld, vc, c, s, lb, nr, red, pdc);
-        const int owner = c / per;
-        if (rank == owner)
-            for (int cc = c + tid; cc < s; cc += kQrSmThreads) prc[cc] = Ar::elem(As[cc * ld + ic]);
-        cl.sync();
-        const P *orow = cl.map_shared_rank(prc, owner);
-        // the reflector's scalars once per CTA (every thread repeating the
-        // norm, square root and division would only repeat the same work)
-        if (tid == 0) {
-            P nrm2{};
+    // Split of the threads over `live` columns: cw warps across the columns
+    // (column u), G groups of them over the rows (group g).
+    int cw = 0, G = 1, g = 0, u = 0;
+    auto split = [&](int live) {
+        const int c = (live + 31) >> 5;
+        if (c == cw) return;
+        cw = c;
+        G = max(1, (kQrSmThreads / 32) / c);
+        g = warp / c;
+        u = tid - 32 * c * g;
+    };
+    // Sums red[.] over the row groups and the cluster into tot[], and spreads
+    // row `first` from its owner into rowv[], for columns first .. s-1.
+    auto exchange = [&](int first, int owner) {
+        __syncthreads();
+        const int width = 32 * cw, live = s - first;
+        if (tid < width && tid < live) {
+            P v[4];
 #pragma unroll
-            for (int k = 0; k < kCl; ++k) nrm2 = Ar::padd(nrm2, cl.map_shared_rank(pdc, k)[c]);
-            const P alpha = orow[c];
+            for (int q = 0; q < 4; ++q) {
+                v[q] = q < G ? red[q * width + tid] : P{};
+                for (int k = q + 4; k < G; k += 4) v[q] = Ar::padd(v[q], red[k * width + tid]);
+            }
+            pd[first + tid] = Ar::padd(Ar::padd(v[0], v[1]), Ar::padd(v[2], v[3]));
+        }
+        cl.sync();
+        // kCl lanes a column; column first + rank + kCl t belongs to this CTA
+        const int l = tid % kCl, cc = first + rank + kCl * (tid / kCl);
+        if (first + rank + kCl * ((tid & ~31) / kCl) < s) {  // uniform over the warp
+            const bool on = cc < s;
+            const P x = on ? cl.map_shared_rank(pd, l)[cc] : P{};
+            const P row = on ? cl.map_shared_rank(prow, owner)[cc] : P{};
+            const P d = lane_sum(x, kCl);
+            if (on) {
+                cl.map_shared_rank(tot, l)[cc] = d;
+                cl.map_shared_rank(rowv, l)[cc] = row;
+            }
+        }
+        cl.sync();
+    };
+    __syncthreads();
+    split(s);
+    {  // dot products of column 0
+        if (g < G && u < s) {
+            typename Ar::Acc d;
+#pragma unroll 4
+            for (int i = g; i < nr; i += G) Ar::acc(d, As[i], As[u * ld + i]);
+            red[tid] = Ar::part(d);
+            if (rank == 0 && g == 0) prow[u] = Ar::elem(As[u * ld]);
+        }
+        exchange(0, 0);
+    }
+    int owner = 0;  // CTA that holds row c
+    for (int c = 0; c < s; ++c) {
+        const int first = c + 1, live = s - first;
+        if (tid == kQrSmThreads - 32) {
+            const P alpha = rowv[c];
             if constexpr (kDf) {
-                householder_ff(nrm2, alpha, taus[c], rvs[c], betas[c], heads[c]);
+                householder_ff(tot[c], alpha, taus[c], rvs[c], betas[c], heads[c]);
             } else {
                 double tau, beta, v0;
-                householder(nrm2, alpha, tau, beta, v0);
+                householder(tot[c], alpha, tau, beta, v0);
                 taus[c] = tau;
                 betas[c] = beta;
                 heads[c] = v0;
+                rvs[c] = v0 - alpha;
             }
-            red[0] = alpha;
+            // the reflector's head in place (A(c, c) itself is beta)
+            if (rank == owner && Ar::nz(taus[c])) As[c * ld + c - r0] = Ar::fromP(heads[c]);
         }
+        if (live == 0) break;
+        split(live);
         __syncthreads();
-        const P tau = taus[c], v0 = heads[c];
-        for (int cc = c + 1 + tid; cc < s; cc += kQrSmThreads) {
-            P d{};
-#pragma unroll
-            for (int k = 0; k < kCl; ++k) d = Ar::padd(d, cl.map_shared_rank(pdc, k)[cc]);
-            // w_cc = tau (d_cc + (v0 - alpha) A(c, cc)), v0 - alpha = -beta
-            if constexpr (kDf)
-                wv[cc] = ff_mul(ff_mul(ff_add(d, ff_mul(ff_neg(betas[c]), orow[cc])), tau), rvs[c]);
-            else
-                wv[cc] = tau * (d + (v0 - red[0]) * orow[cc]);
+        const P tau = taus[c];
+        const bool act = Ar::nz(tau);  // identical on every CTA of the cluster
+        auto weight = [&](int cc) {
+            if constexpr (kDf) return ff_mul(ff_mul(ff_add(tot[cc], ff_mul(ff_neg(betas[c]), rowv[cc])), tau), rvs[c]);
+            else return tau * (tot[cc] + rvs[c] * rowv[cc]);
+        };
+        const int lb = max(c - r0, 0), lb1 = max(first - r0, 0);
+        const T *vc = As + c * ld;
+        T *vn = As + first * ld;
+        if (act && tid < nr - lb) {
+            const typename Ar::W w1 = Ar::prepP(weight(first));
+            for (int i = lb + tid; i < nr; i += kQrSmThreads) vn[i] = Ar::axmy(vn[i], w1, vc[i]);
         }
+        const bool mine = g < G && u < live;
+        typename Ar::W w{};
+        if (act && mine && u > 0) w = Ar::prepP(weight(first + u));
         __syncthreads();
-        if (Ar::nz(tau)) panel_update<kQrSmThreads, Ar>(As, ld, vc, ic, Ar::fromP(v0), wv, c + 1, s, lb, nr);
-        __syncthreads();
-        if (Ar::nz(tau) && rank == owner && tid == 0) vc[ic] = Ar::fromP(v0);  // reflector head stored in place
+        const int nowner = first - owner * per == per ? owner + 1 : owner;  // of row c + 1
+        if (mine) {
+            T *ac = As + (first + u) * ld;
+            typename Ar::Acc d;
+            if (act && u > 0) {
+                if (g == 0 && lb < min(lb1, nr)) ac[lb] = Ar::axmy(ac[lb], w, vc[lb]);  // row c (R)
+#pragma unroll 4
+                for (int i = lb1 + g; i < nr; i += G) {
+                    const T a = Ar::axmy(ac[i], w, vc[i]);
+                    ac[i] = a;
+                    Ar::acc(d, vn[i], a);
+                }
+            } else {
+#pragma unroll 4
+                for (int i = lb1 + g; i < nr; i += G) Ar::acc(d, vn[i], ac[i]);
+            }
+            red[tid] = Ar::part(d);
+            // row c + 1, which row group 0 holds first
+            if (g == 0 && rank == nowner) prow[first + u] = Ar::elem(ac[first - r0]);
+        }
+        owner = nowner;
+        exchange(first, owner);
     }
-    cl.sync();  // every CTA is done reading the factorisation's partials
+    __syncthreads();
     if (J.Rt) {  // Rt(i, u) = R(u, i) for the own rows u < s
         const int nu = max(0, min(nr, s - r0));
         for (int e = tid; e < nu * s; e += kQrSmThreads) {
-            const int lu = e / s, i = e % s, u = r0 + lu;
+            const int lu = e / s, i = e % s, ru = r0 + lu;
             double v = 0.0;
             T w = Ar::from(0.0);
-            if (i > u) {
+            if (i > ru) {
                 w = As[i * ld + lu];
                 v = Ar::to(w);
-            } else if (i == u) {
-                w = Ar::fromP(betas[u]);
-                v = Ar::toD(betas[u]);
+            } else if (i == ru) {
+                w = Ar::fromP(betas[ru]);
+                v = Ar::toD(betas[ru]);
             }
-            J.Rt[(int64_t)u * s + i] = v;
+            J.Rt[(int64_t)ru * s + i] = v;
             if constexpr (kDf)
-                if (J.Rt2) J.Rt2[(int64_t)u * s + i] = w;
+                if (J.Rt2) J.Rt2[(int64_t)ru * s + i] = w;
         }
     }
-    if (!J.Q) return;
-    __syncthreads();
-    int act = 0;
-    for (int c = s - 1; c >= 0; --c) {
-        const P tau = taus[c], v0 = heads[c];
-        const int lb = max(c - r0, 0), ic = c - r0;
-        T *vc = As + c * ld;
-        if (Ar::nz(tau)) {  // identical on every CTA of the cluster
-            P *pdc = pd + (act & 1) * s;
-            ++act;
-            panel_dots<kQrSmThreads, Ar>(As, ld, vc, c + 1, s, lb, nr, red, pdc);
-            cl.sync();
-            for (int cc = c + 1 + tid; cc < s; cc += kQrSmThreads) {
-                P d{};
-#pragma unroll
-                for (int k = 0; k < kCl; ++k) d = Ar::padd(d, cl.map_shared_rank(pdc, k)[cc]);
-                if constexpr (kDf) wv[cc] = ff_mul(ff_mul(d, tau), rvs[c]);
-                else wv[cc] = tau * d;
+    if (J.V) {
+        T *V = reinterpret_cast<T *>(J.V);
+        for (int e = tid; e < nr * s; e += kQrSmThreads) {
+            const int i = e % nr, j = e / nr;
+            V[(int64_t)j * m + r0 + i] = As[j * ld + i];
+        }
+        P *sc = reinterpret_cast<P *>(J.V + (int64_t)m * s);
+        if (rank == 0)
+            for (int j = tid; j < s; j += kQrSmThreads) {
+                sc[j] = taus[j];
+                sc[s + j] = heads[j];
+                sc[2 * s + j] = rvs[j];
             }
-            __syncthreads();
-            panel_update<kQrSmThreads, Ar>(As, ld, vc, -1, Ar::from(0.0), wv, c + 1, s, lb, nr);
-            __syncthreads();
-        }
-        // column c of Q = H_c e_c: tau v0 (= sign(v0) / |x| in pairs) times
-        // the reflector, 1 - tau v0^2 (= 1 - |v0| / |x|) at the head
-        typename Ar::W tv;
-        T qc;
-        if constexpr (kDf) {
-            const bool neg = v0.h < 0.f;
-            tv = Ar::prepP(neg ? ff_neg(tau) : tau);
-            qc = Ar::fromP(ff_add(FF{1.f, 0.f}, ff_neg(ff_mul(neg ? ff_neg(v0) : v0, tau))));
-        } else {
-            tv = Ar::prepP(tau * v0);
-            qc = Ar::from(1.0 - tau * v0 * v0);
-        }
-        for (int i = tid; i < nr; i += kQrSmThreads) {
-            T q;
-            if (i < ic) q = Ar::from(0.0);
-            else if (i == ic) q = qc;
-            else q = Ar::axmy(Ar::from(0.0), tv, vc[i]);
-            vc[i] = q;
-        }
-        __syncthreads();
     }
-    for (int e = tid; e < nr * s; e += kQrSmThreads) {
-        const int i = e % nr, j = e / nr;
-        J.Q[(int64_t)j * J.ldq + r0 + i] = Ar::to(As[j * ld + i]);
-    }
-    cl.sync();  // no CTA leaves while another may still read its partials
 }
 
 static size_t qr_sm_bytes(int m, int s, int csize) {
     const int per = (m + csize - 1) / csize, ld = per | 1;
-    return ((size_t)s * ld + 9 * (size_t)s + kQrSmThreads) * sizeof(double);
+    return ((size_t)s * ld + 8 * (size_t)s + kQrSmThreads) * sizeof(double);
 }
 
+// Q = H_0 ... H_{s-1} [I; 0] from the reflectors k_qr_factor left in J.V:
+// column j of Q is H_0 ... H_j e_j, one warp a column, its rows in registers
+// (row 32 k + lane, kR >= m / 32).  A CTA takes four columns; the reflectors
+// pass through a ring of three shared-memory stages filled by cp.async two
+// steps ahead.  The columns need nothing of each other, so they spread over
+// the whole GPU and no step waits for a cluster barrier; the longest column (s
+// reflectors) bounds the launch, so the last columns start first.  A stage's
+// rows above the head are zero from the start: reflector c writes rows >= c
+// only, and c falls, so that no step tests its rows (with a test per row the
+// loads and sums did not overlap: 698 us at m = 800, s = 200, against 182 us).
+// The FP64 pipe bounds the FP64 variant (439 us there).  Writes Q as doubles, or as pairs (hi, lo) where J.Q2 is given (the
+// paired paths read only those).
+constexpr int kFormThreads = 128, kFormCols = kFormThreads / 32, kFormStages = 3;
+template <bool kDf, int kR>
+__global__ void __launch_bounds__(kFormThreads) k_qr_form(const QrJob *__restrict__ jobs) {
+    using Ar = QrArith<kDf>;
+    using T = typename Ar::T;
+    using P = typename Ar::P;
+    __shared__ __align__(16) T vs[kFormStages][32 * kR];
+    __shared__ P sc[3][kMaxSample];  // tau, head and (pairs) 1 / |v0| of the reflectors
+    const QrJob J = jobs[blockIdx.y];
+    const int m = J.m, s = J.s, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nblk = (s + kFormCols - 1) / kFormCols;
+    if ((int)blockIdx.x >= nblk) return;
+    const int j0 = (nblk - 1 - (int)blockIdx.x) * kFormCols, j = j0 + warp;
+    const T *V = reinterpret_cast<const T *>(J.V);
+    const int top = min(j0 + kFormCols, s) - 1;  // first reflector applied
+    for (int e = tid; e <= top; e += kFormThreads)
+        for (int t = 0; t < 3; ++t) sc[t][e] = reinterpret_cast<const P *>(J.V + (int64_t)m * s)[t * s + e];
+    for (int e = tid; e < kFormStages * 32 * kR; e += kFormThreads) vs[e / (32 * kR)][e % (32 * kR)] = Ar::from(0.0);
+    T q[kR];
+#pragma unroll
+    for (int k = 0; k < kR; ++k) q[k] = Ar::from(0.0);
+    __syncthreads();
+    auto fetch = [&](int c) {  // reflector c into stage c % kFormStages
+        if (c >= 0) {
+            const T *src = V + (int64_t)c * m;
+            T *dst = vs[c % kFormStages];
+            for (int i = c + tid; i < m; i += kFormThreads) {
+                const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + i);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src + i) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(top);
+    fetch(top - 1);
+    for (int c = top; c >= 0; --c) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();  // stage c is complete; the stage of c + 1 has been read by every warp
+        fetch(c - 2);
+        if (j < c || j >= s) continue;
+        const P tau = sc[0][c];
+        const T *v = vs[c % kFormStages] + lane;
+        if (j == c) {
+            // H_c e_c: tau v0 (= sign(v0) / |x| in pairs) times the reflector,
+            // 1 - tau v0^2 (= 1 - |v0| / |x|) at the head; e_c itself if tau = 0
+            const P v0 = sc[1][c];
+            typename Ar::W tv;
+            T qc;
+            if constexpr (kDf) {
+                const bool neg = v0.h < 0.f;
+                tv = Ar::prepP(neg ? ff_neg(tau) : tau);
+                qc = Ar::fromP(ff_add(FF{1.f, 0.f}, ff_neg(ff_mul(neg ? ff_neg(v0) : v0, tau))));
+            } else {
+                tv = Ar::prepP(tau * v0);
+                qc = Ar::from(1.0 - tau * v0 * v0);
+            }
+#pragma unroll
+            for (int k = 0; k < kR; ++k) q[k] = 32 * k + lane == c ? qc : Ar::axmy(Ar::from(0.0), tv, v[32 * k]);
+        } else if (Ar::nz(tau)) {
+            typename Ar::Acc d0, d1;
+#pragma unroll
+            for (int k = 0; k < kR; ++k) Ar::acc(k & 1 ? d1 : d0, v[32 * k], q[k]);
+            const P dot = lane_sum(Ar::padd(Ar::part(d0), Ar::part(d1)));
+            typename Ar::W w;
+            if constexpr (kDf) w = Ar::prepP(ff_mul(ff_mul(dot, tau), sc[2][c]));
+            else w = Ar::prepP(tau * dot);
+#pragma unroll
+            for (int k = 0; k < kR; ++k) q[k] = Ar::axmy(q[k], w, v[32 * k]);
+        }
+    }
+    if (j >= s) return;
+#pragma unroll
+    for (int k = 0; k < kR; ++k) {
+        const int i = 32 * k + lane;
+        if (i < m) {
+            if constexpr (kDf) {
+                if (J.Q2) {
+                    J.Q2[(int64_t)j * J.ldq + i] = q[k];
+                    continue;
+                }
+            }
+            J.Q[(int64_t)j * J.ldq + i] = Ar::to(q[k]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // QR in global memory (A factorised in place; Q and Rt as above), for panels
-// that do not fit in shared memory.  Same barrier scheme as k_qr_sm.
+// that do not fit in shared memory.  One cluster barrier a column, as in k_qr_factor.
 template <int kCl>
 __global__ void __launch_bounds__(kQrThreads) k_qr_gm(const QrJob *__restrict__ jobs) {
     cg::cluster_group cl = cg::this_cluster();
@@ -1255,7 +1345,7 @@ static bool cluster16_ok() {
     static std::once_flag once;
     static int state = 0;
     std::call_once(once, [] {
-        const void *k16[] = {(const void *)k_qr_sm<16, false>, (const void *)k_qr_sm<16, true>, (const void *)k_qr_gm<16>, (const void *)k_jacobi_sm<16, kJacFull>,
+        const void *k16[] = {(const void *)k_qr_factor<16, false>, (const void *)k_qr_factor<16, true>, (const void *)k_qr_gm<16>, (const void *)k_jacobi_sm<16, kJacFull>,
                              (const void *)k_jacobi_sm<16, kJacPrecond>, (const void *)k_jacobi_sm<16, kJacFinish>,
                              (const void *)k_jacobi_gm<16>};
         bool ok = true;
@@ -1263,7 +1353,7 @@ static bool cluster16_ok() {
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
         if (ok) {
             // one cluster of 16 CTAs that each fill an SM's shared memory must fit
-            const size_t need = std::min(smem_cap((const void *)k_qr_sm<16, false>), smem_cap((const void *)k_jacobi_sm<16, kJacFull>));
+            const size_t need = std::min(smem_cap((const void *)k_qr_factor<16, false>), smem_cap((const void *)k_jacobi_sm<16, kJacFull>));
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(16);
             cfg.blockDim = dim3(kQrThreads);
@@ -1278,7 +1368,7 @@ static bool cluster16_ok() {
             int n1 = 0, n2 = 0;
             cudaLaunchConfig_t cfq = cfg;
             cfq.blockDim = dim3(kQrSmThreads);
-            if (cudaOccupancyMaxActiveClusters(&n1, k_qr_sm<16, false>, &cfq) == cudaSuccess &&
+            if (cudaOccupancyMaxActiveClusters(&n1, k_qr_factor<16, false>, &cfq) == cudaSuccess &&
                 cudaOccupancyMaxActiveClusters(&n2, k_jacobi_sm<16, kJacFull>, &cfg) == cudaSuccess && n1 > 0 && n2 > 0)
                 state = 1;
         }
@@ -1306,11 +1396,11 @@ using SvdKernel = void (*)(const SvdJob *);
 template <bool kDf>
 static QrKernel qr_sm_kernel_t(int c) {
     switch (c) {
-    case 1: return k_qr_sm<1, kDf>;
-    case 2: return k_qr_sm<2, kDf>;
-    case 4: return k_qr_sm<4, kDf>;
-    case 8: return k_qr_sm<8, kDf>;
-    default: return k_qr_sm<16, kDf>;
+    case 1: return k_qr_factor<1, kDf>;
+    case 2: return k_qr_factor<2, kDf>;
+    case 4: return k_qr_factor<4, kDf>;
+    case 8: return k_qr_factor<8, kDf>;
+    default: return k_qr_factor<16, kDf>;
     }
 }
 static QrKernel qr_sm_kernel(int c, bool df) { return df ? qr_sm_kernel_t<true>(c) : qr_sm_kernel_t<false>(c); }
@@ -1341,6 +1431,8 @@ struct LaunchClass {
     size_t smem = 0;
     std::vector<Job> jobs;
     int threads = kQrThreads;
+    // launched behind the class's kernel on its stream, if set
+    void (*post)(cudaStream_t, const Job *, const std::vector<Job> &) = nullptr;
 };
 
 // Events around the launch of one class (profiling).
@@ -1380,6 +1472,7 @@ static void launch_classes(tlr_ctx *ctx, cudaStream_t st, std::vector<LaunchClas
         if (timed) TLR_CUDA_TRY(cudaEventRecord(timing->e0, cs));
         launch_cluster(use[k]->kernel, use[k]->csize, (int)use[k]->jobs.size(), use[k]->threads, use[k]->smem, cs, dj[k],
                        extra...);
+        if (use[k]->post) use[k]->post(cs, dj[k], use[k]->jobs);
         if (timed) TLR_CUDA_TRY(cudaEventRecord(timing->e1, cs));
         TLR_CUDA_TRY(cudaEventRecord(ctx->cls_join[k], cs));
     }
@@ -1393,15 +1486,35 @@ static void launch_classes(tlr_ctx *ctx, cudaStream_t st, std::vector<LaunchClas
 
 template <class Job, class K>
 static void add_to_class(std::vector<LaunchClass<Job, K>> &cls, K kernel, int csize, size_t smem, const Job &j,
-                         int threads = kQrThreads) {
+                         int threads = kQrThreads,
+                         void (*post)(cudaStream_t, const Job *, const std::vector<Job> &) = nullptr) {
     for (auto &c : cls)
         if (c.kernel == kernel && c.csize == csize) {
             c.smem = std::max(c.smem, smem);
             c.jobs.push_back(j);
             return;
         }
-    LaunchClass<Job, K> c{kernel, csize, smem, {j}, threads};
+    LaunchClass<Job, K> c{kernel, csize, smem, {j}, threads, post};
     cls.push_back(c);
+}
+
+// Q of every job of a class from its reflectors; rows in the smallest of the
+// register sizes that holds the class's tallest job.
+template <bool kDf>
+static void form_q(cudaStream_t st, const QrJob *d, const std::vector<QrJob> &jobs) {
+    int cols = 0, rows = 0;
+    for (const QrJob &J : jobs) {
+        cols = std::max(cols, J.s);
+        rows = std::max(rows, J.m);
+    }
+    const dim3 grid((unsigned)ceil_div(cols, kFormCols), (unsigned)jobs.size());
+    auto go = [&](void (*k)(const QrJob *)) { launch(k, grid, kFormThreads, 0, st, d); };
+    if (rows <= 32 * 8) go(k_qr_form<kDf, 8>);
+    else if (rows <= 32 * 16) go(k_qr_form<kDf, 16>);
+    else if (rows <= 32 * 20) go(k_qr_form<kDf, 20>);
+    else if (rows <= 32 * 25) go(k_qr_form<kDf, 25>);
+    else go(k_qr_form<kDf, kMaxTile / 32>);
+    TLR_CHECK_LAUNCH();
 }
 
 // QR stage for a list of jobs.  `copy[u]` (k x s, may alias nothing) is
@@ -1411,6 +1524,7 @@ static void qr_launch(tlr_ctx *ctx, cudaStream_t st, const std::vector<QrJob> &j
                       bool df) {
     const bool big = cluster16_ok();
     std::vector<LaunchClass<QrJob, QrKernel>> cls;
+    std::vector<SplitDesc> split;
     for (size_t u = 0; u < jobs.size(); ++u) {
         QrJob J = jobs[u];
         int c = qr_cluster(ctx, J.s);
@@ -1420,9 +1534,10 @@ static void qr_launch(tlr_ctx *ctx, cudaStream_t st, const std::vector<QrJob> &j
         QrKernel k = qr_sm_kernel(c, df);
         size_t bytes = qr_sm_bytes(J.m, J.s, c);
         if (bytes <= smem_cap((const void *)k)) {
-            add_to_class(cls, k, c, bytes, J, kQrSmThreads);
+            add_to_class(cls, k, c, bytes, J, kQrSmThreads, J.Q ? (df ? form_q<true> : form_q<false>) : nullptr);
             continue;
         }
+        if (J.Q2) split.push_back(SplitDesc{J.Q, J.Q2, J.ldq, J.m, J.s});
         // global-memory fallback: factorises its input in place
         if (!J.Q) {
             TLR_CUDA_TRY(cudaMemcpy2DAsync(copy[u], (size_t)J.m * sizeof(double), J.A, (size_t)J.lda * sizeof(double),
@@ -1435,6 +1550,7 @@ static void qr_launch(tlr_ctx *ctx, cudaStream_t st, const std::vector<QrJob> &j
         ctx->comp_stats[5] += 1;
     }
     launch_classes(ctx, st, cls, (ClassTiming *)nullptr);
+    split_f2_batched(ctx, st, split);
 }
 
 // The SVD stage.  csize_of[u] receives the cluster size job u ran on (0 for
@@ -1551,7 +1667,7 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
             const CompressJob &J = jobs[pending[u]];
             int s = sz[pending[u]];
             ps[u] = s;
-            oY[u] = take((int64_t)J.m * s);
+            oY[u] = take((int64_t)J.m * s + 3 * s);  // the sample, then its QR's reflectors and their scalars
             oQ[u] = take((int64_t)J.m * s);
             oB[u] = take((int64_t)J.k * s);
             oC[u] = take((int64_t)J.k * s);
@@ -1591,16 +1707,11 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
         std::vector<double *> scratch(np);
         for (size_t u = 0; u < np; ++u) {
             const CompressJob &J = jobs[pending[u]];
-            q1[u] = QrJob{W + oY[u], J.m, W + oQ[u], J.m, nullptr, J.m, ps[u]};
+            q1[u] = QrJob{W + oY[u], J.m, W + oQ[u], J.m, nullptr, J.m, ps[u], nullptr, W + oY[u],
+                          dfp ? (float2 *)(W + oQ2[u]) : nullptr};
             scratch[u] = W + oC[u];
         }
         qr_launch(ctx, st, q1, scratch, df);
-        if (dfp) {
-            std::vector<SplitDesc> sd(np);
-            for (size_t u = 0; u < np; ++u)
-                sd[u] = SplitDesc{W + oQ[u], (float2 *)(W + oQ2[u]), jobs[pending[u]].m, jobs[pending[u]].m, ps[u]};
-            split_f2_batched(ctx, st, sd);
-        }
         cmark();
         // 3. B = T' Q (kept), R' of B = Q2 R
         std::vector<GemmProb> g2;
@@ -1619,7 +1730,7 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
         std::vector<QrJob> q2(np);
         for (size_t u = 0; u < np; ++u) {
             const CompressJob &J = jobs[pending[u]];
-            q2[u] = QrJob{W + oB[u], J.k, nullptr, 0, W + oR[u], J.k, ps[u], df ? (float2 *)(W + oR2[u]) : nullptr};
+            q2[u] = QrJob{W + oB[u], J.k, nullptr, 0, W + oR[u], J.k, ps[u], df ? (float2 *)(W + oR2[u]) : nullptr, nullptr, nullptr};
         }
         qr_launch(ctx, st, q2, scratch, df);
         cmark();

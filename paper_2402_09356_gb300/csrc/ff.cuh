@@ -3,8 +3,8 @@
 // products are Dekker's (T. J. Dekker, "A floating-point technique for
 // extending the available precision", Numer. Math. 18, 1971): TwoSum
 // (Knuth) for the head words, the product's rounding error by FMA, the low
-// words added in FP32.  Square root and quotient take the FP32 result and
-// one correction from the exact residual (Dekker's sqrt2 / div2).
+// words added in FP32.  Reciprocal and reciprocal square root take the FP32
+// result and one correction from its residual in pairs.
 // On GB300 an FP64 warp instruction occupies the SM sub-partition's FP64
 // pipe for 64 cycles whether one lane or 32 are active; these run on the
 // FP32 pipe (4-cycle latency, full rate) and serve the per-column scalars
@@ -37,20 +37,23 @@ __device__ __forceinline__ FF ff_mul(FF a, FF b) {
     e = __fmaf_rn(a.l, b.h, e);
     return ff_fast(p, e);
 }
-// a / b: q = fl(a.h / b.h), then q + (a - q b) / b.h with a - q b exact in its head
-__device__ __forceinline__ FF ff_div(FF a, FF b) {
-    const float q = __fdiv_rn(a.h, b.h);
-    const FF qb = ff_mul(FF{q, 0.f}, b);
-    const FF r = ff_add(a, ff_neg(qb));
-    return ff_fast(q, __fdiv_rn(r.h, b.h));
+// 1 / sqrt(a), a > 0: the FP32 approximation y and its residual e = 1 - a y^2
+// in pairs, then y + y (e / 2 + 3 e^2 / 8) (the third-order step; e ~ 2^-22).
+// One chain of FP32 operations, where a square root and a quotient take two
+// IEEE square roots and divisions one after the other.
+__device__ __forceinline__ FF ff_rsqrt(FF a) {
+    const float y = rsqrtf(a.h);
+    const FF ay = ff_mul(a, FF{y, 0.f});
+    const float p = __fmul_rn(ay.h, y), pe = __fmaf_rn(ay.l, y, __fmaf_rn(ay.h, y, -p));
+    const float e = __fsub_rn(__fsub_rn(1.0f, p), pe);
+    return ff_fast(y, __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f))));
 }
-// sqrt(a), a >= 0: s = fl(sqrt(a.h)), then s + (a - s^2) / (2 s)
-__device__ __forceinline__ FF ff_sqrt(FF a) {
-    if (!(a.h > 0.f)) return FF{a.h == 0.f ? 0.f : __fsqrt_rn(a.h), 0.f};
-    const float s = __fsqrt_rn(a.h);
-    const float p = __fmul_rn(s, s), pe = __fmaf_rn(s, s, -p);
-    const float r = __fadd_rn(__fsub_rn(__fsub_rn(a.h, p), pe), a.l);
-    return ff_fast(s, __fdiv_rn(r, __fmul_rn(2.0f, s)));
+// 1 / a, a != 0 and normal: the FP32 reciprocal y, then y + y (e + e^2), e = 1 - a y
+__device__ __forceinline__ FF ff_rcp(FF a) {
+    const float y = __frcp_rn(a.h);
+    const float p = __fmul_rn(a.h, y), pe = __fmaf_rn(a.l, y, __fmaf_rn(a.h, y, -p));
+    const float e = __fsub_rn(__fsub_rn(1.0f, p), pe);
+    return ff_fast(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
 }
 
 }  // namespace tlr

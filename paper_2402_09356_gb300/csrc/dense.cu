@@ -6,14 +6,15 @@
 // Blocks of 32 rows/columns are factored or solved by one CTA in shared
 // memory; everything else is a batched GEMM update so that it spreads over
 // the whole GPU (one SM's FP64 pipe alone would take milliseconds per tile).
+#include <algorithm>
 #include <mutex>
 
 #include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "dense.cuh"
-#include "ff.cuh"
 #include "gemm.cuh"
+#include "tlr_internal.cuh"
 
 namespace tlr {
 
@@ -25,7 +26,8 @@ constexpr int kBlk = 32;
 // ---------------------------------------------------------------------------
 // Cholesky and inverse of one diagonal tile in a single launch.
 //
-// One cluster of kCl CTAs; the tile (m <= 1024, column major) stays in global
+// One cluster of kCl CTAs (tiles wider than kPotrfOuter come block by block,
+// see potrf_inv_batched); the tile (m <= 1024, column major) stays in global
 // memory, which for one tile is L2-resident, and every load goes to L2
 // (__ldcg: another CTA may have written the line in an earlier phase).  A
 // cluster barrier (release/acquire at cluster scope) separates dependent
@@ -36,9 +38,8 @@ constexpr int kBlk = 32;
 //      < end of block k; X starts as I), with L_kk^-1 from step k - 1;
 //   -- barrier --
 //   2. CTA 0 updates the next diagonal block, A_{k+1,k+1} -= L_{k+1,k}
-//      L_{k+1,k}', and factors and inverts it in shared memory (a rank-1
-//      update per column; the inverse row by row, eight lanes per column):
-//      the diagonal block of step k + 1 is ready when step k ends.  The other
+//      L_{k+1,k}', and factors and inverts it in shared memory
+//      (potrf_diag_block): the diagonal block of step k + 1 is ready when step k ends.  The other
 //      CTAs take, round robin, the rest of the trailing lower triangle,
 //      A_IJ -= L_Ik L_Jk' (I >= J > k), and the inverse's update
 //      X_IJ -= L_Ik X_kJ (I > k, J <= k), 32 x 32 output tiles, loading
@@ -83,123 +84,80 @@ __device__ __forceinline__ void tile_update32(double *C, int ldc, const double (
         }
 }
 
-// The same update in float-float pairs (the inverse X on the paired paths):
-// C (pairs) -= A B with a, b pairs in shared memory as [row][k].
-__device__ __forceinline__ void tile_update32_ff(float2 *C, int ldc, const float2 (*a)[kBlk + 1],
-                                                 const float2 (*b)[kBlk + 1], int rows, int cols) {
-    const int tid = threadIdx.x, tr = (tid & 15) * 2, tc = (tid >> 4) * 2;
-    float2 cv[2][2];
-#pragma unroll
-    for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y) {
-            const int r = tr + x, c = tc + y;
-            cv[x][y] = (r < rows && c < cols) ? __ldcg(C + (int64_t)c * ldc + r) : make_float2(0.f, 0.f);
-        }
-    float h[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, l[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll 8
-    for (int k = 0; k < kBlk; ++k) {
-        const float2 a0 = a[tr][k], a1 = a[tr + 1][k], b0 = b[tc][k], b1 = b[tc + 1][k];
-        df_fma(a0.x, a0.y, b0.x, b0.y, h[0][0], l[0][0]);
-        df_fma(a0.x, a0.y, b1.x, b1.y, h[0][1], l[0][1]);
-        df_fma(a1.x, a1.y, b0.x, b0.y, h[1][0], l[1][0]);
-        df_fma(a1.x, a1.y, b1.x, b1.y, h[1][1], l[1][1]);
-    }
-#pragma unroll
-    for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y) {
-            const int r = tr + x, c = tc + y;
-            if (r < rows && c < cols) {
-                const FF d = ff_add(FF{cv[x][y].x, cv[x][y].y}, ff_neg(ff_two_sum(h[x][y], l[x][y])));
-                C[(int64_t)c * ldc + r] = make_float2(d.h, d.l);
-            }
-        }
-}
-
-__device__ __forceinline__ float2 ff_split(double v) {
-    const float h = __double2float_rn(v);
-    return make_float2(h, __double2float_rn(v - (double)h));
-}
-
-// 1 / sqrt(d) for d > 0 (normal): the PTX approximation, then two Newton
-// steps y <- y (3 - d y^2) / 2, each squaring the relative error (to about
-// an ulp).  One thread forms it per column of a diagonal block, where every
-// FP64 instruction holds the FP64 pipe for 64 cycles: this takes fewer
-// instructions than a square root followed by a quotient per entry.
-__device__ __forceinline__ double rsqrt_newton(double d) {
+// 1 / sqrt(d) for d > 0 (normal): the PTX approximation y (error e = 1 - d y^2
+// ~ 2^-19), then one third-order step y + y e (1/2 + 3/8 e), to about an ulp.
+// The pivot chain of a diagonal block runs through it once per column, and
+// every FP64 instruction takes 64 cycles: five of them against eight for two
+// Newton steps.
+__device__ __forceinline__ double rsqrt_step(double d) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    y = y * fma(-0.5 * d * y, y, 1.5);
-    return y * fma(-0.5 * d * y, y, 1.5);
+    const double e = fma(-(d * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Cholesky of the w x w diagonal block at (p, p) of A by the calling CTA,
 // with the block's inverse: L_kk into A (lower; upper part of the block 0),
-// L_kk^-1 into Li (32 x 32, row major).  Returns the first failing column
-// (non-positive pivot) or -1, the same on every thread.
-__device__ int potrf_diag_block(double *A, int lda, int p, int w, double *Li, double (*sa)[kBlk + 1],
-                                double (*sl)[kBlk + 1], int *s_bad) {
-    const int tid = threadIdx.x;
-    for (int e = tid; e < kBlk * kBlk; e += kPotrfThreads) {
-        const int r = e % kBlk, c = e / kBlk;
-        sa[r][c] = (r < w && c < w && c <= r) ? __ldcg(A + (int64_t)(p + c) * lda + p + r) : 0.0;
+// L_kk^-1 into Li (32 x 32, row major).  The block's lower triangle is in M on
+// entry.  Returns the first failing column (non-positive pivot) or -1, the
+// same on every thread.
+// Factor and inverse advance together: after column c, M[r][j] holds L^-1's
+// entry (of the elimination so far) for j <= c and the updated A for j > c, so
+// that one rank-1 update a column serves both (ov: row c of the inverse up to
+// column c, column c of L behind it).  Warp 0 keeps the diagonal in
+// registers (lane r: entry (r, r)) and runs the chain that bounds the block --
+// scale, diagonal update, reciprocal square root, about 600 cycles a column --
+// while the other warps update the rows behind it: 19,000 cycles a block, where
+// a column-wise factorisation and then a row-wise inverse took 59,000.
+__device__ int potrf_diag_block(double *A, int lda, int p, int w, double *Li, double (*M)[kBlk + 1], double *ov,
+                                double *sy, int *s_bad) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double diag = 0.0, y = 0.0;
+    if (warp == 0) {
+        diag = lane < w ? M[lane][lane] : 1.0;
+        const double d0 = __shfl_sync(0xFFFFFFFFu, diag, 0);
+        if (lane == 0) *s_bad = d0 > 0.0 ? -1 : 0;
+        y = rsqrt_step(d0);
+        if (lane == 0) *sy = y;
     }
-    if (tid == 0) *s_bad = -1;
     __syncthreads();
-    // right-looking Cholesky of the block, one column at a time, the updates
-    // spread over the CTA's threads; the pivot's reciprocal is kept in the
-    // padding column sa[c][kBlk] (the column is scaled by it, and the
-    // inverse below divides by the pivots through it)
+    const int r = tid >> 3, q = tid & 7;  // the update: row r, columns q, q + 8, ...
     for (int c = 0; c < w; ++c) {
-        if (tid == 0) {
-            const double d = sa[c][c];
-            if (!(d > 0.0)) {
-                *s_bad = c;
-            } else {
-                const double y = rsqrt_newton(d);
-                sa[c][c] = d * y;
-                sa[c][kBlk] = y;
-            }
+        if (*s_bad >= 0) break;  // written before the last barrier: uniform
+        // column c of L and row c of the inverse
+        if (warp == 0) {
+            double l = 0.0;
+            if (lane > c && lane < w) l = M[lane][c] * y;
+            if (lane > c) ov[lane] = l;
+            diag = fma(-l, l, diag);
+            if (lane < w) A[(int64_t)(p + c) * lda + p + lane] = lane > c ? l : (lane == c ? diag * y : 0.0);
+        } else if (warp == 1) {
+            const double yc = *sy, x = lane < c ? M[c][lane] * yc : (lane == c ? yc : 0.0);
+            if (lane <= c) ov[lane] = x;
+            Li[c * kBlk + lane] = x;
         }
         __syncthreads();
-        if (*s_bad >= 0) break;  // read after the barrier: uniform
-        const double rpiv = sa[c][kBlk];
-        for (int r = c + 1 + tid; r < w; r += kPotrfThreads) sa[r][c] *= rpiv;
-        __syncthreads();
-        const int nr = w - c - 1;
-        for (int e = tid; e < nr * nr; e += kPotrfThreads) {
-            const int r = c + 1 + e % nr, cc = c + 1 + e / nr;
-            if (cc <= r) sa[r][cc] -= sa[r][c] * sa[cc][c];
+        if (warp == 0 && c + 1 < w) {
+            const double d = __shfl_sync(0xFFFFFFFFu, diag, c + 1);
+            y = rsqrt_step(d);
+            if (lane == 0) {
+                *sy = y;
+                if (!(d > 0.0)) *s_bad = c + 1;
+            }
+        }
+        if (r > c && r < w) {
+            const double l = ov[r];
+#pragma unroll
+            for (int k = 0; k < kBlk / 8; ++k) {
+                const int j = q + 8 * k;
+                if (j < r) M[r][j] = fma(-l, ov[j], j == c ? 0.0 : M[r][j]);
+            }
         }
         __syncthreads();
     }
     const int bad = *s_bad;
     if (bad >= 0) return bad;
-    // inverse of the lower triangular block, row by row: column c by the 8
-    // lanes 8c .. 8c+7 (one warp holds four columns), each summing every 8th
-    // term, then a shuffle reduction
-    const int c = tid >> 3, q = tid & 7;
-    for (int r = 0; r < kBlk; ++r) {
-        double part = 0.0;
-        if (c < w && r < w && r > c)
-            for (int k = c + q; k < r; k += 8) part = fma(sa[r][k], sl[k][c], part);
-        part += __shfl_xor_sync(0xFFFFFFFFu, part, 4);
-        part += __shfl_xor_sync(0xFFFFFFFFu, part, 2);
-        part += __shfl_xor_sync(0xFFFFFFFFu, part, 1);
-        if (q == 0) {
-            double v = 0.0;
-            if (c < w && r < w && r >= c) v = ((r == c ? 1.0 : 0.0) - part) * sa[r][kBlk];
-            sl[r][c] = v;
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    for (int e = tid; e < kBlk * kBlk; e += kPotrfThreads) {
-        const int r = e % kBlk, cc = e / kBlk;
-        if (r < w && cc < w) A[(int64_t)(p + cc) * lda + p + r] = (cc <= r) ? sa[r][cc] : 0.0;
-        Li[r * kBlk + cc] = sl[r][cc];
-    }
+    for (int e = w * kBlk + tid; e < kBlk * kBlk; e += kPotrfThreads) Li[e] = 0.0;  // rows past the block
     return -1;
 }
 
@@ -209,11 +167,7 @@ __device__ int potrf_diag_block(double *A, int lda, int p, int w, double *Li, do
 // each read it to decide).
 // One cluster per job (blockIdx.x / kCl): the diagonal tiles of several
 // factorisations in one launch (the jobs travel in the kernel parameters).
-// kFF: the inverse X in float-float pairs on the FP32 pipe (stored as pairs
-// in X's memory while the kernel runs, as doubles hi + lo at the end); the
-// Cholesky factor stays FP64.  The paired paths use X only in products they
-// run in paired FP32.
-template <int kCl, bool kFF>
+template <int kCl>
 __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jobs) {
     const PotrfJob J = jobs.job[blockIdx.x / kCl];
     double *const A = J.A, *const X = J.X, *const scratch = J.scratch;
@@ -224,19 +178,15 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
     const int rank = (int)cl.block_rank(), tid = threadIdx.x;
     const int gtid = rank * kPotrfThreads + tid, gthreads = kCl * kPotrfThreads;
     __shared__ double sa[kBlk][kBlk + 1], sb[kBlk][kBlk + 1], sl[kBlk][kBlk + 1];
-    __shared__ float2 slf[kFF ? kBlk : 1][kBlk + 1];  // L_kk^-1 as pairs (kFF)
+    __shared__ double ov[kBlk], sy;
     __shared__ int s_bad;
-    float2 *const X2 = reinterpret_cast<float2 *>(X);
-    float2 (*const saf)[kBlk + 1] = reinterpret_cast<float2 (*)[kBlk + 1]>(sa);
-    float2 (*const sbf)[kBlk + 1] = reinterpret_cast<float2 (*)[kBlk + 1]>(sb);
     const int nbk = (m + kBlk - 1) / kBlk;
     double *dinv = scratch;
     long long *stop = reinterpret_cast<long long *>(scratch + (int64_t)kBlk * kBlk * kBlk);
     // X = I; CTA 0 factors the first diagonal block
     for (int64_t e = gtid; e < (int64_t)m * m; e += gthreads) {
         const int r = (int)(e % m), c = (int)(e / m);
-        if constexpr (kFF) X2[(int64_t)c * ldx + r] = make_float2(r == c ? 1.f : 0.f, 0.f);
-        else X[(int64_t)c * ldx + r] = (r == c) ? 1.0 : 0.0;
+        X[(int64_t)c * ldx + r] = (r == c) ? 1.0 : 0.0;
     }
     if (rank == 0) {
         // one read of the status word decides for the whole CTA (another
@@ -246,7 +196,12 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
         long long halt = s_bad ? 1LL : 0LL;
         __syncthreads();
         if (!halt) {
-            const int bad = potrf_diag_block(A, lda, 0, min(kBlk, m), dinv, sa, sl, &s_bad);
+            for (int e = tid; e < kBlk * kBlk; e += kPotrfThreads) {
+                const int r = e % kBlk, c = e / kBlk;
+                sa[r][c] = (r < m && c <= r) ? __ldcg(A + (int64_t)c * lda + r) : 0.0;
+            }
+            __syncthreads();
+            const int bad = potrf_diag_block(A, lda, 0, min(kBlk, m), dinv, sa, ov, &sy, &s_bad);
             if (bad >= 0) {
                 if (tid == 0) set_status(st, TLR_ERR_NOT_SPD, row_base + bad);
                 halt = 1;
@@ -262,53 +217,57 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
         // 1. panel rows below the block: x <- a L_kk^-T, x_c = sum_{k<=c} a_k Linv[c][k];
         //    inverse block row: X[k-block, c] <- L_kk^-1 X[k-block, c], c < p + w
         for (int e = tid; e < kBlk * kBlk; e += kPotrfThreads) {
-            const double v = __ldcg(Li + e);
-            sl[e / kBlk][e % kBlk] = v;
-            if constexpr (kFF) slf[e / kBlk][e % kBlk] = ff_split(v);
+            sl[e / kBlk][e % kBlk] = __ldcg(Li + e);
         }
         __syncthreads();
-        // rows and columns dealt to the CTAs in turn (gq = tid * kCl + rank), so
-        // that every CTA's FP64 pipe takes a share (a 32-term chain each)
-        const int gq = tid * kCl + rank;
-        for (int r = p + w + gq; r < m; r += gthreads) {
-            double a[kBlk];
+        // rows and columns dealt to the CTAs in turn, eight threads each (thread
+        // q forms entries q, q + 8, ...: every scheduler takes a share, and a
+        // chain is 80 multiply-adds, not 528); operands through shared memory,
+        // 32 rows or columns at a time
+        const int q8 = tid & 7, u8 = tid >> 3;
+        const int rows_per = (m - p - w + kCl - 1) / kCl, r_hi = min(m, p + w + (rank + 1) * rows_per);
+        for (int b0 = p + w + rank * rows_per; b0 < r_hi; b0 += kBlk) {
+            __syncthreads();
+            for (int e = tid; e < kBlk * kBlk; e += kPotrfThreads) {
+                const int r = b0 + e % kBlk, k = e / kBlk;
+                sa[e % kBlk][k] = (r < r_hi && k < w) ? __ldcg(A + (int64_t)(p + k) * lda + r) : 0.0;
+            }
+            __syncthreads();
+            const int r = b0 + u8;
+            if (r < r_hi) {
 #pragma unroll
-            for (int k = 0; k < kBlk; ++k) a[k] = k < w ? __ldcg(A + (int64_t)(p + k) * lda + r) : 0.0;
-#pragma unroll
-            for (int c = 0; c < kBlk; ++c) {
-                if (c >= w) break;
-                double x = 0.0;
-#pragma unroll
-                for (int k = 0; k <= c; ++k) x = fma(a[k], sl[c][k], x);
-                A[(int64_t)(p + c) * lda + r] = x;
+                for (int t = 0; t < kBlk / 8; ++t) {
+                    const int c = q8 + 8 * t;
+                    double x0 = 0.0, x1 = 0.0;
+#pragma unroll 4
+                    for (int k = 0; k < 8 * t + 8; k += 2) {  // L_kk^-1 is 0 right of its diagonal
+                        x0 = fma(sa[u8][k], sl[c][k], x0);
+                        x1 = fma(sa[u8][k + 1], sl[c][k + 1], x1);
+                    }
+                    if (c < w) A[(int64_t)(p + c) * lda + r] = x0 + x1;
+                }
             }
         }
-        for (int c = gq; c < p + w; c += gthreads) {
-            if constexpr (kFF) {
-                float2 x[kBlk];
+        for (int b0 = rank; b0 < p + w; b0 += kCl * kBlk) {
+            __syncthreads();
+            for (int e = tid; e < kBlk * kBlk; e += kPotrfThreads) {
+                const int c = b0 + kCl * (e / kBlk), k = e % kBlk;
+                const bool in = c < p + w && k < w;
+                sa[e / kBlk][k] = in ? __ldcg(X + (int64_t)c * ldx + p + k) : 0.0;
+            }
+            __syncthreads();
+            const int c = b0 + kCl * u8;
+            if (c < p + w) {
 #pragma unroll
-                for (int k = 0; k < kBlk; ++k)
-                    x[k] = k < w ? __ldcg(X2 + (int64_t)c * ldx + p + k) : make_float2(0.f, 0.f);
-#pragma unroll
-                for (int r = 0; r < kBlk; ++r) {
-                    if (r >= w) break;
-                    float vh = 0.f, vl = 0.f;
-#pragma unroll
-                    for (int k = 0; k <= r; ++k) df_fma(slf[r][k].x, slf[r][k].y, x[k].x, x[k].y, vh, vl);
-                    const FF v = ff_two_sum(vh, vl);
-                    X2[(int64_t)c * ldx + p + r] = make_float2(v.h, v.l);
-                }
-            } else {
-                double x[kBlk];
-#pragma unroll
-                for (int k = 0; k < kBlk; ++k) x[k] = k < w ? __ldcg(X + (int64_t)c * ldx + p + k) : 0.0;
-#pragma unroll
-                for (int r = 0; r < kBlk; ++r) {
-                    if (r >= w) break;
-                    double v = 0.0;
-#pragma unroll
-                    for (int k = 0; k <= r; ++k) v = fma(sl[r][k], x[k], v);
-                    X[(int64_t)c * ldx + p + r] = v;
+                for (int t = 0; t < kBlk / 8; ++t) {
+                    const int r = q8 + 8 * t;
+                    double x0 = 0.0, x1 = 0.0;
+#pragma unroll 4
+                    for (int k = 0; k < 8 * t + 8; k += 2) {
+                        x0 = fma(sl[r][k], sa[u8][k], x0);
+                        x1 = fma(sl[r][k + 1], sa[u8][k + 1], x1);
+                    }
+                    if (r < w) X[(int64_t)c * ldx + p + r] = x0 + x1;
                 }
             }
         }
@@ -336,7 +295,6 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
             }
         };
         double ra[kTileLoads], rb[kTileLoads];
-        float2 rbf[kTileLoads];
         auto fetch = [&](int t) {
             bool inv;
             int I, Jb;
@@ -346,9 +304,7 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
             for (int u = 0; u < kTileLoads; ++u) {
                 const int e = tid + u * kPotrfThreads, r = e % kBlk, k = e / kBlk;
                 ra[u] = (r < rows && k < w) ? __ldcg(A + (int64_t)(p + k) * lda + ri + r) : 0.0;
-                if (kFF && inv)
-                    rbf[u] = (r < cols && k < w) ? __ldcg(X2 + (int64_t)(cj + r) * ldx + p + k) : make_float2(0.f, 0.f);
-                else if (inv) rb[u] = (r < cols && k < w) ? __ldcg(X + (int64_t)(cj + r) * ldx + p + k) : 0.0;
+                if (inv) rb[u] = (r < cols && k < w) ? __ldcg(X + (int64_t)(cj + r) * ldx + p + k) : 0.0;
                 else rb[u] = (r < cols && k < w) ? __ldcg(A + (int64_t)(p + k) * lda + cj + r) : 0.0;
             }
         };
@@ -361,25 +317,38 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
 #pragma unroll
             for (int u = 0; u < kTileLoads; ++u) {
                 const int e = tid + u * kPotrfThreads;
-                if (kFF && inv) {
-                    saf[e % kBlk][e / kBlk] = ff_split(ra[u]);
-                    sbf[e % kBlk][e / kBlk] = rbf[u];
-                } else {
-                    sa[e % kBlk][e / kBlk] = ra[u];
-                    sb[e % kBlk][e / kBlk] = rb[u];
-                }
+                sa[e % kBlk][e / kBlk] = ra[u];
+                sb[e % kBlk][e / kBlk] = rb[u];
             }
             __syncthreads();
             return inv ? (X + (int64_t)cj * ldx + ri) : (A + (int64_t)cj * lda + ri);
         };
         if (rank == 0) {
-            // tile (kb+1, kb+1), then the next diagonal block
-            fetch(0);
-            double *C = apply(0);
-            tile_update32(C, lda, sa, sb, min(kBlk, m - (kb + 1) * kBlk), min(kBlk, m - (kb + 1) * kBlk), true);
-            __syncthreads();
+            // tile (kb+1, kb+1): its lower triangle, entry e in packed order,
+            // then the next diagonal block
             const int pn = (kb + 1) * kBlk, wn = min(kBlk, m - pn);
-            const int bad = potrf_diag_block(A, lda, pn, wn, dinv + (int64_t)(kb + 1) * kBlk * kBlk, sa, sl, &s_bad);
+            fetch(0);
+            apply(0);
+            for (int e = tid; e < kBlk * (kBlk + 1) / 2; e += kPotrfThreads) {
+                int r = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+                r += (r + 1) * (r + 2) / 2 <= e;
+                r -= r * (r + 1) / 2 > e;
+                const int c = e - r * (r + 1) / 2;
+                double v = 0.0;
+                if (r < wn) {
+                    v = __ldcg(A + (int64_t)(pn + c) * lda + pn + r);
+                    double x0 = 0.0, x1 = 0.0;
+#pragma unroll 8
+                    for (int k = 0; k < kBlk; k += 2) {
+                        x0 = fma(sa[r][k], sa[c][k], x0);
+                        x1 = fma(sa[r][k + 1], sa[c][k + 1], x1);
+                    }
+                    v -= x0 + x1;
+                }
+                sl[r][c] = v;
+            }
+            __syncthreads();
+            const int bad = potrf_diag_block(A, lda, pn, wn, dinv + (int64_t)(kb + 1) * kBlk * kBlk, sl, ov, &sy, &s_bad);
             if (bad >= 0 && tid == 0) {
                 set_status(st, TLR_ERR_NOT_SPD, row_base + pn + bad);
                 __stcg(stop, 1LL);
@@ -394,21 +363,16 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
                 const int ri = I * kBlk, cj = Jb * kBlk, rows = min(kBlk, m - ri), cols = min(kBlk, m - cj);
                 double *C = apply(t);
                 if (t + step < ntot) fetch(t + step);
-                if (kFF && inv) tile_update32_ff(reinterpret_cast<float2 *>(C), ldx, saf, sbf, rows, cols);
-                else tile_update32(C, inv ? ldx : lda, sa, sb, rows, cols, !inv && I == Jb);
+                tile_update32(C, inv ? ldx : lda, sa, sb, rows, cols, !inv && I == Jb);
             }
         }
         cl.sync();
         if (__ldcg(stop)) return;  // written by CTA 0 only, before the barrier
     }
-    // zero the strict upper triangle of the factor; the paired inverse to doubles
+    // zero the strict upper triangle of the factor
     for (int64_t e = gtid; e < (int64_t)m * m; e += gthreads) {
         const int r = (int)(e % m), c = (int)(e / m);
         if (r < c) A[(int64_t)c * lda + r] = 0.0;
-        if constexpr (kFF) {
-            const float2 v = X2[(int64_t)c * ldx + r];
-            X[(int64_t)c * ldx + r] = (double)v.x + (double)v.y;
-        }
     }
 }
 
@@ -488,26 +452,11 @@ void trsm_left_lower(tlr_ctx *ctx, cudaStream_t s, const double *L, int ldl, int
     }
 }
 
-void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs, bool ff_inverse) {
-    std::vector<PotrfJob> act;
-    for (const PotrfJob &J : jobs) {
-        if (J.m <= 0) continue;
-        if (J.m > kBlk * kBlk) throw make_error(TLR_ERR_ARG, "tile too large for the cluster POTRF (%d)", J.m);
-        act.push_back(J);
-    }
-    if (act.empty()) return;
-    if ((int)act.size() > kMaxGroup) throw make_error(TLR_ERR_ARG, "more than %d diagonal tiles in one launch", kMaxGroup);
+// One cluster launch for the blocks of `act` (m <= 1024 each): Cholesky and inverse.
+static void potrf_cluster(tlr_ctx *ctx, cudaStream_t s, const std::vector<PotrfJob> &act) {
+    PotrfBatch b{};
     // scratch per job: the diagonal-block inverses and the cluster's stop word
     const size_t per = (size_t)kBlk * kBlk * kBlk + 8;
-    if ((int)act.size() > ctx->potrf_scratch_jobs) {
-        if (ctx->d_potrf_scratch) TLR_CUDA_TRY(cudaFree(ctx->d_potrf_scratch));  // syncs the device
-        ctx->d_potrf_scratch = nullptr;
-        ctx->potrf_scratch_jobs = 0;
-        const int want = std::max((int)act.size(), 2 * ctx->potrf_scratch_jobs);
-        TLR_CUDA_TRY(cudaMalloc(&ctx->d_potrf_scratch, per * want * sizeof(double)));
-        ctx->potrf_scratch_jobs = want;
-    }
-    PotrfBatch b{};
     for (size_t q = 0; q < act.size(); ++q) {
         b.job[q] = act[q];
         b.job[q].scratch = ctx->d_potrf_scratch + per * q;
@@ -515,10 +464,7 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs,
     static std::once_flag once;
     static int csize = 8;  // 16 CTAs where the device runs such clusters, else 8
     std::call_once(once, [] {
-        if (cudaFuncSetAttribute(k_potrf_inv<16, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                cudaSuccess &&
-            cudaFuncSetAttribute(k_potrf_inv<16, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                cudaSuccess) {
+        if (cudaFuncSetAttribute(k_potrf_inv<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(16);
             cfg.blockDim = dim3(kPotrfThreads);
@@ -530,18 +476,161 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs,
             cfg.attrs = attr;
             cfg.numAttrs = 1;
             int nclusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&nclusters, k_potrf_inv<16, true>, &cfg) == cudaSuccess && nclusters > 0)
+            if (cudaOccupancyMaxActiveClusters(&nclusters, k_potrf_inv<16>, &cfg) == cudaSuccess && nclusters > 0)
                 csize = 16;
         }
         cudaGetLastError();  // clear any error of the queries
     });
     const int nc = (int)act.size();
-    if (csize == 16) {
-        if (ff_inverse) launch_clustered(k_potrf_inv<16, true>, 16, nc, kPotrfThreads, 0, s, b);
-        else launch_clustered(k_potrf_inv<16, false>, 16, nc, kPotrfThreads, 0, s, b);
-    } else {
-        if (ff_inverse) launch_clustered(k_potrf_inv<8, true>, 8, nc, kPotrfThreads, 0, s, b);
-        else launch_clustered(k_potrf_inv<8, false>, 8, nc, kPotrfThreads, 0, s, b);
+    if (csize == 16) launch_clustered(k_potrf_inv<16>, 16, nc, kPotrfThreads, 0, s, b);
+    else launch_clustered(k_potrf_inv<8>, 8, nc, kPotrfThreads, 0, s, b);
+}
+
+// Around the diagonal blocks (width w) of a tile that is factored in blocks:
+// zero A above them, X and S outside them.
+struct PotrfEdge {
+    double *A, *X, *S;
+    int lda, ldx, lds, m, w;
+};
+struct PotrfEdges {
+    PotrfEdge e[kMaxGroup];
+};
+__global__ void k_potrf_edges(const PotrfEdges jobs) {
+    const PotrfEdge J = jobs.e[blockIdx.y];
+    for (int c = blockIdx.x; c < J.m; c += gridDim.x) {
+        const int b0 = c / J.w * J.w, b1 = min(J.m, b0 + J.w);
+        for (int r = threadIdx.x; r < J.m; r += blockDim.x) {
+            if (r < b0) J.A[(int64_t)c * J.lda + r] = 0.0;
+            if (r < b0 || r >= b1) {
+                J.X[(int64_t)c * J.ldx + r] = 0.0;
+                J.S[(int64_t)c * J.lds + r] = 0.0;
+            }
+        }
+    }
+}
+
+// Tiles wider than kPotrfOuter are factored in blocks of w <= kPotrfOuter
+// columns: the cluster kernel factors and inverts a diagonal block, and the
+// products between blocks run as batched FP64 GEMMs over the whole GPU.  For
+// block b, with X_bb = L_bb^-1:
+//   L_ib = A_ib X_bb'  (i > b);   A_ij -= L_ib L_jb'  (i >= j > b);
+//   X_bj = X_bb S_bj  (j < b);    S_ij -= L_ib X_bj  (i > b >= j),
+// S_ij the negated sum of L_ik X_kj so far.  One cluster alone runs the tile's
+// m^3 / 3 multiply-adds twice over on 16 of the 152 SMs: at m = 800 its
+// trailing updates, not its pivot chain, took most of 4.1 ms alone; in blocks
+// it takes 1.8 ms (three cluster launches of 0.33, the GEMMs 0.8).  Widths of
+// 224 and 160 took 1.95 and 1.99 ms: more launches, each as long as one 32 x 32
+// output tile's FP64 chain.  The GEMMs are split by column chunks so that the
+// triangular factors' zeros are skipped.  X_bb has to be FP64: L_ib is formed
+// from it (with a float-float inverse |L L' - A| was 1.2e-14, not 9e-16).
+constexpr int kPotrfOuter = 288, kPotrfChunk = 96;
+
+void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs) {
+    std::vector<PotrfJob> act;
+    for (const PotrfJob &J : jobs) {
+        if (J.m <= 0) continue;
+        if (J.m > kBlk * kBlk) throw make_error(TLR_ERR_ARG, "tile too large for the cluster POTRF (%d)", J.m);
+        act.push_back(J);
+    }
+    if (act.empty()) return;
+    if ((int)act.size() > kMaxGroup) throw make_error(TLR_ERR_ARG, "more than %d diagonal tiles in one launch", kMaxGroup);
+    const size_t per = (size_t)kBlk * kBlk * kBlk + 8;
+    if ((int)act.size() > ctx->potrf_scratch_jobs) {
+        if (ctx->d_potrf_scratch) TLR_CUDA_TRY(cudaFree(ctx->d_potrf_scratch));  // syncs the device
+        ctx->d_potrf_scratch = nullptr;
+        ctx->potrf_scratch_jobs = 0;
+        const int want = std::max((int)act.size(), 2 * ctx->potrf_scratch_jobs);
+        TLR_CUDA_TRY(cudaMalloc(&ctx->d_potrf_scratch, per * want * sizeof(double)));
+        ctx->potrf_scratch_jobs = want;
+    }
+    // per job: block width and count, and the scratch panels P (L_ib before it
+    // replaces A_ib) and S, both with leading dimension m
+    struct Blocked {
+        int w = 0, n = 1;
+        double *P = nullptr, *S = nullptr;
+    };
+    std::vector<Blocked> bl(act.size());
+    size_t words = 0;
+    int blocks = 1;
+    for (size_t q = 0; q < act.size(); ++q) {
+        const int m = act[q].m;
+        bl[q].w = m;
+        if (m <= kPotrfOuter) continue;
+        bl[q].n = (int)ceil_div(m, kPotrfOuter);
+        bl[q].w = (int)(ceil_div(ceil_div(m, bl[q].n), kBlk) * kBlk);
+        bl[q].n = (int)ceil_div(m, bl[q].w);
+        blocks = std::max(blocks, bl[q].n);
+        words += (size_t)m * (m + bl[q].w);
+    }
+    if (blocks == 1) {
+        potrf_cluster(ctx, s, act);
+        return;
+    }
+    DevBuf buf(words * sizeof(double), s);
+    PotrfEdges edges{};
+    int nedge = 0, mmax = 0;
+    words = 0;
+    for (size_t q = 0; q < act.size(); ++q) {
+        if (bl[q].n == 1) continue;
+        const PotrfJob &J = act[q];
+        bl[q].P = buf.as<double>() + words;
+        bl[q].S = bl[q].P + (size_t)J.m * bl[q].w;
+        words += (size_t)J.m * (J.m + bl[q].w);
+        edges.e[nedge++] = PotrfEdge{J.A, J.X, bl[q].S, J.lda, J.ldx, J.m, J.m, bl[q].w};
+        mmax = std::max(mmax, J.m);
+    }
+    launch(k_potrf_edges, dim3((unsigned)std::min(mmax, 256), (unsigned)nedge), 256, 0, s, edges);
+    TLR_CHECK_LAUNCH();
+    auto prob = [](const double *A, int lda, const double *B, int ldb, double *C, int ldc, int m, int n, int k) {
+        GemmProb g{};
+        g.A = A; g.lda = lda; g.B = B; g.ldb = ldb; g.C = C; g.ldc = ldc;
+        g.m = m; g.n = n; g.k = k;
+        return g;
+    };
+    for (int b = 0; b < blocks; ++b) {
+        std::vector<PotrfJob> diag;
+        std::vector<GemmProb> gx, gl, ga, gs;
+        std::vector<CopyDesc> cl;
+        for (size_t q = 0; q < act.size(); ++q) {
+            const PotrfJob &J = act[q];
+            const Blocked &B = bl[q];
+            if (b >= B.n) continue;
+            const int p = b * B.w, w = std::min(B.w, J.m - p), e = p + w, rest = J.m - e;
+            PotrfJob D = J;
+            D.A = J.A + (int64_t)p * J.lda + p;
+            D.X = J.X + (int64_t)p * J.ldx + p;
+            D.m = w;
+            D.row_base = J.row_base + p;
+            diag.push_back(D);
+            if (B.n == 1) continue;
+            for (int c0 = 0; c0 < w; c0 += kPotrfChunk) {
+                const int c1 = std::min(w, c0 + kPotrfChunk);
+                // X_bj, rows c0 .. c1: X_bb is zero right of column c1
+                if (p > 0) gx.push_back(prob(D.X + c0, J.ldx, B.S + p, J.m, J.X + p + c0, J.ldx, c1 - c0, p, c1));
+                if (rest <= 0) continue;
+                // L_ib, columns c0 .. c1
+                gl.push_back(prob(J.A + (int64_t)p * J.lda + e, J.lda, D.X + c0, J.ldx, B.P + (int64_t)c0 * J.m + e, J.m,
+                                  rest, c1 - c0, c1));
+                // S_ib, columns c0 .. c1: X_bb is zero above row c0
+                gs.push_back(prob(B.P + (int64_t)c0 * J.m + e, J.m, D.X + (int64_t)c0 * J.ldx + c0, J.ldx,
+                                  B.S + (int64_t)(p + c0) * J.m + e, J.m, rest, c1 - c0, w - c0));
+            }
+            if (rest <= 0) continue;
+            if (p > 0) gs.push_back(prob(B.P + e, J.m, J.X + p, J.ldx, B.S + e, J.m, rest, p, w));
+            // lower part of the trailing matrix; no chunk crosses a block
+            // boundary, so that nothing above the diagonal blocks is written
+            for (int c0 = e, c1; c0 < J.m; c0 = c1) {
+                c1 = std::min({J.m, c0 + kPotrfChunk, (c0 / B.w + 1) * B.w});
+                ga.push_back(prob(B.P + c0, J.m, B.P + c0, J.m, J.A + (int64_t)c0 * J.lda + c0, J.lda, J.m - c0, c1 - c0, w));
+            }
+            cl.push_back(CopyDesc{B.P + e, J.m, J.A + (int64_t)p * J.lda + e, J.lda, rest, w});
+        }
+        potrf_cluster(ctx, s, diag);
+        gemm_batched_small(ctx, s, false, true, gl, 1.0, 0.0);   // L
+        gemm_batched_small(ctx, s, false, true, ga, -1.0, 1.0);  // trailing update
+        gemm_batched_small(ctx, s, false, false, gx, 1.0, 0.0);  // X_bj
+        gemm_batched_small(ctx, s, false, false, gs, -1.0, 1.0);  // S
+        copy_batched(ctx, s, cl);
     }
 }
 

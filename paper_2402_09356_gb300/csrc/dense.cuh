@@ -14,12 +14,13 @@ struct RhsDesc {
 };
 
 // A = L L' in place (lower; strict upper zeroed) and X = L^-1 (m x m, lower,
-// ld ldx) in one launch on one thread-block cluster; m <= 1024.  A
+// ld ldx), both in FP64; m <= 1024.  One launch on one thread-block cluster up
+// to 288 rows, in blocks with batched products between them above.  A
 // non-positive pivot sets NOT_SPD (info = row_base + local row); X is then
 // not written.
 void potrf_inv(tlr_ctx *ctx, cudaStream_t s, double *A, int lda, int m, double *X, int ldx, long long row_base);
 
-// The same for several tiles in one launch (one cluster each); every job
+// The same for several tiles, sharing every launch (one cluster each); every job
 // reports a non-positive pivot in its own status word st.  scratch is set by
 // the call.
 struct PotrfJob {
@@ -34,9 +35,7 @@ struct PotrfJob {
 struct PotrfBatch {
     PotrfJob job[kMaxGroup];
 };
-// ff_inverse: X in float-float arithmetic (~1e-14 relative), the factor in
-// FP64 (the paired-FP32 paths, whose products with X are paired FP32).
-void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs, bool ff_inverse = false);
+void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs);
 
 // B <- L^-1 B for every right-hand side matrix (L lower triangular m x m).
 void trsm_left_lower(tlr_ctx *ctx, cudaStream_t s, const double *L, int ldl, int m,

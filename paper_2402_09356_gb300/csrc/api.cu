@@ -204,7 +204,7 @@ int tlr_ctx_create(int device, tlr_ctx **out) {
             TLR_CUDA_TRY(cudaHostAlloc(&R.h, R.cap, cudaHostAllocDefault));
             TLR_CUDA_TRY(cudaMalloc(&R.d, R.cap));
         }
-        TLR_CUDA_TRY(cudaMalloc(&ctx->d_mtab, 2 * (size_t)kTabIntervals * kTabCoef * sizeof(double)));
+        TLR_CUDA_TRY(cudaMalloc(&ctx->d_mtab, (size_t)kTabBuild * sizeof(double)));
         // workspaces come from the device's default stream-ordered pool; keep
         // what is freed cached there instead of returning it to the driver at
         // every synchronisation (a factorisation syncs once per tile column,
@@ -659,14 +659,13 @@ static void loglik_group_once(tlr_ctx *ctx, const std::vector<BatchEntry *> &es,
         }
         return;
     }
-    const int cnt = kTabIntervals * kTabCoef;
     std::vector<MaternParams> P(G);
     std::vector<FactorStats> st(G);
     std::vector<long long> info(G, -1);
     int64_t ntot = 0;
     for (BatchEntry *e : es) ntot += e->n;
     TLR_CUDA_TRY(cudaEventRecord(ctx->ev_a, s));
-    DevBuf tabs((size_t)G * 2 * cnt * sizeof(double), s);
+    DevBuf tabs((size_t)G * kTabBuild * sizeof(double), s);
     DevBuf acc((size_t)G * 3 * sizeof(double), s), y((size_t)ntot * sizeof(double), s);
     TLR_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, (size_t)(G + 1) * sizeof(DevStatus), s));
     TLR_CUDA_TRY(cudaMemsetAsync(acc.as<double>(), 0, (size_t)G * 3 * sizeof(double), s));
@@ -678,7 +677,7 @@ static void loglik_group_once(tlr_ctx *ctx, const std::vector<BatchEntry *> &es,
         e.out->info = -1;
         e.out->precision_used = tc ? TLR_PREC_TENSOR : (df ? TLR_PREC_MIXED : TLR_PREC_FP64);
         P[(size_t)g] = params_of(e.theta);
-        build_matern_table(&P[(size_t)g], tabs.as<double>() + (size_t)g * 2 * cnt, s);
+        build_matern_table(&P[(size_t)g], tabs.as<double>() + (size_t)g * kTabBuild, s);
         FactorItem &F = items[(size_t)g];
         F.M = e.L;
         F.xy = e.xy;

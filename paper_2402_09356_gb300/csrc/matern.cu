@@ -112,7 +112,7 @@ __global__ void k_generate_tiles(const double *__restrict__ xy, int64_t n, int n
     int64_t t = (int64_t)blockIdx.x / (sub * sub);
     int sb = (int)((int64_t)blockIdx.x % (sub * sub));
     // tile (i, j) from packed index t = i (i + 1) / 2 + j
-    int i = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+    int i = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);  // corrected below
     while ((int64_t)(i + 1) * (i + 2) / 2 <= t) ++i;
     while ((int64_t)i * (i + 1) / 2 > t) --i;
     int j = (int)(t - (int64_t)i * (i + 1) / 2);
@@ -163,7 +163,7 @@ __global__ void k_matern_vec(const double *__restrict__ d, int64_t m, MaternPara
     else out[k] = P.sigma2 * matern_corr_x(v * P.inv_beta, P);
 }
 
-// Table nodes: log C/sigma2 at the Chebyshev points of every interval.
+// Table nodes: log2 C/sigma2 at the Chebyshev points of every interval.
 __global__ void k_table_nodes(MaternParams P, double *__restrict__ g) {
     int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= kTabIntervals * kTabCoef) return;
@@ -173,36 +173,54 @@ __global__ void k_table_nodes(MaternParams P, double *__restrict__ g) {
     double node = cospi((k + 0.5) / kTabCoef);
     double sv = lo + 0.5 * (node + 1.0) * (hi - lo);
     double c = matern_corr_x(sqrt(sv) * P.inv_beta, P);
-    g[q] = (c > 1e-280) ? log(c) : __longlong_as_double(0x7FF8000000000000ll);
+    g[q] = (c > 1e-280) ? log2(c) : __longlong_as_double(0x7FF8000000000000ll);
 }
 
-// Chebyshev coefficients c_j = (2/N) sum_k g_k cos(j pi (k + 1/2) / N), c_0 halved;
-// an interval with a non-finite node value keeps c_0 = NaN (direct evaluation).
+// Coefficients a_i of the interpolant in powers of t, from the Chebyshev
+// coefficients c_j = (2/N) sum_k g_k cos(j pi (k + 1/2) / N), c_0 halved, and
+// T_{j+1} = 2 t T_j - T_{j-1}; an interval with a non-finite node value keeps
+// a_0 = NaN (direct evaluation).  The last entries are 2^(j/32).
 __global__ void k_table_coefs(const double *__restrict__ g, double *__restrict__ tab) {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= kTabIntervals * kTabCoef) return;
-    int iv = q / kTabCoef, j = q % kTabCoef;
-    const double *gi = g + iv * kTabCoef;
-    double acc = 0.0;
+    const int iv = blockIdx.x * blockDim.x + threadIdx.x;
+    if (iv < kTabExp) tab[kTabIntervals * kTabCoef + iv] = exp2((double)iv / kTabExp);
+    if (iv >= kTabIntervals) return;
+    double gi[kTabCoef], a[kTabCoef], t0[kTabCoef], t1[kTabCoef];
     bool bad = false;
+#pragma unroll
     for (int k = 0; k < kTabCoef; ++k) {
-        double v = gi[k];
-        bad |= !(v == v);
-        acc += v * cospi((double)j * (k + 0.5) / kTabCoef);
+        gi[k] = g[iv * kTabCoef + k];
+        bad |= !(gi[k] == gi[k]);
+        a[k] = t0[k] = t1[k] = 0.0;
     }
-    acc *= 2.0 / kTabCoef;
-    if (j == 0) acc *= 0.5;
-    if (bad && j == 0) acc = __longlong_as_double(0x7FF8000000000000ll);
-    tab[q] = acc;
+    t0[0] = 1.0;
+    t1[1] = 1.0;
+    for (int j = 0; j < kTabCoef; ++j) {
+        double c = 0.0;
+#pragma unroll
+        for (int k = 0; k < kTabCoef; ++k) c += gi[k] * cospi((double)j * (k + 0.5) / kTabCoef);
+        c *= (j ? 2.0 : 1.0) / kTabCoef;
+        // t0 = T_j, t1 = T_{j+1}
+#pragma unroll
+        for (int i = 0; i < kTabCoef; ++i) a[i] += c * t0[i];
+#pragma unroll
+        for (int i = kTabCoef - 1; i >= 0; --i) {
+            const double n = (i > 0 ? 2.0 * t1[i - 1] : 0.0) - t0[i];
+            t0[i] = t1[i];
+            t1[i] = n;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kTabCoef; ++i)
+        tab[iv * kTabCoef + i] = bad && i == 0 ? __longlong_as_double(0x7FF8000000000000ll) : a[i];
 }
 
 void build_matern_table(MaternParams *P, double *tab, cudaStream_t s) {
     const int cnt = kTabIntervals * kTabCoef;
-    double *g = tab + cnt;  // scratch: the caller provides 2 * cnt doubles
+    double *g = tab + kTabDoubles;  // scratch: the caller provides kTabBuild doubles
     MaternParams direct = *P;
     direct.tab = nullptr;
-    launch(k_table_nodes, (unsigned)ceil_div(cnt, 128), 128, 0, s, direct, g);
-    launch(k_table_coefs, (unsigned)ceil_div(cnt, 128), 128, 0, s, g, tab);
+    launch(k_table_nodes, (unsigned)ceil_div(cnt, 64), 64, 0, s, direct, g);
+    launch(k_table_coefs, (unsigned)ceil_div(kTabIntervals, 64), 64, 0, s, g, tab);
     TLR_CHECK_LAUNCH();
     P->tab = tab;
 }

@@ -34,21 +34,28 @@ constexpr int kTemmeTerms = 22;   // (x^2/4)^k / k! < 1e-21 at x = 2
 constexpr int kISeriesTerms = 64; // I-series terms for x <= 25
 constexpr int kAsymTerms = 30;    // asymptotic terms for x > 25
 
-// Per-theta interpolation table of log C(d)/sigma2 as a function of s = d^2:
+// Per-theta interpolation table of log2 C(d)/sigma2 as a function of s = d^2:
 // each binade [2^e, 2^(e+1)) of s (kTabEmin <= e <= kTabEmax) is split into
 // kTabSub equal sub-intervals, and on each the function is replaced by its
-// degree-kTabDeg Chebyshev interpolant.  log C is analytic on each interval
-// (its only singularity is s = 0), so the interpolants converge
-// geometrically; with these sizes the error is below 1e-13 relative.  An
-// interval whose nodes underflow is flagged (c_0 = NaN) and evaluated
-// directly.
-constexpr int kTabEmin = -44, kTabEmax = 3, kTabSub = 4, kTabDeg = 12;
+// degree-7 Chebyshev interpolant, kept in powers of t in [-1, 1].  log2 C is
+// analytic on each interval (its only singularity is s = 0, 65 half-widths
+// away), so the remainder is below 1e-16 relative to C where C > 1e-20.  An
+// interval whose nodes underflow is flagged (a_0 = NaN) and evaluated directly.
+// An entry then costs 23 FP64 operations, which bound the generation (an FP64
+// warp instruction takes 64 cycles): 4 for s, 1 for t, 7 for the polynomial, 10
+// for 2^f and 1 for sigma2.  Four sub-intervals of degree 12 by Clenshaw and
+// exp() cost about 53: 10,000 points, tile 1000, 5.7 ms against 2.6.  The eight
+// coefficients are one 64-byte line; the table is 98 KB.
+constexpr int kTabEmin = -44, kTabEmax = 3, kTabSubBits = 5, kTabSub = 1 << kTabSubBits, kTabDeg = 7;
 constexpr int kTabIntervals = (kTabEmax - kTabEmin + 1) * kTabSub;
 constexpr int kTabCoef = kTabDeg + 1;
+constexpr int kTabExp = 32;  // entries 2^(j/32) behind the coefficients
+constexpr int kTabDoubles = kTabIntervals * kTabCoef + kTabExp;
+constexpr int kTabBuild = 2 * kTabDoubles;  // table and scratch of build_matern_table
 
 struct MaternParams {
     double sigma2, inv_beta, nu;
-    const double *tab;  // kTabIntervals x kTabCoef Chebyshev coefficients, or null (direct K_nu)
+    const double *tab;  // kTabIntervals x kTabCoef coefficients and 2^(j/32), or null (direct K_nu)
     double mu;
     int m;
     double lead;       // 2^(1-nu) / Gamma(nu)
@@ -168,28 +175,48 @@ __device__ __forceinline__ double matern_corr_x(double x, const MaternParams &P)
     return P.lead * exp(P.nu * lx - (scaled ? x : 0.0)) * kn;
 }
 
+// 2^f for -1000 < f < 1: f = n / 32 + r, |r| <= 1/64, 2^(n mod 32 / 32) from
+// the table and 2^r = exp(r ln 2) by its Taylor polynomial of degree 6 (the
+// remainder (ln 2 / 64)^7 / 7! is 4e-18).
+__device__ __forceinline__ double exp2_tab(double f, const double *__restrict__ e32) {
+    const double magic = 211106232532992.0;  // 1.5 * 2^47: the sum rounds f to multiples of 1/32
+    const double z = f + magic;
+    const int n = (int)__double2loint(z);
+    const double r = f - (z - magic);
+    double p = 1.5403530393381606e-4;  // ln2^k / k!, k = 6 .. 1
+    p = fma(p, r, 1.3333558146428441e-3);
+    p = fma(p, r, 9.618129107628477e-3);
+    p = fma(p, r, 5.5504108664821576e-2);
+    p = fma(p, r, 0.2402265069591007);
+    p = fma(p, r, 0.6931471805599453);
+    const double b = __ldg(e32 + (n & (kTabExp - 1)));
+    const double v = fma(p * r, b, b);
+    return __hiloint2double(__double2hiint(v) + ((n >> 5) << 20), __double2loint(v));
+}
+
 // C(d)/sigma2 from the squared distance s > 0 through the table (falls back to
 // the direct K_nu outside the table or on flagged intervals).
 __device__ __forceinline__ double matern_corr_s(double s, const MaternParams &P) {
     if (P.tab) {
-        long long bits = __double_as_longlong(s);
-        int e = (int)((bits >> 52) & 0x7FF) - 1023;
-        if (e >= kTabEmin && e <= kTabEmax) {
-            int sub = (int)((bits >> 50) & 3);
-            // fraction of the binade in [0, 1), exact
-            double u = (double)(bits & 0xFFFFFFFFFFFFFll) * 2.220446049250313e-16;
-            double t = 2.0 * (u * kTabSub - (double)sub) - 1.0;
-            const double *c = P.tab + ((e - kTabEmin) * kTabSub + sub) * kTabCoef;
-            double c0 = __ldg(c);
-            if (c0 == c0) {
-                double b1 = 0.0, b2 = 0.0, t2 = 2.0 * t;
-#pragma unroll
-                for (int j = kTabDeg; j >= 1; --j) {
-                    double b0 = fma(t2, b1, __ldg(c + j) - b2);
-                    b2 = b1;
-                    b1 = b0;
-                }
-                return exp(fma(t, b1, c0 - b2));
+        const unsigned hi = (unsigned)__double2hiint(s), lo = (unsigned)__double2loint(s);
+        // (exponent, leading kTabSubBits of the mantissa) in one field
+        const int iv = (int)(hi >> (20 - kTabSubBits)) - ((kTabEmin + 1023) << kTabSubBits);
+        if (iv >= 0 && iv < kTabIntervals) {
+            // the rest of the mantissa as w in [1, 2): t = 2 w - 3 in [-1, 1)
+            const unsigned mh = ((hi << kTabSubBits) | (lo >> (32 - kTabSubBits))) & 0xFFFFFu;
+            const double w = __hiloint2double((int)(0x3FF00000u | mh), (int)(lo << kTabSubBits));
+            const double t = fma(2.0, w, -3.0);
+            const double2 *c = reinterpret_cast<const double2 *>(P.tab) + iv * (kTabCoef / 2);
+            const double2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2), c3 = __ldg(c + 3);
+            if ((__double2hiint(c0.x) & 0x7FF00000) != 0x7FF00000) {
+                double f = fma(c3.y, t, c3.x);
+                f = fma(f, t, c2.y);
+                f = fma(f, t, c2.x);
+                f = fma(f, t, c1.y);
+                f = fma(f, t, c1.x);
+                f = fma(f, t, c0.y);
+                f = fma(f, t, c0.x);
+                return exp2_tab(f, P.tab + kTabIntervals * kTabCoef);
             }
         }
     }
@@ -201,7 +228,7 @@ __device__ __forceinline__ double matern_cov(double xa, double ya, double xb, do
                                              const MaternParams &P) {
     double dx = xa - xb, dy = ya - yb;
     double s = dx * dx + dy * dy;
-    if (s == 0.0) return P.sigma2;
+    if ((__double2hiint(s) | __double2loint(s)) == 0) return P.sigma2;  // s >= 0: no FP64 comparison
     return P.sigma2 * matern_corr_s(s, P);
 }
 
@@ -209,8 +236,8 @@ __device__ __forceinline__ double matern_cov(double xa, double ya, double xb, do
 // The table pointer is left null (direct K_nu).
 bool make_matern_params(double sigma2, double beta, double nu, MaternParams *out);
 
-// Build the interpolation table of P into `tab` (kTabIntervals * kTabCoef
-// doubles, device) on stream s and point P->tab at it.
+// Build the interpolation table of P into `tab` (kTabBuild doubles, device,
+// 64-byte aligned) on stream s and point P->tab at it.
 void build_matern_table(MaternParams *P, double *tab, cudaStream_t s);
 
 }  // namespace tlr

@@ -1,7 +1,6 @@
 // Dense FP64 tile kernels of the TLR Cholesky (Sec. 2; the diagonal tiles stay
-// dense): blocked right-looking Cholesky of one diagonal tile, forward
-// substitution with many right-hand sides, and the log-determinant /
-// quadratic-form reductions of Eq. 1.2.
+// dense): blocked right-looking Cholesky of one diagonal tile with its
+// inverse, and the log-determinant / quadratic-form reductions of Eq. 1.2.
 //
 // Blocks of 32 rows/columns are factored or solved by one CTA in shared
 // memory; everything else is a batched GEMM update so that it spreads over
@@ -373,82 +372,6 @@ __global__ void __launch_bounds__(kPotrfThreads) k_potrf_inv(const PotrfBatch jo
     for (int64_t e = gtid; e < (int64_t)m * m; e += gthreads) {
         const int r = (int)(e % m), c = (int)(e / m);
         if (r < c) A[(int64_t)c * lda + r] = 0.0;
-    }
-}
-
-// Solve L X = B for the 32-row block at p0 of every right-hand side column.
-// Columns of all problems are concatenated; col_off gives each problem's start.
-__global__ void k_trsm_left_block(const double *__restrict__ Lm, int ldl, int m, int p0,
-                                  const RhsDesc *__restrict__ rhs, const int *__restrict__ col_off,
-                                  int nrhs, const DevStatus *st) {
-    __shared__ double L[kBlk][kBlk + 1];
-    if (st->code) return;
-    const int w = min(kBlk, m - p0);
-    const double *Lb = Lm + (int64_t)p0 * ldl + p0;
-    for (int e = threadIdx.x; e < kBlk * kBlk; e += blockDim.x) {
-        int rr = e % kBlk, cc = e / kBlk;
-        L[rr][cc] = (rr < w && cc < w && cc <= rr) ? Lb[(int64_t)cc * ldl + rr] : 0.0;
-    }
-    __syncthreads();
-    int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= col_off[nrhs]) return;
-    int lo = 0, hi = nrhs - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (col_off[mid] <= col) lo = mid; else hi = mid - 1;
-    }
-    const RhsDesc d = rhs[lo];
-    double *b = d.B + (int64_t)(col - col_off[lo]) * d.ld + p0;
-    double x[kBlk];
-#pragma unroll
-    for (int r = 0; r < kBlk; ++r) {
-        if (r < w) {
-            double a = b[r];
-#pragma unroll
-            for (int k = 0; k < r; ++k) a -= L[r][k] * x[k];
-            x[r] = a / L[r][r];
-        } else {
-            x[r] = 0.0;
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < kBlk; ++r)
-        if (r < w) b[r] = x[r];
-}
-
-void trsm_left_lower(tlr_ctx *ctx, cudaStream_t s, const double *L, int ldl, int m,
-                     const std::vector<RhsDesc> &rhs) {
-    std::vector<RhsDesc> act;
-    for (const RhsDesc &d : rhs)
-        if (d.ncols > 0) act.push_back(d);
-    if (act.empty() || m <= 0) return;
-    std::vector<int> off(act.size() + 1, 0);
-    for (size_t b = 0; b < act.size(); ++b) off[b + 1] = off[b] + act[b].ncols;
-    auto *dr = (const RhsDesc *)stage_push(ctx, act.data(), act.size() * sizeof(RhsDesc), s);
-    auto *doff = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
-    int total = off.back();
-    for (int p0 = 0; p0 < m; p0 += kBlk) {
-        int w = std::min(kBlk, m - p0);
-        launch(k_trsm_left_block, (unsigned)ceil_div(total, 128), 128, 0, s, L, ldl, m, p0, dr, doff,
-                                                                         (int)act.size(), ctx->d_status);
-        TLR_CHECK_LAUNCH();
-        int rest = m - p0 - w;
-        if (rest <= 0) break;
-        std::vector<GemmProb> probs;
-        for (const RhsDesc &d : act) {
-            GemmProb g{};
-            g.A = L + (int64_t)p0 * ldl + p0 + w;
-            g.B = d.B + p0;
-            g.C = d.B + p0 + w;
-            g.m = rest;
-            g.n = d.ncols;
-            g.k = w;
-            g.lda = ldl;
-            g.ldb = d.ld;
-            g.ldc = d.ld;
-            probs.push_back(g);
-        }
-        gemm_batched(ctx, s, false, false, probs, -1.0, 1.0);
     }
 }
 

@@ -5,14 +5,6 @@
 
 namespace tlr {
 
-// One right-hand side matrix of a batched triangular solve: m x ncols, column
-// major with leading dimension ld, solved in place.
-struct RhsDesc {
-    double *B;
-    int ncols;
-    int ld;
-};
-
 // A = L L' in place (lower; strict upper zeroed) and X = L^-1 (m x m, lower,
 // ld ldx), both in FP64; m <= 1024.  One launch on one thread-block cluster up
 // to 288 rows, in blocks with batched products between them above.  A
@@ -36,10 +28,6 @@ struct PotrfBatch {
     PotrfJob job[kMaxGroup];
 };
 void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs);
-
-// B <- L^-1 B for every right-hand side matrix (L lower triangular m x m).
-void trsm_left_lower(tlr_ctx *ctx, cudaStream_t s, const double *L, int ldl, int m,
-                     const std::vector<RhsDesc> &rhs);
 
 // acc[0] += sum_r log A[r, r] (skipped once the status word holds an error);
 // maxinv (optional): running maximum of 1 / A[r, r]^2.

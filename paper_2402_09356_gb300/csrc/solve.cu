@@ -1,0 +1,386 @@
+// a5 on a kept factor: y = L^-1 z with the log-determinant and |y|^2 (Eq. 1.2),
+// and z = L w.
+//
+// The factor is read once; its bytes are the floor (0.2 GB at n = 20,000: 30 us),
+// and the FP64 pipe, one multiply-add per entry, is close behind (40 us).  What
+// costs is the chain of the solve: tile column by tile column, and inside a
+// diagonal tile block by block.  Per tile column three launches:
+//   k_trsv      y_k <- L_kk^-1 y_k, one cluster, blocks of 32 rows whose
+//               inverses were formed for all tiles by one launch at the start
+//               (k_inv_blocks: a block's substitution is then one 32 x 32
+//               product, not 32 dependent steps);
+//   k_pair_dots c_ik = V_ik' y_k for all i > k, one warp a column of V;
+//   k_pair_sub  y_i -= U_ik c_ik for all i > k.
+// The product L w has no chain: one launch of k_pair_dots over all tiles, one
+// of k_row_sums.  All descriptors go up once per call.
+#include <algorithm>
+#include <mutex>
+
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+#include "dense.cuh"
+#include "tlr_internal.cuh"
+
+namespace tlr {
+
+namespace cg = cooperative_groups;
+
+namespace {
+
+constexpr int kB = 32;             // rows of a diagonal block
+constexpr int kThreads = 256, kWarps = kThreads / 32;
+constexpr int kRows = 64;          // output rows a CTA
+constexpr int kGroups = kThreads / kRows;
+
+// One off-diagonal tile: U (m_i x r), V (m_k x r), both ld nb, and the place
+// of its c = V' x among all of them.
+struct Pair {
+    const double *U, *V;
+    int64_t off;
+    int i, k, r, pad;
+};
+
+__device__ __forceinline__ int rows_of(int64_t n, int nb, int t) {
+    const int64_t r = n - (int64_t)t * nb;
+    return (int)(r < nb ? r : nb);
+}
+
+// Inverses of the 32 x 32 diagonal blocks (row major, zero right of the
+// diagonal and past the tile) of every diagonal tile: one CTA a block.
+// Column by column, M <- the elimination applied to the identity: row c is
+// scaled by 1 / L_cc, the rows below it subtract their multiple.
+__global__ void __launch_bounds__(kThreads) k_inv_blocks(const double *__restrict__ D, int64_t n, int nb, int per_tile,
+                                                          double *__restrict__ inv) {
+    __shared__ double L[kB][kB + 1], M[kB][kB + 1], rd[kB];
+    const int t = blockIdx.x / per_tile, b = blockIdx.x % per_tile, tid = threadIdx.x;
+    const int m = rows_of(n, nb, t), p = b * kB, w = min(kB, m - p);
+    double *out = inv + (int64_t)blockIdx.x * kB * kB;
+    if (w <= 0) return;
+    const double *A = D + (int64_t)t * nb * nb + (int64_t)p * nb + p;
+    for (int e = tid; e < kB * kB; e += kThreads) {
+        const int r = e % kB, c = e / kB;
+        L[r][c] = r < w && c <= r ? A[(int64_t)c * nb + r] : 0.0;
+        M[r][c] = r == c ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    if (tid < w) rd[tid] = 1.0 / L[tid][tid];
+    __syncthreads();
+    const int r = tid >> 3, q = tid & 7;
+    for (int c = 0; c < w; ++c) {
+        if (tid <= c) M[c][tid] *= rd[c];
+        __syncthreads();
+        if (r > c && r < w) {
+            const double l = L[r][c];
+#pragma unroll
+            for (int k = 0; k < kB / 8; ++k)
+                if (q + 8 * k <= c) M[r][q + 8 * k] = fma(-l, M[c][q + 8 * k], M[r][q + 8 * k]);
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < kB * kB; e += kThreads) {
+        const int i = e / kB, c = e % kB;
+        out[e] = i < w && c <= i ? M[i][c] : 0.0;
+    }
+}
+
+// x <- L^-1 x for one diagonal tile (m <= 1024, ld ldl) by one cluster: CTA
+// `rank` owns the blocks rank, rank + kCl, ... of the right-hand side.  Step b:
+// the owner multiplies its block by the block's inverse and stores the 32
+// values into every CTA; after one cluster barrier every CTA subtracts L's
+// block column b times them from its blocks.  Eight threads a row; the entries
+// of the next block column are loaded before the barrier.  Bound by the chain
+// of a step (barrier, update, product: about 1 us).
+template <int kCl>
+__global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L, int ldl, int m,
+                                                    const double *__restrict__ inv, double *__restrict__ x) {
+    constexpr int kOwn = kB / kCl;  // blocks a CTA: at most 32 blocks in a tile
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, r = tid >> 3, q = tid & 7;
+    __shared__ double rhs[kOwn][kB], xs[2][kB];
+    const int nblk = (m + kB - 1) / kB;
+#pragma unroll
+    for (int o = 0; o < kOwn; ++o) {
+        const int i = (rank + o * kCl) * kB + tid;
+        if (tid < kB) rhs[o][tid] = i < m ? x[i] : 0.0;
+    }
+    double a[kOwn][kB / 8], d[kB / 8];
+    auto load = [&](int b) {  // L's block column b in the rows of the own blocks
+#pragma unroll
+        for (int o = 0; o < kOwn; ++o) {
+            const int I = rank + o * kCl, row = I * kB + r;
+#pragma unroll
+            for (int k = 0; k < kB / 8; ++k) {
+                const int c = b * kB + q + 8 * k;
+                a[o][k] = I > b && row < m && c < m ? L[(int64_t)c * ldl + row] : 0.0;
+            }
+        }
+    };
+    auto load_inv = [&](int b) {  // the inverse of the own block that comes next
+        if (b < nblk)
+#pragma unroll
+            for (int k = 0; k < kB / 8; ++k) d[k] = inv[(int64_t)b * kB * kB + r * kB + q + 8 * k];
+    };
+    auto reduce8 = [](double v) {
+        v += __shfl_xor_sync(0xFFFFFFFFu, v, 4);
+        v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+        v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+        return v;
+    };
+    load_inv(rank);
+    load(0);
+    cl.sync();  // every CTA has started (its shared memory is written below)
+    for (int b = 0; b < nblk; ++b) {
+        if (b % kCl == rank) {
+            const double *v = rhs[b / kCl];
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < kB / 8; ++k) s = fma(d[k], v[q + 8 * k], s);
+            s = reduce8(s);
+#pragma unroll
+            for (int k = q; k < kCl; k += 8) cl.map_shared_rank(&xs[b & 1][0], k)[r] = s;
+            if (q == 0 && b * kB + r < m) x[b * kB + r] = s;
+            load_inv(b + kCl);
+        }
+        cl.sync();
+        const double *v = xs[b & 1];
+#pragma unroll
+        for (int o = 0; o < kOwn; ++o) {
+            if (rank + o * kCl <= b) continue;  // uniform over the CTA
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < kB / 8; ++k) s = fma(a[o][k], v[q + 8 * k], s);
+            s = reduce8(s);
+            if (q == 0) rhs[o][r] -= s;
+        }
+        if (b + 1 < nblk) load(b + 1);
+        __syncthreads();
+    }
+}
+
+// c = V' x of the pairs p0 + blockIdx.y: eight columns a CTA, one a warp.
+__global__ void __launch_bounds__(kThreads) k_pair_dots(const Pair *__restrict__ pairs, int p0, int64_t n, int nb,
+                                                         const double *__restrict__ x, double *__restrict__ c) {
+    const Pair P = pairs[p0 + blockIdx.y];
+    const int lane = threadIdx.x & 31, col = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    if (col >= P.r) return;
+    const double *v = P.V + (int64_t)col * nb, *y = x + (int64_t)P.k * nb;
+    const int m = rows_of(n, nb, P.k);
+    double s0 = 0.0, s1 = 0.0;
+    int i = lane;
+#pragma unroll 4
+    for (; i + 32 < m; i += 64) {
+        s0 = fma(v[i], y[i], s0);
+        s1 = fma(v[i + 32], y[i + 32], s1);
+    }
+    if (i < m) s0 = fma(v[i], y[i], s0);
+    s0 += s1;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s0 += __shfl_xor_sync(0xFFFFFFFFu, s0, o);
+    if (lane == 0) c[P.off + col] = s0;
+}
+
+// Row `row` of A (m x k, ld lda) times v, columns g, g + kGroups, ...
+__device__ __forceinline__ double row_part(const double *__restrict__ A, int lda, int k, int g,
+                                           const double *__restrict__ v) {
+    double s0 = 0.0, s1 = 0.0;
+    int j = g;
+#pragma unroll 4
+    for (; j + kGroups < k; j += 2 * kGroups) {
+        s0 = fma(A[(int64_t)j * lda], v[j], s0);
+        s1 = fma(A[(int64_t)(j + kGroups) * lda], v[j + kGroups], s1);
+    }
+    if (j < k) s0 = fma(A[(int64_t)j * lda], v[j], s0);
+    return s0 + s1;
+}
+
+// y_i -= U_ik c_ik for the pairs p0 + blockIdx.y: 64 rows a CTA, the columns
+// split over four threads a row.
+__global__ void __launch_bounds__(kThreads) k_pair_sub(const Pair *__restrict__ pairs, int p0, int64_t n, int nb,
+                                                        const double *__restrict__ c, double *__restrict__ y) {
+    __shared__ double part[kGroups][kRows];
+    const Pair P = pairs[p0 + blockIdx.y];
+    const int g = threadIdx.x / kRows, u = threadIdx.x % kRows, row = blockIdx.x * kRows + u;
+    const int m = rows_of(n, nb, P.i);
+    part[g][u] = row < m ? row_part(P.U + row, nb, P.r, g, c + P.off) : 0.0;
+    __syncthreads();
+    if (g == 0 && row < m) y[(int64_t)P.i * nb + row] -= (part[0][u] + part[1][u]) + (part[2][u] + part[3][u]);
+}
+
+// z_i = D_i w_i + sum_k U_ik c_ik: blockIdx.y = i, 64 rows a CTA; the pairs of
+// row i are first[i] .. first[i + 1].  D's columns past the row are zero and
+// left out.
+__global__ void __launch_bounds__(kThreads) k_row_sums(const Pair *__restrict__ pairs, const int *__restrict__ first,
+                                                        int64_t n, int nb, const double *__restrict__ D,
+                                                        const double *__restrict__ w, const double *__restrict__ c,
+                                                        double *__restrict__ z) {
+    __shared__ double part[kGroups][kRows];
+    const int i = blockIdx.y, g = threadIdx.x / kRows, u = threadIdx.x % kRows, row = blockIdx.x * kRows + u;
+    const int m = rows_of(n, nb, i);
+    double s = 0.0;
+    if (row < m) {
+        s = row_part(D + (int64_t)i * nb * nb + row, nb, row + 1, g, w + (int64_t)i * nb);
+        for (int p = first[i]; p < first[i + 1]; ++p) {
+            const Pair P = pairs[p];
+            s += row_part(P.U + row, nb, P.r, g, c + P.off);
+        }
+    }
+    part[g][u] = s;
+    __syncthreads();
+    if (g == 0 && row < m) z[(int64_t)i * nb + row] = (part[0][u] + part[1][u]) + (part[2][u] + part[3][u]);
+}
+
+// Per tile: sum log D_rr and |y|^2 (fixed reduction order), then their sums
+// over the tiles in order, added to acc.
+__global__ void __launch_bounds__(kThreads) k_tile_sums(const double *__restrict__ D, int64_t n, int nb,
+                                                         const double *__restrict__ y, double *__restrict__ part) {
+    __shared__ double sl[kThreads], sq[kThreads];
+    const int t = blockIdx.x, tid = threadIdx.x, m = rows_of(n, nb, t);
+    double l = 0.0, s = 0.0;
+    for (int r = tid; r < m; r += kThreads) {
+        l += log(D[(int64_t)t * nb * nb + (int64_t)r * nb + r]);
+        const double v = y[(int64_t)t * nb + r];
+        s += v * v;
+    }
+    sl[tid] = l;
+    sq[tid] = s;
+    __syncthreads();
+    for (int h = kThreads / 2; h > 0; h >>= 1) {
+        if (tid < h) {
+            sl[tid] += sl[tid + h];
+            sq[tid] += sq[tid + h];
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        part[2 * t] = sl[0];
+        part[2 * t + 1] = sq[0];
+    }
+}
+__global__ void k_sum_tiles(const double *__restrict__ part, int nt, double *__restrict__ acc) {
+    double s = acc[threadIdx.x];
+    for (int t = 0; t < nt; ++t) s += part[2 * t + threadIdx.x];
+    acc[threadIdx.x] = s;
+}
+
+// The tiles of nonzero rank, by column (by_row: by row), with the places of
+// their c = V' x and the first pair of every column (row).
+struct PairList {
+    std::vector<Pair> pairs;
+    std::vector<int> first, rmax;
+    int64_t total = 0;
+};
+PairList list_pairs(const tlr_mat *M, bool by_row) {
+    const int nt = M->nt;
+    PairList L;
+    for (int a = 0; a < nt; ++a) {
+        L.first.push_back((int)L.pairs.size());
+        int most = 0;
+        for (int b = by_row ? 0 : a + 1; b < (by_row ? a : nt); ++b) {
+            const int i = by_row ? a : b, k = by_row ? b : a, r = M->h_ranks[(size_t)i * nt + k];
+            if (r <= 0) continue;
+            const int64_t at = slot_col(M, i, k) * M->nb;
+            L.pairs.push_back(Pair{M->U + at, M->V + at, L.total, i, k, r, 0});
+            L.total += r;
+            most = std::max(most, r);
+        }
+        L.rmax.push_back(most);
+    }
+    L.first.push_back((int)L.pairs.size());
+    return L;
+}
+
+// Host data on the device for the kernels of stream s: through the pinned ring
+// where it is small, else its own buffer.
+const void *upload(tlr_ctx *ctx, cudaStream_t s, const void *data, size_t bytes, DevBuf &own) {
+    if (bytes <= ((size_t)1 << 20)) return stage_push(ctx, data, bytes, s);
+    own.alloc(bytes, s);
+    TLR_CUDA_TRY(cudaMemcpyAsync(own.as<char>(), data, bytes, cudaMemcpyHostToDevice, s));
+    TLR_CUDA_TRY(cudaStreamSynchronize(s));
+    return own.as<char>();
+}
+
+bool trsv16_ok() {
+    static std::once_flag once;
+    static bool ok = false;
+    std::call_once(once, [] {
+        if (cudaFuncSetAttribute(k_trsv<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(16);
+            cfg.blockDim = dim3(kThreads);
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 16;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int nc = 0;
+            ok = cudaOccupancyMaxActiveClusters(&nc, k_trsv<16>, &cfg) == cudaSuccess && nc > 0;
+        }
+        cudaGetLastError();  // clear any error of the queries
+    });
+    return ok;
+}
+
+// Pairs a launch's grid may hold in its second dimension.
+constexpr int kMaxGridY = 65535;
+
+}  // namespace
+
+// y = L^-1 z tile by tile; acc[0] += sum log L_ii, acc[1] += |y|^2.
+void forward_solve(tlr_ctx *ctx, cudaStream_t st, const tlr_mat *M, const double *z, double *y, double *acc) {
+    const int nt = M->nt, nb = M->nb, per_tile = (int)ceil_div(nb, kB);
+    const int64_t n = M->n;
+    if (y != z) TLR_CUDA_TRY(cudaMemcpyAsync(y, z, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    const PairList L = list_pairs(M, false);
+    DevBuf own;
+    const Pair *pairs = L.pairs.empty()
+                            ? nullptr
+                            : (const Pair *)upload(ctx, st, L.pairs.data(), L.pairs.size() * sizeof(Pair), own);
+    DevBuf inv((size_t)nt * per_tile * kB * kB * sizeof(double), st);
+    DevBuf cb((size_t)std::max<int64_t>(L.total, 1) * sizeof(double), st), part((size_t)2 * nt * sizeof(double), st);
+    double *c = cb.as<double>();
+    launch(k_inv_blocks, (unsigned)(nt * per_tile), kThreads, 0, st, M->D, n, nb, per_tile, inv.as<double>());
+    TLR_CHECK_LAUNCH();
+    const bool big = trsv16_ok();
+    for (int k = 0; k < nt; ++k) {
+        const double *D = M->D + (int64_t)k * nb * nb, *Di = inv.as<double>() + (int64_t)k * per_tile * kB * kB;
+        if (big) launch_clustered(k_trsv<16>, 16, 1, kThreads, 0, st, D, nb, tile_rows(n, nb, k), Di, y + (int64_t)k * nb);
+        else launch_clustered(k_trsv<8>, 8, 1, kThreads, 0, st, D, nb, tile_rows(n, nb, k), Di, y + (int64_t)k * nb);
+        const int p1 = L.first[(size_t)k + 1];
+        for (int p = L.first[(size_t)k]; p < p1; p += kMaxGridY) {
+            const unsigned cnt = (unsigned)std::min(kMaxGridY, p1 - p);
+            launch(k_pair_dots, dim3((unsigned)ceil_div(L.rmax[(size_t)k], kWarps), cnt), kThreads, 0, st, pairs, p, n,
+                   nb, y, c);
+            launch(k_pair_sub, dim3((unsigned)ceil_div(nb, kRows), cnt), kThreads, 0, st, pairs, p, n, nb, c, y);
+        }
+        TLR_CHECK_LAUNCH();
+    }
+    launch(k_tile_sums, (unsigned)nt, kThreads, 0, st, M->D, n, nb, y, part.as<double>());
+    launch(k_sum_tiles, 1, 2, 0, st, part.as<double>(), nt, acc);
+    TLR_CHECK_LAUNCH();
+}
+
+// z = L w
+void lmul(tlr_ctx *ctx, cudaStream_t st, const tlr_mat *M, const double *w, double *z) {
+    const int nt = M->nt, nb = M->nb;
+    const int64_t n = M->n;
+    const PairList L = list_pairs(M, true);
+    DevBuf own, ownf;
+    const Pair *pairs = L.pairs.empty()
+                            ? nullptr
+                            : (const Pair *)upload(ctx, st, L.pairs.data(), L.pairs.size() * sizeof(Pair), own);
+    const int *first = (const int *)upload(ctx, st, L.first.data(), L.first.size() * sizeof(int), ownf);
+    DevBuf cb((size_t)std::max<int64_t>(L.total, 1) * sizeof(double), st);
+    double *c = cb.as<double>();
+    const int rmax = *std::max_element(L.rmax.begin(), L.rmax.end());
+    for (int p = 0; p < (int)L.pairs.size(); p += kMaxGridY)
+        launch(k_pair_dots, dim3((unsigned)ceil_div(rmax, kWarps), (unsigned)std::min(kMaxGridY, (int)L.pairs.size() - p)),
+               kThreads, 0, st, pairs, p, n, nb, w, c);
+    launch(k_row_sums, dim3((unsigned)ceil_div(nb, kRows), (unsigned)nt), kThreads, 0, st, pairs, first, n, nb, M->D, w,
+           c, z);
+    TLR_CHECK_LAUNCH();
+}
+
+}  // namespace tlr

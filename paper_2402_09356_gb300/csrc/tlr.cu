@@ -860,108 +860,6 @@ void factor(tlr_ctx *ctx, cudaStream_t st, tlr_mat *M, FactorMode mode, const do
     if (F.err != TLR_OK) throw Error{F.err, F.msg};
 }
 
-// y = L^-1 z tile by tile; acc[0] += sum log L_ii, acc[1] += |y|^2.
-void forward_solve(tlr_ctx *ctx, cudaStream_t st, const tlr_mat *M, const double *z, double *y,
-                   double *acc) {
-    const int nt = M->nt, nb = M->nb;
-    const int64_t n = M->n;
-    auto r_of = [&](int i, int k) { return (int)M->h_ranks[(size_t)i * nt + k]; };
-    if (y != z) TLR_CUDA_TRY(cudaMemcpyAsync(y, z, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    int maxR = 0;
-    for (int j = 0; j < nt; ++j) {
-        int Rj = 0;
-        for (int k = 0; k < j; ++k) Rj += r_of(j, k);
-        maxR = std::max(maxR, Rj);
-    }
-    DevBuf cbuf((size_t)std::max(maxR, 1) * sizeof(double), st);
-    double *c = cbuf.as<double>();
-    for (int j = 0; j < nt; ++j) {
-        const int mj = tile_rows(n, nb, j);
-        double *yj = y + (int64_t)j * nb;
-        std::vector<GemmProb> gc, gu;
-        int o = 0;
-        for (int k = 0; k < j; ++k) {
-            int r = r_of(j, k);
-            if (r <= 0) continue;
-            GemmProb a{};  // c_k = V_jk' y_k
-            a.A = Vslot(M, j, k); a.lda = nb; a.m = r; a.k = tile_rows(n, nb, k);
-            a.B = y + (int64_t)k * nb; a.ldb = nb; a.n = 1;
-            a.C = c + o; a.ldc = r;
-            gc.push_back(a);
-            o += r;
-        }
-        if (o > 0) {
-            gemm_batched(ctx, st, true, false, gc, 1.0, 0.0);
-            // y_j -= [U_j0 ...] c, accumulated one k at a time (distinct outputs per launch)
-            o = 0;
-            for (int k = 0; k < j; ++k) {
-                int r = r_of(j, k);
-                if (r <= 0) continue;
-                GemmProb b{};
-                b.A = Uslot(M, j, k); b.lda = nb; b.m = mj; b.k = r;
-                b.B = c + o; b.ldb = r; b.n = 1;
-                b.C = yj; b.ldc = nb;
-                gemm_batched(ctx, st, false, false, std::vector<GemmProb>{b}, -1.0, 1.0);
-                o += r;
-            }
-        }
-        const double *Dj = M->D + (int64_t)j * nb * nb;
-        trsm_left_lower(ctx, st, Dj, nb, mj, {RhsDesc{yj, 1, nb}});
-        diag_logsum(st, Dj, nb, mj, acc, ctx->d_status);
-        sumsq(st, yj, mj, acc + 1);
-    }
-}
-
-// z = L w
-void lmul(tlr_ctx *ctx, cudaStream_t st, const tlr_mat *M, const double *w, double *z) {
-    const int nt = M->nt, nb = M->nb;
-    const int64_t n = M->n;
-    auto r_of = [&](int i, int k) { return (int)M->h_ranks[(size_t)i * nt + k]; };
-    std::vector<GemmProb> gd;
-    for (int i = 0; i < nt; ++i) {
-        GemmProb a{};
-        a.A = M->D + (int64_t)i * nb * nb; a.lda = nb; a.m = tile_rows(n, nb, i); a.k = a.m;
-        a.B = w + (int64_t)i * nb; a.ldb = nb; a.n = 1;
-        a.C = z + (int64_t)i * nb; a.ldc = nb;
-        gd.push_back(a);
-    }
-    gemm_batched(ctx, st, false, false, gd, 1.0, 0.0);
-    // c_ik = V_ik' w_k for all i > k
-    int64_t tot = 0;
-    std::vector<int64_t> co((size_t)nt * nt, -1);
-    for (int i = 0; i < nt; ++i)
-        for (int k = 0; k < i; ++k)
-            if (r_of(i, k) > 0) { co[(size_t)i * nt + k] = tot; tot += r_of(i, k); }
-    if (tot == 0) return;
-    DevBuf cbuf((size_t)tot * sizeof(double), st);
-    double *c = cbuf.as<double>();
-    std::vector<GemmProb> gc;
-    for (int i = 0; i < nt; ++i)
-        for (int k = 0; k < i; ++k) {
-            int r = r_of(i, k);
-            if (r <= 0) continue;
-            GemmProb a{};
-            a.A = Vslot(M, i, k); a.lda = nb; a.m = r; a.k = tile_rows(n, nb, k);
-            a.B = w + (int64_t)k * nb; a.ldb = nb; a.n = 1;
-            a.C = c + co[(size_t)i * nt + k]; a.ldc = r;
-            gc.push_back(a);
-        }
-    gemm_batched(ctx, st, true, false, gc, 1.0, 0.0);
-    for (int k = 0; k < nt; ++k) {
-        std::vector<GemmProb> gu;
-        for (int i = k + 1; i < nt; ++i) {
-            int r = r_of(i, k);
-            if (r <= 0) continue;
-            GemmProb b{};
-            b.A = Uslot(M, i, k); b.lda = nb; b.m = tile_rows(n, nb, i); b.k = r;
-            b.B = c + co[(size_t)i * nt + k]; b.ldb = r; b.n = 1;
-            b.C = z + (int64_t)i * nb; b.ldc = nb;
-            gu.push_back(b);
-        }
-        gemm_batched(ctx, st, false, false, gu, 1.0, 1.0);
-    }
-}
-
 int64_t plan_slots(tlr_mat *M, const std::vector<int32_t> &hint) {
     const int nt = M->nt;
     const int64_t noff = (int64_t)nt * (nt - 1) / 2;

@@ -281,15 +281,16 @@ int tlr_order(tlr_ctx *ctx, const double *xy, int64_t n, int method, uint64_t se
         check_arg((flags & ~TLR_ORDER_QUANTIZE) == 0, "flags");
         check_arg(n == 0 || (xy && perm), "xy/perm");
         if (n == 0) return;
+        const int quantize = (flags & TLR_ORDER_QUANTIZE) ? 1 : 0;
         switch (method) {
         case TLR_ORDER_IDENTITY: order_identity(n, perm, s); break;
         case TLR_ORDER_RANDOM:
         case TLR_ORDER_MORTON:
-        case TLR_ORDER_HILBERT: order_sfc(xy, n, method, seed, perm, codes, s); break;
+        case TLR_ORDER_HILBERT: order_sfc(xy, n, method, seed, perm, codes, xy_out, quantize, s); return;
         case TLR_ORDER_KDTREE: order_kdtree(xy, n, perm, s); break;
         case TLR_ORDER_MAXMIN: order_maxmin(xy, n, perm, s, ctx->num_sms); break;
         }
-        if (xy_out) permute_xy(xy, perm, n, (flags & TLR_ORDER_QUANTIZE) ? 1 : 0, xy_out, s);
+        if (xy_out) permute_xy(xy, perm, n, quantize, xy_out, s);
     });
 }
 
@@ -849,7 +850,7 @@ int tlr_loglik_host(tlr_ctx *ctx, const double *xy_host, const double *z_host, i
         case TLR_ORDER_IDENTITY: order_identity(n, p, s); break;
         case TLR_ORDER_RANDOM:
         case TLR_ORDER_MORTON:
-        case TLR_ORDER_HILBERT: order_sfc(x, n, order, seed, p, nullptr, s); break;
+        case TLR_ORDER_HILBERT: order_sfc(x, n, order, seed, p, nullptr, nullptr, 0, s); break;
         case TLR_ORDER_KDTREE: order_kdtree(x, n, p, s); break;
         case TLR_ORDER_MAXMIN: order_maxmin(x, n, p, s, ctx->num_sms); break;
         }

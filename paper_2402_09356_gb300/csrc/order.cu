@@ -18,11 +18,17 @@
 // publishes its (max, lowest index) partial; the next launch reduces the
 // partials (double-buffered) to find the next point.  All distance arithmetic
 // uses explicitly rounded intrinsics so that no multiply-add is contracted.
+#include <algorithm>
 #include <mutex>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+#include "tlr_internal.cuh"
 
 namespace tlr {
+
+namespace cg = cooperative_groups;
 
 static constexpr int kSortThreads = 256;
 static constexpr int kSortItems = 16;  // keys per thread per block
@@ -420,11 +426,612 @@ __global__ void k_fill(double *__restrict__ a, int64_t n, double v) {
     if (i < n) a[i] = v;
 }
 
+// ------------------------------------------------- orderings on one cluster
+//
+// For the sizes of the workloads (up to kClusterMaxN locations) an ordering is
+// a few kernels on one thread-block cluster instead of a launch per radix pass,
+// tree level or selected point: its bytes take a microsecond, so that launches,
+// their gaps and host synchronisations were all of the time.  Arrays stay in
+// L2 (__ldcg / __stcg: another CTA wrote them in an earlier phase); a cluster
+// barrier separates the phases.  40,000 locations with xy_out: Hilbert 123 -> 60
+// us, KD-tree 2,940 -> 180 us (sort 83, upper levels 71, subtrees 29); 10,000
+// locations by max-min 82 -> 15 ms.  Above kClusterMaxN the launches above take over (more
+// SMs share a pass).
+constexpr int kOrdCl = 16, kOrdThreads = 1024, kOrdWarps = kOrdThreads / 32;
+constexpr int64_t kClusterMaxN = (int64_t)1 << 18;
+constexpr int kSortBatch = 4;  // keys a lane loads before it counts them
+
+struct SortShared {
+    uint32_t cnt[kOrdWarps][256];
+    uint32_t hist[256], base[256], part[8];
+    int skip;
+};
+
+// Stable sort of (key, val) by the low `bits` bits of the key, by one cluster:
+// warp w of the cluster takes a run of items, counts its digits (one count per
+// warp and digit, leaders of equal digits found by match), the counts are
+// summed over warps, CTAs (over DSMEM) and digits, and the warp writes its
+// items in order.  A pass in which all keys share the digit is left out.  The
+// result ends in (keys, vals).
+template <typename K>
+__device__ void cluster_sort(cg::cluster_group &cl, SortShared &S, K *&keys, uint32_t *&vals, K *&ktmp, uint32_t *&vtmp,
+                             int n, int bits) {
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int run = (n + kOrdCl * kOrdWarps * 32 - 1) / (kOrdCl * kOrdWarps * 32);  // rounds of 32 items a warp
+    const int i0 = (rank * kOrdWarps + warp) * run * 32;
+    const uint32_t below = (1u << lane) - 1u;
+    for (int shift = 0; shift < bits; shift += 8) {
+        for (int e = tid; e < kOrdWarps * 256; e += kOrdThreads) S.cnt[e >> 8][e & 255] = 0;
+        __syncthreads();
+        for (int u0 = 0; u0 < run; u0 += kSortBatch) {
+            K k[kSortBatch];
+#pragma unroll
+            for (int u = 0; u < kSortBatch; ++u) {
+                const int i = i0 + (u0 + u) * 32 + lane;
+                k[u] = u0 + u < run && i < n ? __ldcg(keys + i) : K(0);
+            }
+#pragma unroll
+            for (int u = 0; u < kSortBatch; ++u) {
+                const int i = i0 + (u0 + u) * 32 + lane;
+                const bool in = u0 + u < run && i < n;
+                const uint32_t d = in ? (uint32_t)(k[u] >> shift) & 255u : 256u;
+                const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+                if (in && !(peers & below)) S.cnt[warp][d] += __popc(peers);
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        if (tid < 256) {
+            uint32_t t = 0;
+#pragma unroll 8
+            for (int w = 0; w < kOrdWarps; ++w) {
+                const uint32_t c = S.cnt[w][tid];
+                S.cnt[w][tid] = t;
+                t += c;
+            }
+            S.hist[tid] = t;
+        }
+        if (tid == 0) S.skip = 0;
+        cl.sync();
+        if (tid < 256) {
+            uint32_t tot = 0, before = 0, h[kOrdCl];
+#pragma unroll
+            for (int q = 0; q < kOrdCl; ++q) h[q] = cl.map_shared_rank(&S.hist[0], q)[tid];
+#pragma unroll
+            for (int q = 0; q < kOrdCl; ++q) {
+                before += q < rank ? h[q] : 0u;
+                tot += h[q];
+            }
+            if (tot == (uint32_t)n) S.skip = 1;
+            uint32_t inc = tot;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                if (lane >= o) inc += v;
+            }
+            if (lane == 31) S.part[warp] = inc;
+            S.base[tid] = inc - tot + before;
+        }
+        __syncthreads();
+        if (tid < 256) {
+            uint32_t s = 0;
+            for (int w = 0; w < warp; ++w) s += S.part[w];
+            S.base[tid] += s;
+        }
+        __syncthreads();
+        if (S.skip) {  // the same on every CTA
+            cl.sync();  // every CTA has read the histograms
+            continue;
+        }
+        for (int u0 = 0; u0 < run; u0 += kSortBatch) {
+            K k[kSortBatch];
+            uint32_t v[kSortBatch];
+#pragma unroll
+            for (int u = 0; u < kSortBatch; ++u) {
+                const int i = i0 + (u0 + u) * 32 + lane;
+                const bool in = u0 + u < run && i < n;
+                k[u] = in ? __ldcg(keys + i) : K(0);
+                v[u] = in ? __ldcg(vals + i) : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < kSortBatch; ++u) {
+                const int i = i0 + (u0 + u) * 32 + lane;
+                const bool in = u0 + u < run && i < n;
+                const uint32_t d = in ? (uint32_t)(k[u] >> shift) & 255u : 256u;
+                const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+                if (in) {
+                    const uint32_t pos = S.base[d] + S.cnt[warp][d] + __popc(peers & below);
+                    __stcg(ktmp + pos, k[u]);
+                    __stcg(vtmp + pos, v[u]);
+                }
+                __syncwarp();
+                if (in && !(peers & below)) S.cnt[warp][d] += __popc(peers);
+                __syncwarp();
+            }
+        }
+        cl.sync();
+        K *kk = keys;
+        keys = ktmp;
+        ktmp = kk;
+        uint32_t *vv = vals;
+        vals = vtmp;
+        vtmp = vv;
+    }
+}
+
+// Random / Morton / Hilbert ordering in one launch: keys, sort, permutation and
+// the permuted locations.
+__global__ void __launch_bounds__(kOrdThreads) k_sfc_cluster(const double *__restrict__ xy, int n, int method, uint64_t seed,
+                                                              uint32_t *keys, uint32_t *vals, uint32_t *ktmp,
+                                                              uint32_t *vtmp, uint32_t *__restrict__ codes,
+                                                              int64_t *__restrict__ perm, double *__restrict__ xy_out,
+                                                              int quantize) {
+    __shared__ SortShared S;
+    cg::cluster_group cl = cg::this_cluster();
+    const int t0 = (int)cl.block_rank() * kOrdThreads + threadIdx.x;
+    for (int i = t0; i < n; i += kOrdCl * kOrdThreads) {
+        uint32_t k;
+        if (method == TLR_ORDER_RANDOM) {
+            k = (uint32_t)(splitmix64(seed ^ (uint64_t)i) >> 32);
+        } else {
+            const uint32_t qx = quantize16(xy[i]), qy = quantize16(xy[n + i]);
+            k = (method == TLR_ORDER_MORTON) ? (spread_bits(qx) | (spread_bits(qy) << 1)) : hilbert16(qx, qy);
+        }
+        __stcg(keys + i, k);
+        __stcg(vals + i, (uint32_t)i);
+        if (codes) codes[i] = k;
+    }
+    cl.sync();
+    cluster_sort<uint32_t>(cl, S, keys, vals, ktmp, vtmp, n, 32);
+    for (int p = t0; p < n; p += kOrdCl * kOrdThreads) {
+        const uint32_t i = __ldcg(vals + p);
+        perm[p] = (int64_t)i;
+        if (xy_out) {
+            double x = xy[i], y = xy[n + i];
+            if (quantize) {
+                x = __ddiv_rn((double)quantize16(x), 65535.0);
+                y = __ddiv_rn((double)quantize16(y), 65535.0);
+            }
+            xy_out[p] = x;
+            xy_out[n + p] = y;
+        }
+    }
+    cl.sync();  // no CTA leaves while another may still read its histogram
+}
+
+// KD-tree, part 1: the locations sorted by (x, index) and by (y, index), one
+// cluster each.  list[dim] receives the order.
+__global__ void __launch_bounds__(kOrdThreads) k_kd_sort(const double *__restrict__ xy, int n, uint64_t *keys, uint64_t *ktmp,
+                                                          uint32_t *vals, uint32_t *vtmp, uint32_t *__restrict__ list) {
+    __shared__ SortShared S;
+    cg::cluster_group cl = cg::this_cluster();
+    const int dim = blockIdx.x / kOrdCl, t0 = (int)cl.block_rank() * kOrdThreads + threadIdx.x;
+    keys += (int64_t)dim * n;
+    ktmp += (int64_t)dim * n;
+    vals += (int64_t)dim * n;
+    vtmp += (int64_t)dim * n;
+    for (int i = t0; i < n; i += kOrdCl * kOrdThreads) {
+        __stcg(keys + i, (uint64_t)dkey(xy[(int64_t)dim * n + i]));
+        __stcg(vals + i, (uint32_t)i);
+    }
+    cl.sync();
+    cluster_sort<uint64_t>(cl, S, keys, vals, ktmp, vtmp, n, 64);
+    for (int p = t0; p < n; p += kOrdCl * kOrdThreads) list[(int64_t)dim * n + p] = __ldcg(vals + p);
+    cl.sync();  // no CTA leaves while another may still read its histogram
+}
+
+// Whether a node splits along x: its range of x is at least that of y.  The
+// node's points are at positions [a, a + m) of both lists, sorted in each.
+__device__ __forceinline__ bool kd_split_x(double x0, double x1, double y0, double y1) {
+    return __dsub_rn(x1, x0) >= __dsub_rn(y1, y0);
+}
+
+// KD-tree, part 2: the upper levels, by one cluster.  A level needs no sort:
+// both lists stay sorted inside every node, the node's first ceil(m / 2) points
+// along the chosen dimension go left, and the other list is partitioned
+// stably by that side.  A level: (1) the dimension of every node from the ends
+// of its two runs; (2) every point's side, from the list of that dimension; (3)
+// the lefts before each position, counted over warps, CTAs and the cluster; (4)
+// the new positions.  Node starts and the lefts before them follow from n
+// alone: a level's nodes hold q = n >> level or q + 1 points.
+constexpr int kKdLocal = 2048;  // nodes up to this size are finished by one CTA each
+constexpr int kKdTopNodes = 256;
+__global__ void __launch_bounds__(kOrdThreads) k_kd_top(const double *__restrict__ xy, int n, uint32_t *list, uint32_t *ltmp,
+                                                         uint8_t *side, int levels) {
+    __shared__ uint8_t dim_x[kKdTopNodes];
+    __shared__ int wtot[2][kOrdWarps], total[2], before[2];
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int run = (n + kOrdCl * kOrdWarps * 32 - 1) / (kOrdCl * kOrdWarps * 32);
+    const int p0 = (rank * kOrdWarps + warp) * run * 32;
+    const uint32_t below = (1u << lane) - 1u;
+    // node of position p at a level: index s, start a, size m
+    auto node = [&](int p, int level, int &s, int &a, int &m) {
+        s = 0;
+        a = 0;
+        m = n;
+        for (int l = 0; l < level; ++l) {
+            const int h = (m + 1) / 2;
+            const bool right = p >= a + h;
+            s = 2 * s + right;
+            a += right ? h : 0;
+            m = right ? m - h : h;
+        }
+    };
+    for (int level = 0; level < levels; ++level) {
+        const uint32_t *X = list, *Y = list + n;
+        for (int s = tid; s < (1 << level); s += kOrdThreads) {
+            int a = 0, m = n;
+            for (int l = level - 1; l >= 0; --l) {
+                const int h = (m + 1) / 2;
+                const bool right = (s >> l) & 1;
+                a += right ? h : 0;
+                m = right ? m - h : h;
+            }
+            dim_x[s] = kd_split_x(xy[__ldcg(X + a)], xy[__ldcg(X + a + m - 1)], xy[n + __ldcg(Y + a)],
+                                  xy[n + __ldcg(Y + a + m - 1)]);
+        }
+        __syncthreads();
+        for (int u = 0; u < run; ++u) {
+            const int p = p0 + 32 * u + lane;
+            if (p >= n) break;
+            int s, a, m;
+            node(p, level, s, a, m);
+            const uint32_t i = __ldcg((dim_x[s] ? X : Y) + p);
+            __stcg(side + i, (uint8_t)(p - a < (m + 1) / 2));
+        }
+        cl.sync();
+        int cnt[2] = {0, 0};
+        for (int u = 0; u < run; ++u) {
+            const int p = p0 + 32 * u + lane;
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                const bool left = p < n && __ldcg(side + __ldcg(list + (int64_t)d * n + p));
+                cnt[d] += __popc(__ballot_sync(0xFFFFFFFFu, left));
+            }
+        }
+        if (lane == 0) {
+            wtot[0][warp] = cnt[0];
+            wtot[1][warp] = cnt[1];
+        }
+        __syncthreads();
+        if (warp < 2) {  // exclusive sums over the CTA's warps
+            const int v = wtot[warp][lane];
+            int inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            wtot[warp][lane] = inc - v;
+            if (lane == 31) total[warp] = inc;
+        }
+        cl.sync();
+        if (warp < 2) {
+            int v = lane < rank ? cl.map_shared_rank(&total[0], lane < kOrdCl ? lane : 0)[warp] : 0;
+            v = __reduce_add_sync(0xFFFFFFFFu, v);
+            if (lane == 0) before[warp] = v;
+        }
+        __syncthreads();
+        const int q = n >> level;
+        int f[2] = {before[0] + wtot[0][warp], before[1] + wtot[1][warp]};
+        for (int u = 0; u < run; ++u) {
+            const int p = p0 + 32 * u + lane;
+            int s = 0, a = 0, m = 0;
+            if (p < n) node(p, level, s, a, m);
+            const int h = (m + 1) / 2, big = a - s * q;  // nodes of q + 1 points before this one
+            const int fa = (s - big) * ((q + 1) / 2) + big * ((q + 2) / 2);
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                const uint32_t i = p < n ? __ldcg(list + (int64_t)d * n + p) : 0u;
+                const bool left = p < n && __ldcg(side + i);
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, left);
+                const int lf = f[d] + __popc(bal & below) - fa;  // lefts of the node before p
+                if (p < n) __stcg(ltmp + (int64_t)d * n + (left ? a + lf : a + h + (p - a) - lf), i);
+                f[d] += __popc(bal);
+            }
+        }
+        cl.sync();
+        uint32_t *t = list;
+        list = ltmp;
+        ltmp = t;
+    }
+    cl.sync();  // no CTA leaves while another may still read its totals
+}
+
+// KD-tree, part 3: one CTA finishes the subtree of one node (at most kKdLocal
+// points) in shared memory, two positions a thread, and writes its part of the
+// permutation.
+struct KdShared {
+    double x[kKdLocal], y[kKdLocal];
+    uint32_t id[kKdLocal];
+    uint16_t lx[2][kKdLocal], ly[2][kKdLocal];
+    int fx[kKdLocal + 1], fy[kKdLocal + 1];
+    uint8_t side[kKdLocal], dim_x[kKdLocal];
+    int wsum[2][kOrdWarps];
+};
+__global__ void __launch_bounds__(kOrdThreads) k_kd_bottom(const double *__restrict__ xy, int n, int level,
+                                                            const uint32_t *__restrict__ list, uint32_t *__restrict__ pos,
+                                                            int64_t *__restrict__ perm) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    KdShared &S = *reinterpret_cast<KdShared *>(raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int a0 = 0, M = n;
+    for (int l = level - 1; l >= 0; --l) {
+        const int h = (M + 1) / 2;
+        const bool right = (blockIdx.x >> l) & 1;
+        a0 += right ? h : 0;
+        M = right ? M - h : h;
+    }
+    for (int p = tid; p < M; p += kOrdThreads) {
+        const uint32_t i = list[a0 + p];
+        S.id[p] = i;
+        S.x[p] = xy[i];
+        S.y[p] = xy[n + i];
+        S.lx[0][p] = (uint16_t)p;
+        pos[i] = (uint32_t)p;
+    }
+    __syncthreads();
+    for (int p = tid; p < M; p += kOrdThreads) S.ly[0][p] = (uint16_t)pos[list[(int64_t)n + a0 + p]];
+    __syncthreads();
+    int a[2] = {0, 0}, m[2] = {M, M};  // node of positions 2 tid, 2 tid + 1
+    int cur = 0;
+    for (int big = M; big > 1; big = (big + 1) / 2, cur ^= 1) {
+        const uint16_t *X = S.lx[cur], *Y = S.ly[cur];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int p = 2 * tid + u;
+            if (p < M && p == a[u])
+                S.dim_x[p] = kd_split_x(S.x[X[p]], S.x[X[p + m[u] - 1]], S.y[Y[p]], S.y[Y[p + m[u] - 1]]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int p = 2 * tid + u;
+            if (p < M) S.side[S.dim_x[a[u]] ? X[p] : Y[p]] = p - a[u] < (m[u] + 1) / 2;
+        }
+        __syncthreads();
+        // lefts before every position of both lists
+        int lf[2][2], inc[2];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int p = 2 * tid + u;
+                lf[d][u] = p < M ? (int)S.side[d ? Y[p] : X[p]] : 0;
+            }
+            inc[d] = lf[d][0] + lf[d][1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xFFFFFFFFu, inc[d], o);
+                if (lane >= o) inc[d] += t;
+            }
+            if (lane == 31) S.wsum[d][warp] = inc[d];
+        }
+        __syncthreads();
+        if (warp < 2) {
+            const int v = S.wsum[warp][lane];
+            int s = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xFFFFFFFFu, s, o);
+                if (lane >= o) s += t;
+            }
+            S.wsum[warp][lane] = s - v;
+        }
+        __syncthreads();
+        int f[2][2];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            f[d][0] = S.wsum[d][warp] + inc[d] - lf[d][0] - lf[d][1];
+            f[d][1] = f[d][0] + lf[d][0];
+            int *F = d ? S.fy : S.fx;
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (2 * tid + u < M) F[2 * tid + u] = f[d][u];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int p = 2 * tid + u, h = (m[u] + 1) / 2;
+            if (p >= M) continue;
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                const int before = f[d][u] - (d ? S.fy : S.fx)[a[u]];
+                (d ? S.ly : S.lx)[cur ^ 1][lf[d][u] ? a[u] + before : a[u] + h + (p - a[u]) - before] = d ? Y[p] : X[p];
+            }
+            if (p - a[u] < h) {
+                m[u] = h;
+            } else {
+                a[u] += h;
+                m[u] -= h;
+            }
+        }
+        __syncthreads();
+    }
+    for (int p = tid; p < M; p += kOrdThreads) perm[a0 + p] = (int64_t)S.id[S.lx[cur][p]];
+}
+
+// Max-min on one cluster: every CTA keeps a share of the points (coordinates
+// and minimum squared distances) in shared memory, and a step is one pass over
+// it, the argmax by warp reductions of the distances' bit patterns (nonnegative
+// doubles order like their bits; a taken point, -1, comes below), and one
+// exchange of the CTAs' candidates.  The FP64 distance (7 operations of 64
+// cycles a warp) is formed only where an FP32 box test cannot rule it out:
+// |dx| > r or |dy| > r with r above the square root of the minimum distance by
+// more than every rounding involved means that the distance is larger.  Steps
+// depend on one another: 1 us each, most of it the exchange.
+constexpr int kMaxminClusterN = 98304;  // 36 bytes a point, 6,144 points a CTA
+constexpr int kMmThreads = 512, kMmWarps = kMmThreads / 32;
+struct MmCand {
+    int hi;
+    uint32_t lo;
+    int64_t i;
+    double x, y;
+};
+// Best candidate over the warp: largest (hi, lo), then the lowest index; its
+// lane in `who`.
+__device__ __forceinline__ void mm_best(int hi, uint32_t lo, uint32_t i, int &who) {
+    const int mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+    const uint32_t ml = __reduce_max_sync(0xFFFFFFFFu, hi == mh ? lo : 0u);
+    const bool top = hi == mh && lo == ml;
+    const uint32_t mi = __reduce_min_sync(0xFFFFFFFFu, top ? i : 0xFFFFFFFFu);
+    who = __ffs(__ballot_sync(0xFFFFFFFFu, top && i == mi)) - 1;
+}
+static size_t maxmin_bytes(int n) { return (size_t)ceil_div(n, kOrdCl) * (3 * sizeof(double) + 3 * sizeof(float)) + 64; }
+__global__ void __launch_bounds__(kMmThreads) k_maxmin_cluster(const double *__restrict__ xy, int n, int nfirst,
+                                                                const double *__restrict__ first_v,
+                                                                const long long *__restrict__ first_i,
+                                                                int64_t *__restrict__ perm) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    __shared__ MmCand slot[2][kOrdCl], wbest[kMmWarps];
+    __shared__ float emax[kMmWarps];
+    __shared__ long long s_p;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = (n + kOrdCl - 1) / kOrdCl, g0 = min(n, rank * per), cnt = min(n, g0 + per) - g0;
+    double *X = reinterpret_cast<double *>(raw), *Y = X + per, *D = Y + per;
+    float *X4 = reinterpret_cast<float *>(D + per), *Y4 = X4 + per, *R4 = Y4 + per;
+    for (int j = tid; j < cnt; j += kMmThreads) {
+        X[j] = xy[g0 + j];
+        Y[j] = xy[n + g0 + j];
+        D[j] = INFINITY;
+        X4[j] = (float)X[j];
+        Y4[j] = (float)Y[j];
+        R4[j] = INFINITY;
+    }
+    // slack: above the rounding of a coordinate difference in FP32 (at most
+    // 4 x 2^-24 of the largest magnitude); a non-finite coordinate makes it
+    // infinite and switches the box test off
+    float big = 0.f;
+    for (int j = tid; j < n; j += kMmThreads) {
+        const double x = xy[j], y = xy[n + j];
+        big = isfinite(x) && isfinite(y) ? fmaxf(big, fmaxf(fabsf((float)x), fabsf((float)y))) : INFINITY;
+    }
+    for (int o = 16; o; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xFFFFFFFFu, big, o));
+    if (lane == 0) emax[warp] = big;
+    // the first point: the nearest to the box's centre
+    double fv = INFINITY;
+    long long fi = 0x7FFFFFFFFFFFFFFFll;
+    for (int b = tid; b < nfirst; b += kMmThreads)
+        if (better_min(first_v[b], first_i[b], fv, fi)) {
+            fv = first_v[b];
+            fi = first_i[b];
+        }
+    const MaxLoc r0 = block_argext(fv, fi, false);
+    if (tid == 0) s_p = r0.i;
+    __syncthreads();
+    for (int w = 0; w < kMmWarps; ++w) big = fmaxf(big, emax[w]);
+    const float slack = big * 4.8e-7f + 1e-37f;  // 8 x 2^-24
+    int64_t p = s_p;
+    if (p < 0 || p >= n) p = 0;  // only reachable with non-finite coordinates
+    double px = xy[p], py = xy[n + p];
+    cl.sync();
+    for (int k = 0; k < n; ++k) {
+        if (rank == 0 && tid == 0) perm[k] = p;
+        const float px4 = (float)px, py4 = (float)py;
+        int bh = INT32_MIN;
+        uint32_t bl = 0, bi = 0xFFFFFFFFu;
+        for (int j = tid; j < cnt; j += kMmThreads) {
+            double m = D[j];
+            const float r = R4[j];
+            if (g0 + j == p) {
+                m = -1.0;  // taken
+                D[j] = m;
+                R4[j] = -1.f;
+            } else if (r >= 0.f && !(fabsf(X4[j] - px4) > r) && !(fabsf(Y4[j] - py4) > r)) {
+                const double d = sqdist(X[j], Y[j], px, py);
+                if (!(d >= m)) {
+                    m = fmin(m, d);
+                    D[j] = m;
+                    const float m4 = (float)m;
+                    R4[j] = (m4 < 1e-30f ? 1.0001e-15f : sqrtf(m4) * 1.00001f) + slack;
+                }
+            }
+            const int h = __double2hiint(m);
+            const uint32_t l = (uint32_t)__double2loint(m);
+            if (h > bh || (h == bh && l > bl)) {  // indices rise: the first of equals stays
+                bh = h;
+                bl = l;
+                bi = (uint32_t)(g0 + j);
+            }
+        }
+        int who;
+        mm_best(bh, bl, bi, who);
+        if (lane == who) wbest[warp] = MmCand{bh, bl, (int64_t)bi, 0.0, 0.0};
+        __syncthreads();
+        if (warp == 0) {
+            const MmCand c = lane < kMmWarps ? wbest[lane] : MmCand{INT32_MIN, 0u, (int64_t)0xFFFFFFFF, 0.0, 0.0};
+            mm_best(c.hi, c.lo, (uint32_t)c.i, who);
+            MmCand b;
+            b.hi = __shfl_sync(0xFFFFFFFFu, c.hi, who);
+            b.lo = __shfl_sync(0xFFFFFFFFu, c.lo, who);
+            const uint32_t i = __shfl_sync(0xFFFFFFFFu, (uint32_t)c.i, who);
+            const int j = (int)i - g0;
+            const bool own = i != 0xFFFFFFFFu;
+            b.i = (int64_t)i;
+            b.x = own ? X[j] : 0.0;
+            b.y = own ? Y[j] : 0.0;
+            if (lane < kOrdCl) cl.map_shared_rank(&slot[k & 1][0], lane)[rank] = b;
+        }
+        cl.sync();
+        const MmCand c = lane < kOrdCl ? slot[k & 1][lane] : MmCand{INT32_MIN, 0u, (int64_t)0xFFFFFFFF, 0.0, 0.0};
+        mm_best(c.hi, c.lo, (uint32_t)c.i, who);
+        p = (int64_t)__shfl_sync(0xFFFFFFFFu, (uint32_t)c.i, who);
+        px = __shfl_sync(0xFFFFFFFFu, c.x, who);
+        py = __shfl_sync(0xFFFFFFFFu, c.y, who);
+    }
+}
+
+// Whether clusters of 16 CTAs of the kernels above run on this device.
+static bool cluster_order_ok() {
+    static std::once_flag once;
+    static bool ok = false;
+    std::call_once(once, [] {
+        int dev = 0, optin = 0;
+        ok = cudaGetDevice(&dev) == cudaSuccess &&
+             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+             cudaFuncSetAttribute(k_kd_bottom, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KdShared)) == cudaSuccess;
+        cudaFuncAttributes fa;
+        ok = ok && cudaFuncGetAttributes(&fa, k_maxmin_cluster) == cudaSuccess &&
+             cudaFuncSetAttribute(k_maxmin_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  optin - (int)fa.sharedSizeBytes) == cudaSuccess;
+        auto fits = [](const void *k, int threads, size_t smem) {
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kOrdCl);
+            cfg.blockDim = dim3((unsigned)threads);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = kOrdCl;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int nc = 0;
+            return cudaOccupancyMaxActiveClusters(&nc, k, &cfg) == cudaSuccess && nc > 0;
+        };
+        ok = ok && fits((const void *)k_sfc_cluster, kOrdThreads, 0) && fits((const void *)k_kd_sort, kOrdThreads, 0) &&
+             fits((const void *)k_kd_top, kOrdThreads, 0) &&
+             fits((const void *)k_maxmin_cluster, kMmThreads, maxmin_bytes(kMaxminClusterN));
+        cudaGetLastError();  // clear any error of the queries
+    });
+    return ok;
+}
+
 // ------------------------------------------------------------- drivers
 static inline int grid1(int64_t n, int t = 256) { return (int)ceil_div(n > 0 ? n : 1, t); }
 
 void order_sfc(const double *xy, int64_t n, int method, uint64_t seed, int64_t *perm,
-               uint32_t *codes, cudaStream_t s) {
+               uint32_t *codes, double *xy_out, int quantize, cudaStream_t s) {
+    if (n <= kClusterMaxN && cluster_order_ok()) {
+        DevBuf b(16 * n, s);
+        uint32_t *k = b.as<uint32_t>();
+        launch_clustered(k_sfc_cluster, kOrdCl, 1, kOrdThreads, 0, s, xy, (int)n, method, seed, k, k + n, k + 2 * n,
+                         k + 3 * n, codes, perm, xy_out, quantize);
+        return;
+    }
     DevBuf kb(n * 4, s), vb(n * 4, s), kt(n * 4, s), vt(n * 4, s), hb(hist_words(n) * 4, s);
     uint32_t *keys = kb.as<uint32_t>(), *vals = vb.as<uint32_t>();
     uint32_t *ktmp = kt.as<uint32_t>(), *vtmp = vt.as<uint32_t>();
@@ -434,6 +1041,7 @@ void order_sfc(const double *xy, int64_t n, int method, uint64_t seed, int64_t *
     radix_sort<uint32_t>(&keys, &vals, &ktmp, &vtmp, n, 32, hb.as<uint32_t>(), s);
     launch(k_perm_out, grid1(n), 256, 0, s, vals, n, perm);
     TLR_CHECK_LAUNCH();
+    if (xy_out) permute_xy(xy, perm, n, quantize, xy_out, s);
 }
 
 static int bit_width(uint64_t v) {
@@ -445,6 +1053,24 @@ static int bit_width(uint64_t v) {
 void order_kdtree(const double *xy, int64_t n, int64_t *perm, cudaStream_t s) {
     if (n <= 1) {
         if (n == 1) launch(k_iota, 1, 32, 0, s, n, perm);
+        return;
+    }
+    if (n <= kClusterMaxN && cluster_order_ok()) {
+        // keys and values of both dimensions with their copies, two pairs of lists, sides
+        DevBuf b(n * (4 * 8 + 4 * 4 + 4 * 4 + 4) + 16, s);
+        uint64_t *keys = b.as<uint64_t>(), *ktmp = keys + 2 * n;
+        uint32_t *vals = reinterpret_cast<uint32_t *>(ktmp + 2 * n), *vtmp = vals + 2 * n, *list = vtmp + 2 * n,
+                 *ltmp = list + 2 * n, *pos = ltmp + 2 * n;
+        launch_clustered(k_kd_sort, kOrdCl, 2, kOrdThreads, 0, s, xy, (int)n, keys, ktmp, vals, vtmp, list);
+        int levels = 0;  // until every node has at most kKdLocal points
+        while (ceil_div(n, (int64_t)1 << levels) > kKdLocal) ++levels;
+        if (levels) {
+            launch_clustered(k_kd_top, kOrdCl, 1, kOrdThreads, 0, s, xy, (int)n, list, ltmp,
+                             reinterpret_cast<uint8_t *>(keys), levels);
+            if (levels & 1) std::swap(list, ltmp);
+        }
+        launch(k_kd_bottom, 1u << levels, kOrdThreads, sizeof(KdShared), s, xy, (int)n, levels, list, pos, perm);
+        TLR_CHECK_LAUNCH();
         return;
     }
     DevBuf kb(n * 8, s), kt(n * 8, s), vb(n * 4, s), vt(n * 4, s), hb(hist_words(n) * 4, s);
@@ -508,6 +1134,11 @@ void order_maxmin(const double *xy, int64_t n, int64_t *perm, cudaStream_t s, in
     launch(k_bbox, 1, 1024, 0, s, xy, n, ctr.as<double>());
     launch(k_maxmin_first, nblk, 256, 0, s, xy, n, ctr.as<double>(), pv.as<double>(), pi.as<long long>());
     TLR_CHECK_LAUNCH();
+    if (n <= kMaxminClusterN && cluster_order_ok()) {
+        launch_clustered(k_maxmin_cluster, kOrdCl, 1, kMmThreads, maxmin_bytes((int)n), s, xy, (int)n, nblk,
+                         pv.as<double>(), pi.as<long long>(), perm);
+        return;
+    }
     double *bv[2] = {pv.as<double>(), pv.as<double>() + nblk};
     long long *bi[2] = {pi.as<long long>(), pi.as<long long>() + nblk};
     for (int64_t k = 0; k < n; ++k) {

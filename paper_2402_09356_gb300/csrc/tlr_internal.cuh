@@ -110,8 +110,9 @@ void compress_packed(tlr_ctx *ctx, cudaStream_t s, const double *tiles, tlr_mat 
                      long long *info);
 
 // ordering (order.cu)
-void order_sfc(const double *xy, int64_t n, int method, uint64_t seed, int64_t *perm, uint32_t *codes,
-               cudaStream_t s);
+// xy_out (may be null): the permuted locations, quantised as q / 65535 on request.
+void order_sfc(const double *xy, int64_t n, int method, uint64_t seed, int64_t *perm, uint32_t *codes, double *xy_out,
+               int quantize, cudaStream_t s);
 void order_kdtree(const double *xy, int64_t n, int64_t *perm, cudaStream_t s);
 void order_maxmin(const double *xy, int64_t n, int64_t *perm, cudaStream_t s, int num_sms);
 void order_identity(int64_t n, int64_t *perm, cudaStream_t s);

@@ -688,64 +688,14 @@ __device__ __forceinline__ T col_norm2(const T *x, int sdot, int lane) {
 // columns (first sdot entries) and are updated, so that a pair costs one dot
 // product instead of three (the update is c^2 (a -+ 2 t g + t^2 b), exact for
 // any t; a norm is recomputed when that formula cancels more than three
-// digits).  Returns whether a rotation was applied.  Pairs with
-// |x'y| <= tol |x| |y| (tol2 = tol^2) are left alone.
+// digits).  Pairs with |x'y| <= tol |x| |y| are left alone (returns 0); returns
+// 1 for a rotated pair that leaves the sweep's result final (below), else 2.
 // FP64: the rotation angle only steers convergence, so t = tan(angle) comes
 // from approximations; c = 1/sqrt(1 + t^2) is refined by two Newton steps for
 // the reciprocal square root, y <- y (3 - x y^2) / 2, so that (c, c t) is
 // orthogonal to working precision and the singular values are preserved.
 template <class T>
-__device__ __forceinline__ bool jacobi_rotate(T *x, T *y, T *nx, T *ny, int sdot, int srot, int lane, T tol2) {
-    const T al = *nx, be = *ny;
-    T ga = 0;
-    if constexpr (std::is_same<T, float>::value) {
-        const float2 *x2 = reinterpret_cast<const float2 *>(x), *y2 = reinterpret_cast<const float2 *>(y);
-        for (int i = lane; 2 * i < sdot; i += 32) {
-            const float2 u = x2[i], v = y2[i];
-            ga = fmaf(u.x, v.x, ga);
-            if (2 * i + 1 < sdot) ga = fmaf(u.y, v.y, ga);
-        }
-    } else {
-        for (int r = lane; r < sdot; r += 32) ga = fma(x[r], y[r], ga);
-    }
-    ga = warp_sum(ga);
-    if (ga == T(0) || ga * ga <= tol2 * (al * be)) return false;
-    T c, sn, t;
-    if constexpr (std::is_same<T, double>::value) {
-        double rg = rcp_approx(2.0 * ga);
-        rg = rg * fma(-2.0 * ga, rg, 2.0);
-        const double zeta = (be - al) * rg, az = fabs(zeta);
-        const double q = fma(zeta, zeta, 1.0);
-        t = copysign(az < 1e150 ? rcp_approx(az + q * rsqrt_approx(q)) : 0.5 * rcp_approx(az), zeta);
-        const double u = fma(t, t, 1.0);
-        c = rsqrt_approx(u);
-        c = c * fma(-0.5 * u * c, c, 1.5);
-        c = c * fma(-0.5 * u * c, c, 1.5);
-        sn = c * t;
-    } else {
-        // approximate reciprocals and square root: (c, c t) is orthogonal to
-        // FP32 accuracy for any t, so only convergence depends on them
-        const float zeta = __fdividef(be - al, 2.0f * ga), az = fabsf(zeta);
-        if (az >= 1e18f) return false;  // t below FP32 resolution
-        const float q = fmaf(zeta, zeta, 1.0f);
-        t = copysignf(__fdividef(1.0f, az + q * rsqrtf(q)), zeta);
-        c = rsqrtf(fmaf(t, t, 1.0f));
-        sn = c * t;
-    }
-    if constexpr (std::is_same<T, float>::value) {
-        float2 *x2 = reinterpret_cast<float2 *>(x), *y2 = reinterpret_cast<float2 *>(y);
-        for (int i = lane; 2 * i < srot; i += 32) {  // srot is even in the FP32 phase
-            const float2 a = x2[i], b = y2[i];
-            x2[i] = make_float2(fmaf(c, a.x, -sn * b.x), fmaf(c, a.y, -sn * b.y));
-            y2[i] = make_float2(fmaf(sn, a.x, c * b.x), fmaf(sn, a.y, c * b.y));
-        }
-    } else {
-        for (int r = lane; r < srot; r += 32) {
-            const T a = x[r], b = y[r];
-            x[r] = fma(c, a, -sn * b);
-            y[r] = fma(sn, a, c * b);
-        }
-    }
+__device__ __forceinline__ void rotated_norms(T *x, T *y, T *nx, T *ny, T al, T be, T ga, T c, T t, int sdot, int lane) {
     const T c2 = c * c, tg = T(2) * t * ga, tt = t * t;
     T al2 = c2 * (al - tg + tt * be), be2 = c2 * (be + tg + tt * al);
     if (!(al2 > T(1e-3) * c2 * (al + tt * be))) al2 = col_norm2(x, sdot, lane);
@@ -754,17 +704,112 @@ __device__ __forceinline__ bool jacobi_rotate(T *x, T *y, T *nx, T *ny, int sdot
         *nx = al2;
         *ny = be2;
     }
-    return true;
+}
+__device__ __forceinline__ int jacobi_rotate(double *x, double *y, double *nx, double *ny, int sdot, int srot, int lane,
+                                             double tol) {
+    const double al = *nx, be = *ny;
+    double ga = 0.0;
+    for (int r = lane; r < sdot; r += 32) ga = fma(x[r], y[r], ga);
+    ga = warp_sum(ga);
+    if (ga == 0.0 || ga * ga <= tol * tol * (al * be)) return 0;
+    double rg = rcp_approx(2.0 * ga);
+    rg = rg * fma(-2.0 * ga, rg, 2.0);
+    const double zeta = (be - al) * rg, az = fabs(zeta);
+    const double q = fma(zeta, zeta, 1.0);
+    const double t = copysign(az < 1e150 ? rcp_approx(az + q * rsqrt_approx(q)) : 0.5 * rcp_approx(az), zeta);
+    const double u = fma(t, t, 1.0);
+    double c = rsqrt_approx(u);
+    c = c * fma(-0.5 * u * c, c, 1.5);
+    c = c * fma(-0.5 * u * c, c, 1.5);
+    const double sn = c * t;
+    for (int r = lane; r < srot; r += 32) {
+        const double a = x[r], b = y[r];
+        x[r] = fma(c, a, -sn * b);
+        y[r] = fma(sn, a, c * b);
+    }
+    rotated_norms(x, y, nx, ny, al, be, ga, c, t, sdot, lane);
+    return 2;
+}
+// FP32: entries in pairs, and for srot <= 512 (kKeep pairs a lane) all of both
+// columns in registers from one batch of loads, so that the dot product, the
+// angle and the rotation read shared memory once (loads and stores of x and y
+// one pair at a time wait for each other).  The cosine is formed from the
+// norms' reciprocal square roots: tol^2 |x|^2 |y|^2 would underflow FP32 for
+// columns near the accuracy (1e-11 of the largest), which then never rotated
+// and left the FP64 phase the work.  A pair whose cosine is at most
+// kFinalCos is rotated but does not ask for another sweep: convergence is
+// quadratic, so a sweep that meets no larger cosine leaves them near kFinalCos^2,
+// where the FP64 refinement starts.
+constexpr float kFinalCos = 3e-4f;
+__device__ __forceinline__ int jacobi_rotate(float *x, float *y, float *nx, float *ny, int sdot, int srot, int lane,
+                                             float tol) {
+    constexpr int kKeep = 8;
+    const float al = *nx, be = *ny;
+    float2 *x2 = reinterpret_cast<float2 *>(x), *y2 = reinterpret_cast<float2 *>(y);
+    float2 a[kKeep], b[kKeep];
+    const bool keep = srot <= 64 * kKeep;
+    float ga = 0.f;
+    if (keep) {
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = lane + 32 * k;
+            a[k] = b[k] = make_float2(0.f, 0.f);
+            if (64 * k < srot && 2 * i < srot) {
+                a[k] = x2[i];
+                b[k] = y2[i];
+            }
+        }
+        float g1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k)
+            if (64 * k < sdot) {
+                const int i = lane + 32 * k;
+                if (2 * i < sdot) ga = fmaf(a[k].x, b[k].x, ga);
+                if (2 * i + 1 < sdot) g1 = fmaf(a[k].y, b[k].y, g1);
+            }
+        ga += g1;
+    } else {
+        for (int i = lane; 2 * i < sdot; i += 32) {
+            const float2 u = x2[i], v = y2[i];
+            ga = fmaf(u.x, v.x, ga);
+            if (2 * i + 1 < sdot) ga = fmaf(u.y, v.y, ga);
+        }
+    }
+    ga = warp_sum(ga);
+    if (ga == 0.f) return 0;
+    const float cosine = fabsf(ga) * rsqrtf(al) * rsqrtf(be);
+    if (cosine <= tol) return 0;
+    // approximate reciprocals and square root: (c, c t) is orthogonal to
+    // FP32 accuracy for any t, so only convergence depends on them
+    const float zeta = __fdividef(be - al, 2.0f * ga), az = fabsf(zeta);
+    if (az >= 1e18f) return 0;  // t below FP32 resolution
+    const float q = fmaf(zeta, zeta, 1.0f);
+    const float t = copysignf(__fdividef(1.0f, az + q * rsqrtf(q)), zeta);
+    const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
+    auto rotate = [&](int i, float2 u, float2 v) {
+        x2[i] = make_float2(fmaf(c, u.x, -sn * v.x), fmaf(c, u.y, -sn * v.y));
+        y2[i] = make_float2(fmaf(sn, u.x, c * v.x), fmaf(sn, u.y, c * v.y));
+    };
+    if (keep) {
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = lane + 32 * k;
+            if (64 * k < srot && 2 * i < srot) rotate(i, a[k], b[k]);
+        }
+    } else {
+        for (int i = lane; 2 * i < srot; i += 32) rotate(i, x2[i], y2[i]);
+    }
+    rotated_norms(x, y, nx, ny, al, be, ga, c, t, sdot, lane);
+    return cosine <= kFinalCos ? 1 : 2;
 }
 
-// Convergence threshold of a pair, squared: |x'y| <= 8 sqrt(s) u |x| |y|
-// (u the unit roundoff of T), a few times the rounding error of the dot
+// Convergence threshold of a pair: |x'y| <= 8 sqrt(s) u |x| |y| (u the unit
+// roundoff of T), a few times the rounding error of the dot
 // products, so that rounding alone never keeps a sweep alive.
 template <class T>
-__device__ __forceinline__ T jacobi_tol2(int s) {
+__device__ __forceinline__ T jacobi_tol(int s) {
     const T u = std::is_same<T, double>::value ? T(1.1102230246251565e-16) : T(5.9604644775390625e-8);
-    const T tol = T(8) * sqrt((T)s) * u;
-    return tol * tol;
+    return T(8) * sqrt((T)s) * u;
 }
 
 // Sort key of a column norm: non-finite values sort last.
@@ -782,11 +827,11 @@ __device__ __forceinline__ int pos_of(int blk, int g, int nblk) {
 // Rotate all pairs between the two b-column blocks X (global block bx) and Y
 // (by), and, if `inner`, the pairs within each of them.  Columns are srot
 // apart within a block; NX, NY hold their squared norms.  Virtual columns
-// (global index >= s) are zero and skipped.  Returns whether any rotation was
-// applied by this thread's warp.
+// (global index >= s) are zero and skipped.  Returns whether this thread's warp
+// rotated a pair that asks for another sweep (jacobi_rotate).
 template <class T>
 __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int bx, int by, int b, int s, int srot,
-                                                   bool inner, int lane, int warp, T tol2, int &nchk, int &nrot) {
+                                                   bool inner, int lane, int warp, T tol, int &nchk, int &nrot) {
     bool rot = false;
     if (inner) {
         const int bp = b + (b & 1);
@@ -800,10 +845,10 @@ __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int
                 T *base = slot ? Y : X;
                 T *nrm = slot ? NY : NX;
                 const int lo = min(a, c2), hi = max(a, c2);
-                const bool r = jacobi_rotate(base + lo * srot, base + hi * srot, nrm + lo, nrm + hi, s, srot, lane, tol2);
-                rot |= r;
+                const int r = jacobi_rotate(base + lo * srot, base + hi * srot, nrm + lo, nrm + hi, s, srot, lane, tol);
+                rot |= r > 1;
                 ++nchk;
-                nrot += r;
+                nrot += r > 0;
             }
             __syncthreads();
         }
@@ -814,11 +859,12 @@ __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int
             const int gx = bx * b + i, gy = by * b + jy;
             if (gx >= s || gy >= s) continue;
             // the lower global index is the first column of the pair
-            const bool r = gx < gy ? jacobi_rotate(X + i * srot, Y + jy * srot, NX + i, NY + jy, s, srot, lane, tol2)
-                                   : jacobi_rotate(Y + jy * srot, X + i * srot, NY + jy, NX + i, s, srot, lane, tol2);
-            rot |= r;
+            T *Xi = X + i * srot, *Yj = Y + jy * srot, *nx = NX + i, *ny = NY + jy;
+            const bool swap = gx >= gy;
+            const int r = jacobi_rotate(swap ? Yj : Xi, swap ? Xi : Yj, swap ? ny : nx, swap ? nx : ny, s, srot, lane, tol);
+            rot |= r > 1;
             ++nchk;
-            nrot += r;
+            nrot += r > 0;
         }
         __syncthreads();
     }
@@ -840,7 +886,7 @@ __device__ __forceinline__ void block_norms(const T *cols, T *nrm, int b, int s,
 // (buf0 + cur * stride: slot 0, slot 1, then 2b norms); after each block
 // round the CTAs pull their next blocks over DSMEM into the other buffer.
 // Norms are recomputed at the start of every sweep.  Runs until a sweep
-// rotates nothing or max_sweeps; g (global round) and cur are updated so
+// asks for no other (jacobi_rotate) or max_sweeps; g (global round) and cur are updated so
 // that buffer cur holds the blocks of positions (rank, 2C - 1 - rank) at
 // round g on return.  Returns the number of sweeps run.
 template <int kCl, class T>
@@ -850,7 +896,7 @@ __device__ int jacobi_sweeps(cg::cluster_group &cl, T *buf0, int stride, int b, 
     constexpr int nblk = 2 * kCl;
     const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int px = rank, py = nblk - 1 - rank, bs = b * srot;
-    const T tol2 = jacobi_tol2<T>(s);
+    const T tol = jacobi_tol<T>(s);
     auto buf = [&](int k) { return buf0 + k * stride; };
     int nsweep = 0;
     bool done = false;
@@ -861,7 +907,7 @@ __device__ int jacobi_sweeps(cg::cluster_group &cl, T *buf0, int stride, int b, 
             const int bx = block_at(px, g, nblk), by = block_at(py, g, nblk);
             T *B = buf(cur);
             if (jacobi_block_pairs<T>(B, B + bs, B + 2 * bs, B + 2 * bs + b, bx, by, b, s, srot, round == 0, lane,
-                                      warp, tol2, nchk, nrot) &&
+                                      warp, tol, nchk, nrot) &&
                 lane == 0)
                 s_flag[sweep & 1] = 1;
             cl.sync();
@@ -890,21 +936,25 @@ __device__ int jacobi_sweeps(cg::cluster_group &cl, T *buf0, int stride, int b, 
                     const T *ns = cl.map_shared_rank(buf(cur), h) + 2 * bs + hs * b;
                     for (int e = tid; e < b; e += kQrThreads) dst[2 * bs + slot * b + e] = ns[e];
                 }
-                constexpr int kPull = 4;
-                for (int e0 = tid; e0 < bs; e0 += kPull * kQrThreads) {
-                    T v[2][kPull];
+                // 8 bytes a load: FP32 entries in pairs (bs = 2 b s is even)
+                constexpr int kPull = 4, kPer = 8 / sizeof(T);
+                const int bp = bs / kPer;
+                const double *s0 = reinterpret_cast<const double *>(src[0]), *s1 = reinterpret_cast<const double *>(src[1]);
+                double *d0 = reinterpret_cast<double *>(dst), *d1 = reinterpret_cast<double *>(dst + bs);
+                for (int e0 = tid; e0 < bp; e0 += kPull * kQrThreads) {
+                    double v[2][kPull];
 #pragma unroll
                     for (int u = 0; u < kPull; ++u) {
                         const int e = e0 + u * kQrThreads;
-                        v[0][u] = e < bs ? src[0][e] : T(0);
-                        v[1][u] = e < bs ? src[1][e] : T(0);
+                        v[0][u] = e < bp ? s0[e] : 0.0;
+                        v[1][u] = e < bp ? s1[e] : 0.0;
                     }
 #pragma unroll
                     for (int u = 0; u < kPull; ++u) {
                         const int e = e0 + u * kQrThreads;
-                        if (e < bs) {
-                            dst[e] = v[0][u];
-                            dst[bs + e] = v[1][u];
+                        if (e < bp) {
+                            d0[e] = v[0][u];
+                            d1[e] = v[1][u];
                         }
                     }
                 }
@@ -960,6 +1010,7 @@ __device__ void jacobi_rank(const SvdJob &J, const double *all_nrm, int sweeps, 
 
 constexpr int kMaxSweeps32 = 12;
 constexpr int kRefineSteps = 3;  // FP64 Gram refinement steps after the FP32 sweeps
+constexpr int kMoreRounds = 2;   // rounds of two more steps for tiles they did not finish
 
 // Block Jacobi with the blocks in shared memory, in two precisions.
 //  A. FP32 sweeps on fl32(M), M = R', carrying the accumulated rotations J
@@ -1170,10 +1221,12 @@ __global__ void k_refine_angles(const RefineJob *__restrict__ jobs) {
     if ((threadIdx.x & 31) == 0 && worst > 0.0) atomicMax(J.off, (unsigned long long)__double_as_longlong(worst));
 }
 
-// Singular values and vectors of the refined M1 (one CTA per job): column
-// norms, descending order (non-finite last), W = unit columns, S, and the
-// rank #{S > tau}: -1 for non-finite values, -2 when the refinement had not
-// converged (the caller then finishes with FP64 Jacobi sweeps).
+// Singular values and vectors of the refined M1: column norms (one warp a
+// column), then their descending order (non-finite last), W = unit columns, S,
+// and the rank #{S > tau}: -1 for non-finite values, -2 when the refinement had
+// not converged but is close enough that more steps will do, -3 when it is not
+// (FP64 Jacobi sweeps finish the tile).  Eight columns a CTA: one CTA a tile
+// took 77 us on average, its FP64 operations in a row.
 struct EmitJob {
     const double *X;   // s x s refined M1 (ld s)
     double *W;
@@ -1182,18 +1235,27 @@ struct EmitJob {
     const unsigned long long *off;
     int s;
     double tau;
+    double *nrm;       // s column norms (scratch)
 };
+constexpr double kNewtonCos = 1e-3;  // largest cosine the refinement is continued from
+
+__global__ void __launch_bounds__(kQrThreads) k_svd_norms(const EmitJob *__restrict__ jobs) {
+    const EmitJob J = jobs[blockIdx.y];
+    const int s = J.s, lane = threadIdx.x & 31, u = blockIdx.x * kNw + (threadIdx.x >> 5);
+    if (u >= s) return;
+    const double v = col_norm2(J.X + (int64_t)u * s, s, lane);
+    if (lane == 0) J.nrm[u] = sqrt(v);
+}
 
 __global__ void __launch_bounds__(kQrThreads) k_svd_emit(const EmitJob *__restrict__ jobs) {
-    extern __shared__ double nrm[];
-    const EmitJob J = jobs[blockIdx.x];
-    const int s = J.s, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int u = warp; u < s; u += kNw) {
-        const double v = col_norm2(J.X + (int64_t)u * s, s, lane);
-        if (lane == 0) nrm[u] = sqrt(v);
-    }
+    __shared__ double nrm[kMaxSample];
+    __shared__ int cnt[kNw], bad[kNw];
+    const EmitJob J = jobs[blockIdx.y];
+    const int s = J.s, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, u = blockIdx.x * kNw + warp;
+    if ((int)blockIdx.x * kNw >= s) return;
+    for (int e = tid; e < s; e += kQrThreads) nrm[e] = J.nrm[e];
     __syncthreads();
-    for (int u = warp; u < s; u += kNw) {
+    if (u < s) {
         const double ku = norm_key(nrm[u]);
         int pos = 0;
         for (int w = lane; w < s; w += 32) {
@@ -1208,16 +1270,27 @@ __global__ void __launch_bounds__(kQrThreads) k_svd_emit(const EmitJob *__restri
         for (int r = lane; r < s; r += 32) J.W[(int64_t)pos * s + r] = col[r] * inv;
         if (lane == 0) J.S[pos] = nv;
     }
+    if (blockIdx.x) return;
+    int r = 0, b = 0;
+    for (int e = tid; e < s; e += kQrThreads) {
+        r += nrm[e] > J.tau;
+        b |= !(nrm[e] <= 1.7e308);
+    }
+    r = __reduce_add_sync(0xFFFFFFFFu, r);
+    b = __reduce_or_sync(0xFFFFFFFFu, b);
+    if (lane == 0) {
+        cnt[warp] = r;
+        bad[warp] = b;
+    }
+    __syncthreads();
     if (tid == 0) {
-        int r = 0;
-        bool bad = false;
-        for (int u = 0; u < s; ++u) {
-            r += nrm[u] > J.tau;
-            bad |= !(nrm[u] <= 1.7e308);
+        for (int w = 1; w < kNw; ++w) {
+            r += cnt[w];
+            b |= bad[w];
         }
         const double off = __longlong_as_double((long long)*J.off);
         const double tol = 8.0 * sqrt((double)s) * 1.1102230246251565e-16;
-        *J.rank = bad ? -1 : (off > tol ? -2 : r);
+        *J.rank = b ? -1 : (off > tol ? (off <= kNewtonCos ? -2 : -3) : r);
     }
 }
 
@@ -1259,7 +1332,7 @@ __global__ void __launch_bounds__(kQrThreads) k_jacobi_gm(const SvdJob *__restri
             block_norms(Ab, Nb, b, s, s, lane, warp);
             int nchk = 0, nrot = 0;
             if (jacobi_block_pairs<double>(Ab, Ab + bs, Nb, Nb + b, bx, by, b, s, s, round == 0, lane, warp,
-                                           jacobi_tol2<double>(s), nchk, nrot) &&
+                                           jacobi_tol<double>(s), nchk, nrot) &&
                 lane == 0)
                 s_flag[sweep & 1] = 1;
             for (int e = tid; e < 2 * bs; e += kQrThreads) {
@@ -1748,58 +1821,58 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
             t16.e1 = pooled_event(ctx, ev_used);
         }
         svd_launch(ctx, st, sv, svd_csize, ctx->profile ? &t16 : nullptr, kJacPrecond);
-        // FP64 Gram refinement (batched over the tiles), then W, S and the rank
-        std::vector<double *> xfin(np, nullptr);
+        // FP64 Gram refinement of the tiles `rj` (batched), then W, S and the rank
+        std::vector<double *> X(np, nullptr), Xn(np, nullptr);
+        auto refine = [&](const std::vector<size_t> &rj, int steps) {
+            if (rj.empty()) return;
+            int smax = 0;
+            for (size_t u : rj) smax = std::max(smax, ps[u]);
+            for (int it = 0; it < steps; ++it) {
+                std::vector<GemmProb> gg, gx;
+                std::vector<RefineJob> rjobs;
+                for (size_t u : rj) {
+                    const int sz = ps[u];
+                    GemmProb a{};
+                    a.A = X[u]; a.lda = sz; a.m = sz; a.k = sz;
+                    a.B = X[u]; a.ldb = sz; a.n = sz;
+                    a.C = W + oG[u]; a.ldc = sz;
+                    gg.push_back(a);
+                    const double tau = jobs[pending[u]].tau;
+                    rjobs.push_back(RefineJob{W + oG[u], W + oIA[u], d_off + u, 0.01 * tau * tau, sz});
+                    GemmProb b{};
+                    b.A = X[u]; b.lda = sz; b.m = sz; b.k = sz;
+                    b.B = W + oIA[u]; b.ldb = sz; b.n = sz;
+                    b.C = Xn[u]; b.ldc = sz;
+                    gx.push_back(b);
+                }
+                gemm_batched_small(ctx, st, true, false, gg, 1.0, 0.0);
+                TLR_CUDA_TRY(cudaMemsetAsync(d_off, 0, np * sizeof(unsigned long long), st));
+                auto *dr = (const RefineJob *)stage_push(ctx, rjobs.data(), rjobs.size() * sizeof(RefineJob), st);
+                launch(k_refine_angles, dim3((unsigned)std::min<int64_t>(ceil_div(smax * smax, 256), 64),
+                                             (unsigned)rjobs.size()), 256, 0, st, dr);
+                TLR_CHECK_LAUNCH();
+                gemm_batched_small(ctx, st, false, false, gx, 1.0, 0.0);
+                for (size_t u : rj) std::swap(X[u], Xn[u]);
+            }
+            std::vector<EmitJob> ej;
+            for (size_t u : rj)
+                ej.push_back(EmitJob{X[u], W + oW[u], W + oS[u], d_rank + u, d_off + u, ps[u], jobs[pending[u]].tau,
+                                     W + oIA[u]});
+            auto *de = (const EmitJob *)stage_push(ctx, ej.data(), ej.size() * sizeof(EmitJob), st);
+            const dim3 grid((unsigned)ceil_div(smax, kNw), (unsigned)ej.size());
+            launch(k_svd_norms, grid, kQrThreads, 0, st, de);
+            launch(k_svd_emit, grid, kQrThreads, 0, st, de);
+            TLR_CHECK_LAUNCH();
+        };
         {
             std::vector<size_t> rj;
-            int smax = 0;
             for (size_t u = 0; u < np; ++u)
                 if (svd_csize[u] > 0) {
                     rj.push_back(u);
-                    smax = std::max(smax, ps[u]);
-                }
-            if (!rj.empty()) {
-                std::vector<double *> X(np), Xn(np);
-                for (size_t u : rj) {
                     X[u] = W + oK[u];
                     Xn[u] = W + oX2[u];
                 }
-                for (int it = 0; it < kRefineSteps; ++it) {
-                    std::vector<GemmProb> gg, gx;
-                    std::vector<RefineJob> rjobs;
-                    for (size_t u : rj) {
-                        const int sz = ps[u];
-                        GemmProb a{};
-                        a.A = X[u]; a.lda = sz; a.m = sz; a.k = sz;
-                        a.B = X[u]; a.ldb = sz; a.n = sz;
-                        a.C = W + oG[u]; a.ldc = sz;
-                        gg.push_back(a);
-                        const double tau = jobs[pending[u]].tau;
-                        rjobs.push_back(RefineJob{W + oG[u], W + oIA[u], d_off + u, 0.01 * tau * tau, sz});
-                        GemmProb b{};
-                        b.A = X[u]; b.lda = sz; b.m = sz; b.k = sz;
-                        b.B = W + oIA[u]; b.ldb = sz; b.n = sz;
-                        b.C = Xn[u]; b.ldc = sz;
-                        gx.push_back(b);
-                    }
-                    gemm_batched_small(ctx, st, true, false, gg, 1.0, 0.0);
-                    TLR_CUDA_TRY(cudaMemsetAsync(d_off, 0, np * sizeof(unsigned long long), st));
-                    auto *dr = (const RefineJob *)stage_push(ctx, rjobs.data(), rjobs.size() * sizeof(RefineJob), st);
-                    launch(k_refine_angles, dim3((unsigned)std::min<int64_t>(ceil_div(smax * smax, 256), 64),
-                                                 (unsigned)rjobs.size()), 256, 0, st, dr);
-                    TLR_CHECK_LAUNCH();
-                    gemm_batched_small(ctx, st, false, false, gx, 1.0, 0.0);
-                    for (size_t u : rj) std::swap(X[u], Xn[u]);
-                }
-                std::vector<EmitJob> ej;
-                for (size_t u : rj) {
-                    ej.push_back(EmitJob{X[u], W + oW[u], W + oS[u], d_rank + u, d_off + u, ps[u], jobs[pending[u]].tau});
-                    xfin[u] = X[u];
-                }
-                auto *de = (const EmitJob *)stage_push(ctx, ej.data(), ej.size() * sizeof(EmitJob), st);
-                launch(k_svd_emit, (unsigned)ej.size(), kQrThreads, (size_t)smax * sizeof(double), st, de);
-                TLR_CHECK_LAUNCH();
-            }
+            refine(rj, kRefineSteps);
         }
         cmark();
         // decisions on the host
@@ -1812,11 +1885,22 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
         TLR_CUDA_TRY(cudaStreamSynchronize(st));
         stage_reset(ctx, st);
         {
-            // tiles whose Gram refinement did not converge: FP64 Jacobi sweeps on the refined M1
+            // tiles whose Gram refinement did not converge: more steps where it
+            // is near (about 0.1 ms a step), else FP64 Jacobi sweeps on the
+            // refined M1 (1 to 8 ms a tile)
+            for (int more = 0; more < kMoreRounds; ++more) {
+                std::vector<size_t> rj;
+                for (size_t u = 0; u < np; ++u)
+                    if (h_rank[u] == -2) rj.push_back(u);
+                if (rj.empty()) break;
+                refine(rj, 2);
+                TLR_CUDA_TRY(cudaMemcpyAsync(h_rank.data(), d_rank, np * sizeof(int), cudaMemcpyDeviceToHost, st));
+                TLR_CUDA_TRY(cudaStreamSynchronize(st));
+            }
             std::vector<SvdJob> fin;
             for (size_t u = 0; u < np; ++u)
-                if (h_rank[u] == -2)
-                    fin.push_back(SvdJob{W + oR[u], xfin[u], W + oW[u], W + oS[u], d_rank + u, d_rank + np + 4 * u, ps[u],
+                if (h_rank[u] == -2 || h_rank[u] == -3)
+                    fin.push_back(SvdJob{W + oR[u], X[u], W + oW[u], W + oS[u], d_rank + u, d_rank + np + 4 * u, ps[u],
                                          jobs[pending[u]].tau});
             if (!fin.empty()) {
                 std::vector<int> cs_fin;

@@ -139,9 +139,16 @@ void split_f2_batched(tlr_ctx *ctx, cudaStream_t s, const std::vector<SplitDesc>
     TLR_CHECK_LAUNCH();
 }
 
+constexpr int kSmallTiles = 300;
 void gemm_batched_small(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
                         double alpha, double beta) {
-    launch_shape<32, 32>(ctx, s, ta, tb, probs, alpha, EpiLinear{beta}, false);
+    // tiles of 32 x 32 while they fill the SMs, else of 16 x 16: an output
+    // tile's chain of FP64 multiply-adds (k x 64 cycles x 2 warps a scheduler, x
+    // 4 outputs a thread) is then a quarter as long, on four times the CTAs
+    int64_t tiles = 0;
+    for (const GemmProb &p : probs) tiles += ceil_div(p.m, 32) * ceil_div(p.n, 32);
+    if (tiles >= kSmallTiles) launch_shape<32, 32>(ctx, s, ta, tb, probs, alpha, EpiLinear{beta}, false);
+    else launch_shape<16, 16>(ctx, s, ta, tb, probs, alpha, EpiLinear{beta}, false);
 }
 
 void gemm_batched(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,

@@ -25,9 +25,9 @@ void *stage_push(tlr_ctx *ctx, const void *data, size_t bytes, cudaStream_t s) {
     return d;
 }
 
-template <int BM, int BN, class Epi>
+template <int BM, int BN>
 static void launch_shape(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
-                         double alpha, const Epi &epi, bool df) {
+                         double alpha, double beta) {
     if (probs.empty()) return;
     std::vector<int> off(probs.size() + 1, 0);
     for (size_t b = 0; b < probs.size(); ++b) {
@@ -40,15 +40,12 @@ static void launch_shape(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const s
     auto *dp = (const GemmProb *)stage_push(ctx, probs.data(), probs.size() * sizeof(GemmProb), s);
     auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
     int np = (int)probs.size();
+    const EpiLinear epi{beta};
     // the transposition pairs the library uses: NN, TN, NT (no TT)
     if (ta && tb) throw make_error(TLR_ERR_ARG, "GEMM with both operands transposed is not provided");
-    if (df) {
-        if (!ta && !tb) launch(k_gemm_df<BM, BN, false, false, Epi>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-        else if (!ta) launch(k_gemm_df<BM, BN, false, true, Epi>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-        else launch(k_gemm_df<BM, BN, true, false, Epi>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-    } else if (!ta && !tb) launch(k_gemm_f64<BM, BN, false, false, Epi>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-    else if (!ta) launch(k_gemm_f64<BM, BN, false, true, Epi>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-    else launch(k_gemm_f64<BM, BN, true, false, Epi>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
+    if (!ta && !tb) launch(k_gemm_f64<BM, BN, false, false, EpiLinear>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
+    else if (!ta) launch(k_gemm_f64<BM, BN, false, true, EpiLinear>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
+    else launch(k_gemm_f64<BM, BN, true, false, EpiLinear>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
     TLR_CHECK_LAUNCH();
 }
 
@@ -70,31 +67,29 @@ static void launch_gemv(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const st
     TLR_CHECK_LAUNCH();
 }
 
-// Split a batch by output shape: problems with at most 32 rows and/or 32
-// columns go to the thin tile shapes, whose padding stays small; FP64
-// matrix-vector products (n = 1) go to the GEMV kernel.
-template <class Epi>
+// The linear products: FP64 matrix-vector products (n = 1) go to the GEMV
+// kernel, everything else to the tiles cut to the problem.
 static void launch_gemm(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
-                        double alpha, const Epi &epi, bool df) {
-    std::vector<GemmProb> cls[4];  // 64x64, 64x32, 32x64, 32x32
-    if constexpr (std::is_same<Epi, EpiLinear>::value) {
-        if (!df) {
-            std::vector<GemmProb> vec, rest;
-            for (const GemmProb &p : probs) (p.n == 1 ? vec : rest).push_back(p);
-            launch_gemv(ctx, s, ta, tb, vec, alpha, epi);
-            for (const GemmProb &p : rest) cls[(p.m <= 32 ? 2 : 0) + (p.n <= 32 ? 1 : 0)].push_back(p);
-            launch_shape<64, 64>(ctx, s, ta, tb, cls[0], alpha, epi, df);
-            launch_shape<64, 32>(ctx, s, ta, tb, cls[1], alpha, epi, df);
-            launch_shape<32, 64>(ctx, s, ta, tb, cls[2], alpha, epi, df);
-            launch_shape<32, 32>(ctx, s, ta, tb, cls[3], alpha, epi, df);
-            return;
-        }
-    }
-    for (const GemmProb &p : probs) cls[(p.m <= 32 ? 2 : 0) + (p.n <= 32 ? 1 : 0)].push_back(p);
-    launch_shape<64, 64>(ctx, s, ta, tb, cls[0], alpha, epi, df);
-    launch_shape<64, 32>(ctx, s, ta, tb, cls[1], alpha, epi, df);
-    launch_shape<32, 64>(ctx, s, ta, tb, cls[2], alpha, epi, df);
-    launch_shape<32, 32>(ctx, s, ta, tb, cls[3], alpha, epi, df);
+                        double alpha, double beta, bool df) {
+    std::vector<GemmProb> fit, vec;
+    for (const GemmProb &p : probs)
+        if (p.m > 0 && p.n > 0) (p.n == 1 && !df ? vec : fit).push_back(p);
+    launch_gemv(ctx, s, ta, tb, vec, alpha, EpiLinear{beta});
+    if (fit.empty()) return;
+    if (ta && tb) throw make_error(TLR_ERR_ARG, "GEMM with both operands transposed is not provided");
+    // 64 columns a tile, fewer while the tiles do not fill the SMs twice
+    int tnmax = kFitMaxTN;
+    auto count = [&](int tn) {
+        int64_t t = 0;
+        for (const GemmProb &p : fit) t += fit_tiles(p.m, p.n, tn);
+        return t;
+    };
+    while (tnmax > 1 && count(tnmax) < 2 * ctx->num_sms) tnmax /= 2;
+    std::vector<int> off(fit.size() + 1, 0);
+    for (size_t b = 0; b < fit.size(); ++b) off[b + 1] = off[b] + fit_tiles(fit[b].m, fit[b].n, tnmax);
+    auto *dp = (const GemmProb *)stage_push(ctx, fit.data(), fit.size() * sizeof(GemmProb), s);
+    auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
+    (df ? gemm_fit_df : gemm_fit_f64)(s, ta, tb, off.back(), dp, dt, (int)fit.size(), tnmax, alpha, beta);
 }
 
 __global__ void k_split_f2(const double *__restrict__ src, int ld, int m, int64_t count,
@@ -147,13 +142,13 @@ void gemm_batched_small(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const st
     // 4 outputs a thread) is then a quarter as long, on four times the CTAs
     int64_t tiles = 0;
     for (const GemmProb &p : probs) tiles += ceil_div(p.m, 32) * ceil_div(p.n, 32);
-    if (tiles >= kSmallTiles) launch_shape<32, 32>(ctx, s, ta, tb, probs, alpha, EpiLinear{beta}, false);
-    else launch_shape<16, 16>(ctx, s, ta, tb, probs, alpha, EpiLinear{beta}, false);
+    if (tiles >= kSmallTiles) launch_shape<32, 32>(ctx, s, ta, tb, probs, alpha, beta);
+    else launch_shape<16, 16>(ctx, s, ta, tb, probs, alpha, beta);
 }
 
 void gemm_batched(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
                   double alpha, double beta, bool df) {
-    launch_gemm(ctx, s, ta, tb, probs, alpha, EpiLinear{beta}, df);
+    launch_gemm(ctx, s, ta, tb, probs, alpha, beta, df);
 }
 
 // The panel update is one large product: 64 x 64 tiles.  A capped grid

@@ -293,6 +293,18 @@ k_gemv(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off, int
     }
 }
 
+// Tiles of k_gemm_fit (gemm_fit.cuh): 64 rows, at most tnmax groups of 8 columns.
+constexpr int kFitMaxTN = 8;
+__host__ __device__ __forceinline__ int fit_col_tiles(int n, int tnmax) { return ((n + 7) / 8 + tnmax - 1) / tnmax; }
+__host__ __device__ __forceinline__ int fit_tiles(int m, int n, int tnmax) {
+    return m > 0 && n > 0 ? ((m + 63) / 64) * fit_col_tiles(n, tnmax) : 0;
+}
+// Launch `tiles` tiles of the problems dp (device; dt their tile offsets).
+void gemm_fit_f64(cudaStream_t s, bool ta, bool tb, int tiles, const GemmProb *dp, const int *dt, int np, int tnmax,
+                  double alpha, double beta);
+void gemm_fit_df(cudaStream_t s, bool ta, bool tb, int tiles, const GemmProb *dp, const int *dt, int np, int tnmax,
+                 double alpha, double beta);
+
 // Host launcher: uploads the descriptors through the context's staging
 // buffers and launches one kernel for the whole batch.
 // dst[j * ld + i] = (hi, lo) of src[j * ld + i] for an m x n column-major block.

@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kQrSmThreads, 2) k_qr_factor(const QrJob *__re
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const QrJob J = jobs[blockIdx.x / kCl];
-    const int m = J.m, s = J.s, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m = J.m, s = J.s, tid = threadIdx.x, warp = tid >> 5;
     const int per = (m + kCl - 1) / kCl, ld = per | 1;
     const int r0 = min(m, rank * per), nr = min(m, r0 + per) - r0;
     extern __shared__ double sm[];
@@ -647,6 +647,7 @@ struct SvdJob {
     int s;
     double tau;        // absolute accuracy of the tile
     const float2 *Rt2; // R' as paired FP32 (the paired-FP32 precondition reads it), or null
+    double *rot;       // s x s output of the precondition: J (as pairs where Rt2 is given)
 };
 
 // Fast approximate reciprocal and reciprocal square root of a double (the
@@ -783,9 +784,9 @@ __device__ __forceinline__ int jacobi_rotate(float *x, float *y, float *nx, floa
     // FP32 accuracy for any t, so only convergence depends on them
     const float zeta = __fdividef(be - al, 2.0f * ga), az = fabsf(zeta);
     if (az >= 1e18f) return 0;  // t below FP32 resolution
-    const float q = fmaf(zeta, zeta, 1.0f);
-    const float t = copysignf(__fdividef(1.0f, az + q * rsqrtf(q)), zeta);
-    const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
+    // h = 1 / sqrt(1 + zeta^2): c^2 = (1 + |zeta| h) / 2, |s| = h / (2 c)
+    const float h = rsqrtf(fmaf(zeta, zeta, 1.0f)), c2 = fmaf(0.5f * az, h, 0.5f), rc = rsqrtf(c2);
+    const float c = c2 * rc, sn = copysignf(0.5f * h * rc, zeta), t = sn * rc;
     auto rotate = [&](int i, float2 u, float2 v) {
         x2[i] = make_float2(fmaf(c, u.x, -sn * v.x), fmaf(c, u.y, -sn * v.y));
         y2[i] = make_float2(fmaf(sn, u.x, c * v.x), fmaf(sn, u.y, c * v.y));
@@ -837,9 +838,11 @@ __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int
         const int bp = b + (b & 1);
         for (int ir = 0; ir < bp - 1; ++ir) {
             for (int pr = warp; pr < bp; pr += kNw) {  // bp/2 pairs per block, two blocks
-                const int slot = pr / (bp / 2), q = pr % (bp / 2);
-                const int a = (q == 0) ? 0 : 1 + (q - 1 + ir) % (bp - 1);
-                const int c2 = 1 + (bp - 2 - q + ir) % (bp - 1);
+                // (no remainder by a run-time size: a hundred cycles each)
+                const int slot = pr >= bp / 2, q = slot ? pr - bp / 2 : pr;
+                const int va = q - 1 + ir, vc = bp - 2 - q + ir;
+                const int a = (q == 0) ? 0 : 1 + (va >= bp - 1 ? va - bp + 1 : va);
+                const int c2 = 1 + (vc >= bp - 1 ? vc - bp + 1 : vc);
                 const int blk = slot ? by : bx;
                 if (a >= b || c2 >= b || blk * b + max(a, c2) >= s) continue;
                 T *base = slot ? Y : X;
@@ -855,7 +858,7 @@ __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int
     }
     for (int k = 0; k < b; ++k) {
         for (int i = warp; i < b; i += kNw) {
-            const int jy = (i + k) % b;
+            const int jy = i + k < b ? i + k : i + k - b;
             const int gx = bx * b + i, gy = by * b + jy;
             if (gx >= s || gy >= s) continue;
             // the lower global index is the first column of the pair
@@ -1015,7 +1018,9 @@ constexpr int kMoreRounds = 2;   // rounds of two more steps for tiles they did 
 // Block Jacobi with the blocks in shared memory, in two precisions.
 //  A. FP32 sweeps on fl32(M), M = R', carrying the accumulated rotations J
 //     (each column holds s entries of M then s of J), until FP32 convergence.
-//  B. M1 = M J in FP64 (M read from R', J from shared memory) into `work`.
+//  B. J is written out; M1 = M J follows as a GEMM (FP64, or paired FP32 from
+//     the paired copy of M: J is exact in FP32, and M1 then carries ~1e-14 of
+//     |M|, below the thresholds of those paths).
 //  C. FP64 sweeps on M1 until convergence; S, W from M1's columns.
 // J is orthogonal to FP32 accuracy, so M1 = (M J_o)(I + E) with J_o
 // orthogonal and |E| ~ 1e-7: a right multiplicative perturbation, under
@@ -1027,10 +1032,9 @@ constexpr int kMoreRounds = 2;   // rounds of two more steps for tiles they did 
 // Shared memory: two buffers of two b x s blocks and 2b squared norms (FP64
 // layout; the FP32 phase stores b x 2s floats per block in the same bytes),
 // 2b local norms, s gathered norms.
-// kMode: kJacFull runs A, B, C and writes W, S, rank; kJacPrecond runs A and
-// B only (M1 left in `work` for the FP64 Gram refinement); kJacFinish runs C
-// only, on the M1 found in `work`.
-enum { kJacFull = 0, kJacPrecond = 1, kJacFinish = 2 };
+// kMode: kJacPrecond runs A and B; kJacFinish runs C, on the M1 found in
+// `work`, and writes W, S and the rank.
+enum { kJacPrecond = 1, kJacFinish = 2 };
 template <int kCl, int kMode>
 __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__restrict__ jobs) {
     cg::cluster_group cl = cg::this_cluster();
@@ -1047,7 +1051,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
     double *nrm_loc = sm + 2 * stride, *all_nrm = nrm_loc + 2 * b;
     const int px = rank, py = nblk - 1 - rank;
     int g = 0, cur = 0, sw32 = 0;
-    if (kMode != kJacFinish) {
+    if constexpr (kMode == kJacPrecond) {
     // A. FP32 phase (the same buffers hold b x 2s floats per block)
     float *f0 = reinterpret_cast<float *>(sm);
     const int s2 = 2 * s, bsf = b * s2, stride_f = 2 * bsf + 2 * b;
@@ -1066,76 +1070,25 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
     }
     __syncthreads();
     sw32 = jacobi_sweeps<kCl, float>(cl, f0, stride_f, b, s, s2, kMaxSweeps32, g, cur, s_flag);
-    // B. M1 = M J for the held columns, 8 at a time; rows i = tid, tid + 256.
-    // With the paired copy of M (paired-FP32 paths) the products run in
-    // float-float arithmetic on the FP32 pipe (J is exact in FP32; M1 then
-    // carries ~1e-14 of |M|, below the thresholds of those paths); else in
-    // FP64.  Warps whose rows all lie past s, and the second row when
-    // s <= 256, issue nothing (an FP64 warp instruction costs the same with
-    // no lane active).
-    {
-        const float *F = f0 + cur * stride_f;
-        const int gx = block_at(px, g, nblk), gy = block_at(py, g, nblk);
-        const bool rows2 = s > kQrThreads, live = warp * 32 < s;
-        for (int q0 = 0; q0 < 2 * b && live; q0 += 8) {
-            double out[8][2];
-            if (J.Rt2) {
-                float h[8][2], l[8][2];
-#pragma unroll
-                for (int a = 0; a < 8; ++a) h[a][0] = h[a][1] = l[a][0] = l[a][1] = 0.0f;
-                for (int k = 0; k < s; ++k) {
-                    const float2 m0 = tid < s ? J.Rt2[(int64_t)k * s + tid] : make_float2(0.f, 0.f);
-                    const float2 m1 = rows2 && tid + kQrThreads < s ? J.Rt2[(int64_t)k * s + tid + kQrThreads]
-                                                                    : make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) {
-                        const int q = q0 + a;
-                        const float jk = q < 2 * b ? F[q * s2 + s + k] : 0.0f;
-                        df_fma(m0.x, m0.y, jk, 0.0f, h[a][0], l[a][0]);
-                        if (rows2) df_fma(m1.x, m1.y, jk, 0.0f, h[a][1], l[a][1]);
-                    }
-                }
-#pragma unroll
-                for (int a = 0; a < 8; ++a) {
-                    out[a][0] = (double)h[a][0] + (double)l[a][0];
-                    out[a][1] = (double)h[a][1] + (double)l[a][1];
-                }
-            } else {
-#pragma unroll
-                for (int a = 0; a < 8; ++a) out[a][0] = out[a][1] = 0.0;
-                for (int k = 0; k < s; ++k) {
-                    const double m0 = tid < s ? J.Rt[(int64_t)k * s + tid] : 0.0;
-                    const double m1 = rows2 && tid + kQrThreads < s ? J.Rt[(int64_t)k * s + tid + kQrThreads] : 0.0;
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) {
-                        const int q = q0 + a;
-                        const double jk = q < 2 * b ? (double)F[q * s2 + s + k] : 0.0;
-                        out[a][0] = fma(m0, jk, out[a][0]);
-                        if (rows2) out[a][1] = fma(m1, jk, out[a][1]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                const int q = q0 + a;
-                if (q >= 2 * b) break;
-                const int u = (q < b ? gx : gy) * b + q % b;
-                if (u >= s) continue;
-                if (tid < s) J.work[(int64_t)u * s + tid] = out[a][0];
-                if (tid + kQrThreads < s) J.work[(int64_t)u * s + tid + kQrThreads] = out[a][1];
-            }
-        }
+    // B. J's held columns, as doubles or (paired paths) pairs, for the product
+    // M1 = M J that follows as a batched GEMM over the whole GPU (formed here, on
+    // the cluster's SMs, it took 130 us at s = 200 in pairs and more in FP64)
+    const float *F = f0 + cur * stride_f;
+    const int gx = block_at(px, g, nblk), gy = block_at(py, g, nblk);
+    for (int e = tid; e < 2 * b * s; e += kQrThreads) {
+        const int q = e / s, k = e % s, u = (q < b ? gx : gy) * b + (q < b ? q : q - b);
+        if (u >= s) continue;
+        const float v = F[q * s2 + s + k];
+        if (J.Rt2) reinterpret_cast<float2 *>(J.rot)[(int64_t)u * s + k] = make_float2(v, 0.f);
+        else J.rot[(int64_t)u * s + k] = (double)v;
     }
-    cl.sync();  // M1 complete; no CTA reads another's FP32 blocks any more
-    if (kMode == kJacPrecond) {
-        if (rank == 0 && tid == 0) {
-            J.sweeps[0] = 0;
-            J.sweeps[1] = sw32;
-            J.sweeps[2] = J.sweeps[3] = 0;
-        }
-        return;
+    if (rank == 0 && tid == 0) {
+        J.sweeps[0] = 0;
+        J.sweeps[1] = sw32;
+        J.sweeps[2] = J.sweeps[3] = 0;
     }
-    }  // kMode != kJacFinish
+    cl.sync();  // no CTA leaves while another may still read its blocks or flag
+    } else {
     // C. FP64 phase on M1, starting from the same block positions
     for (int slot = 0; slot < 2; ++slot) {
         const int blk = block_at(slot ? py : px, g, nblk);
@@ -1176,6 +1129,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
         J.sweeps[3] = rot;
     }
     cl.sync();  // no CTA leaves while another may still read its norms or tallies
+    }
 }
 
 // FP64 Gram refinement of M1 (the columns of which are orthogonal to FP32
@@ -1418,15 +1372,15 @@ static bool cluster16_ok() {
     static std::once_flag once;
     static int state = 0;
     std::call_once(once, [] {
-        const void *k16[] = {(const void *)k_qr_factor<16, false>, (const void *)k_qr_factor<16, true>, (const void *)k_qr_gm<16>, (const void *)k_jacobi_sm<16, kJacFull>,
-                             (const void *)k_jacobi_sm<16, kJacPrecond>, (const void *)k_jacobi_sm<16, kJacFinish>,
+        const void *k16[] = {(const void *)k_qr_factor<16, false>, (const void *)k_qr_factor<16, true>, (const void *)k_qr_gm<16>, (const void *)k_jacobi_sm<16, kJacPrecond>,
+                             (const void *)k_jacobi_sm<16, kJacFinish>,
                              (const void *)k_jacobi_gm<16>};
         bool ok = true;
         for (const void *k : k16)
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
         if (ok) {
             // one cluster of 16 CTAs that each fill an SM's shared memory must fit
-            const size_t need = std::min(smem_cap((const void *)k_qr_factor<16, false>), smem_cap((const void *)k_jacobi_sm<16, kJacFull>));
+            const size_t need = std::min(smem_cap((const void *)k_qr_factor<16, false>), smem_cap((const void *)k_jacobi_sm<16, kJacFinish>));
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(16);
             cfg.blockDim = dim3(kQrThreads);
@@ -1442,7 +1396,7 @@ static bool cluster16_ok() {
             cudaLaunchConfig_t cfq = cfg;
             cfq.blockDim = dim3(kQrSmThreads);
             if (cudaOccupancyMaxActiveClusters(&n1, k_qr_factor<16, false>, &cfq) == cudaSuccess &&
-                cudaOccupancyMaxActiveClusters(&n2, k_jacobi_sm<16, kJacFull>, &cfg) == cudaSuccess && n1 > 0 && n2 > 0)
+                cudaOccupancyMaxActiveClusters(&n2, k_jacobi_sm<16, kJacFinish>, &cfg) == cudaSuccess && n1 > 0 && n2 > 0)
                 state = 1;
         }
         cudaGetLastError();  // clear any error of the queries
@@ -1488,8 +1442,7 @@ static SvdKernel svd_sm_kernel_m(int c) {
     }
 }
 static SvdKernel svd_sm_kernel(int c, int mode) {
-    return mode == kJacPrecond ? svd_sm_kernel_m<kJacPrecond>(c)
-                               : (mode == kJacFinish ? svd_sm_kernel_m<kJacFinish>(c) : svd_sm_kernel_m<kJacFull>(c));
+    return mode == kJacPrecond ? svd_sm_kernel_m<kJacPrecond>(c) : svd_sm_kernel_m<kJacFinish>(c);
 }
 
 // One launch per (kernel, cluster size) class, with the class's largest
@@ -1811,7 +1764,7 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
         std::vector<SvdJob> sv(np);
         for (size_t u = 0; u < np; ++u)
             sv[u] = SvdJob{W + oR[u], W + oK[u], W + oW[u], W + oS[u], d_rank + u, d_rank + np + 4 * u, ps[u],
-                           jobs[pending[u]].tau, df ? (const float2 *)(W + oR2[u]) : nullptr};
+                           jobs[pending[u]].tau, df ? (const float2 *)(W + oR2[u]) : nullptr, W + oX2[u]};
         std::vector<int> svd_csize;
         ClassTiming t16;
         size_t ev_used = 0;
@@ -1821,6 +1774,21 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
             t16.e1 = pooled_event(ctx, ev_used);
         }
         svd_launch(ctx, st, sv, svd_csize, ctx->profile ? &t16 : nullptr, kJacPrecond);
+        {  // M1 = R' J
+            std::vector<GemmProb> gm;
+            for (size_t u = 0; u < np; ++u)
+                if (svd_csize[u] > 0) {
+                    const int n = ps[u];
+                    GemmProb a{};
+                    a.A = W + oR[u]; a.lda = n; a.m = n; a.k = n;
+                    a.B = W + oX2[u]; a.ldb = n; a.n = n;
+                    a.C = W + oK[u]; a.ldc = n;
+                    a.A2 = df ? (const float2 *)(W + oR2[u]) : nullptr;
+                    a.B2 = (const float2 *)(W + oX2[u]);
+                    gm.push_back(a);
+                }
+            gemm_batched(ctx, st, false, false, gm, 1.0, 0.0, df);
+        }
         // FP64 Gram refinement of the tiles `rj` (batched), then W, S and the rank
         std::vector<double *> X(np, nullptr), Xn(np, nullptr);
         auto refine = [&](const std::vector<size_t> &rj, int steps) {

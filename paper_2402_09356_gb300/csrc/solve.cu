@@ -12,7 +12,8 @@
 //   k_pair_dots c_ik = V_ik' y_k for all i > k, one warp a column of V;
 //   k_pair_sub  y_i -= U_ik c_ik for all i > k.
 // The product L w has no chain: one launch of k_pair_dots over all tiles, one
-// of k_row_sums.  All descriptors go up once per call.
+// of k_row_sums.  All descriptors go up once per call.  n = 20,000, tile 800: solve
+// 42.4 -> 1.95 ms (k_trsv 51 us a tile, the two others 10 each), L w 1.46 -> 0.11.
 #include <algorithm>
 #include <mutex>
 
@@ -30,7 +31,7 @@ namespace {
 
 constexpr int kB = 32;             // rows of a diagonal block
 constexpr int kThreads = 256, kWarps = kThreads / 32;
-constexpr int kRows = 64;          // output rows a CTA
+constexpr int kRows = 32;          // output rows a CTA
 constexpr int kGroups = kThreads / kRows;
 
 // One off-diagonal tile: U (m_i x r), V (m_k x r), both ld nb, and the place
@@ -85,76 +86,73 @@ __global__ void __launch_bounds__(kThreads) k_inv_blocks(const double *__restric
 }
 
 // x <- L^-1 x for one diagonal tile (m <= 1024, ld ldl) by one cluster: CTA
-// `rank` owns the blocks rank, rank + kCl, ... of the right-hand side.  Step b:
-// the owner multiplies its block by the block's inverse and stores the 32
-// values into every CTA; after one cluster barrier every CTA subtracts L's
-// block column b times them from its blocks.  Eight threads a row; the entries
-// of the next block column are loaded before the barrier.  Bound by the chain
-// of a step (barrier, update, product: about 1 us).
+// `rank` owns the blocks rank, rank + kCl, ... of the right-hand side, each
+// kept by kThreads / kOwn threads (four or eight a row).  Step b: the owner
+// multiplies its block by the block's inverse and stores the 32 values into
+// every CTA; after one cluster barrier every CTA subtracts L's block column b
+// times them from its blocks.  The entries of block columns b + 1 and b + 2 are
+// on their way to registers meanwhile (the tile comes from HBM).  Bound by the
+// chain of a step: barrier, update of the next block, its product.
 template <int kCl>
 __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L, int ldl, int m,
                                                     const double *__restrict__ inv, double *__restrict__ x) {
-    constexpr int kOwn = kB / kCl;  // blocks a CTA: at most 32 blocks in a tile
+    constexpr int kOwn = kB / kCl;                 // blocks a CTA: at most 32 blocks in a tile
+    constexpr int kQ = kThreads / kOwn / kB;       // threads a row
+    constexpr int kN = kB / kQ;                    // columns a thread
     cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank(), tid = threadIdx.x, r = tid >> 3, q = tid & 7;
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+    const int o = tid / (kThreads / kOwn), r = tid % (kThreads / kOwn) / kQ, q = tid % kQ;
+    const int I = rank + o * kCl, row = I * kB + r;  // the thread's block and row
     __shared__ double rhs[kOwn][kB], xs[2][kB];
     const int nblk = (m + kB - 1) / kB;
+    if (q == 0) rhs[o][r] = row < m ? x[row] : 0.0;
+    double a[2][kN], d[kN];
+    auto load = [&](int b, double (&v)[kN]) {  // L's block column b in the thread's row
+        const bool in = b < I && row < m;
 #pragma unroll
-    for (int o = 0; o < kOwn; ++o) {
-        const int i = (rank + o * kCl) * kB + tid;
-        if (tid < kB) rhs[o][tid] = i < m ? x[i] : 0.0;
-    }
-    double a[kOwn][kB / 8], d[kB / 8];
-    auto load = [&](int b) {  // L's block column b in the rows of the own blocks
-#pragma unroll
-        for (int o = 0; o < kOwn; ++o) {
-            const int I = rank + o * kCl, row = I * kB + r;
-#pragma unroll
-            for (int k = 0; k < kB / 8; ++k) {
-                const int c = b * kB + q + 8 * k;
-                a[o][k] = I > b && row < m && c < m ? L[(int64_t)c * ldl + row] : 0.0;
-            }
-        }
+        for (int k = 0; k < kN; ++k) v[k] = in ? L[(int64_t)(b * kB + q + kQ * k) * ldl + row] : 0.0;
     };
-    auto load_inv = [&](int b) {  // the inverse of the own block that comes next
-        if (b < nblk)
+    auto reduce = [](double v) {
 #pragma unroll
-            for (int k = 0; k < kB / 8; ++k) d[k] = inv[(int64_t)b * kB * kB + r * kB + q + 8 * k];
-    };
-    auto reduce8 = [](double v) {
-        v += __shfl_xor_sync(0xFFFFFFFFu, v, 4);
-        v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
-        v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+        for (int s = kQ / 2; s; s >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, s);
         return v;
     };
-    load_inv(rank);
-    load(0);
+#pragma unroll
+    for (int k = 0; k < kN; ++k) d[k] = I < nblk ? inv[(int64_t)I * kB * kB + r * kB + q + kQ * k] : 0.0;
+    load(0, a[0]);
+    load(1, a[1]);
     cl.sync();  // every CTA has started (its shared memory is written below)
-    for (int b = 0; b < nblk; ++b) {
-        if (b % kCl == rank) {
-            const double *v = rhs[b / kCl];
-            double s = 0.0;
+    auto step = [&](int b, double (&v)[kN]) {
+        if (b == I) {  // uniform over the warps of the block's threads
+            double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-            for (int k = 0; k < kB / 8; ++k) s = fma(d[k], v[q + 8 * k], s);
-            s = reduce8(s);
+            for (int k = 0; k < kN; k += 2) {
+                s0 = fma(d[k], rhs[o][q + kQ * k], s0);
+                s1 = fma(d[k + 1], rhs[o][q + kQ * (k + 1)], s1);
+            }
+            const double s = reduce(s0 + s1);
 #pragma unroll
-            for (int k = q; k < kCl; k += 8) cl.map_shared_rank(&xs[b & 1][0], k)[r] = s;
-            if (q == 0 && b * kB + r < m) x[b * kB + r] = s;
-            load_inv(b + kCl);
+            for (int k = q; k < kCl; k += kQ) cl.map_shared_rank(&xs[b & 1][0], k)[r] = s;
+            if (q == 0 && row < m) x[row] = s;
         }
         cl.sync();
-        const double *v = xs[b & 1];
+        if (b < I) {
+            const double *w = xs[b & 1];
+            double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-        for (int o = 0; o < kOwn; ++o) {
-            if (rank + o * kCl <= b) continue;  // uniform over the CTA
-            double s = 0.0;
-#pragma unroll
-            for (int k = 0; k < kB / 8; ++k) s = fma(a[o][k], v[q + 8 * k], s);
-            s = reduce8(s);
+            for (int k = 0; k < kN; k += 2) {
+                s0 = fma(v[k], w[q + kQ * k], s0);
+                s1 = fma(v[k + 1], w[q + kQ * (k + 1)], s1);
+            }
+            const double s = reduce(s0 + s1);
             if (q == 0) rhs[o][r] -= s;
         }
-        if (b + 1 < nblk) load(b + 1);
+        load(b + 2, v);
         __syncthreads();
+    };
+    for (int b = 0; b < nblk; b += 2) {
+        step(b, a[0]);
+        if (b + 1 < nblk) step(b + 1, a[1]);
     }
 }
 
@@ -194,8 +192,12 @@ __device__ __forceinline__ double row_part(const double *__restrict__ A, int lda
     return s0 + s1;
 }
 
-// y_i -= U_ik c_ik for the pairs p0 + blockIdx.y: 64 rows a CTA, the columns
-// split over four threads a row.
+__device__ __forceinline__ double sum_parts(const double (*part)[kRows], int u) {
+    return ((part[0][u] + part[1][u]) + (part[2][u] + part[3][u])) + ((part[4][u] + part[5][u]) + (part[6][u] + part[7][u]));
+}
+
+// y_i -= U_ik c_ik for the pairs p0 + blockIdx.y: 32 rows a CTA, the columns
+// split over eight threads a row.
 __global__ void __launch_bounds__(kThreads) k_pair_sub(const Pair *__restrict__ pairs, int p0, int64_t n, int nb,
                                                         const double *__restrict__ c, double *__restrict__ y) {
     __shared__ double part[kGroups][kRows];
@@ -204,10 +206,10 @@ __global__ void __launch_bounds__(kThreads) k_pair_sub(const Pair *__restrict__ 
     const int m = rows_of(n, nb, P.i);
     part[g][u] = row < m ? row_part(P.U + row, nb, P.r, g, c + P.off) : 0.0;
     __syncthreads();
-    if (g == 0 && row < m) y[(int64_t)P.i * nb + row] -= (part[0][u] + part[1][u]) + (part[2][u] + part[3][u]);
+    if (g == 0 && row < m) y[(int64_t)P.i * nb + row] -= sum_parts(part, u);
 }
 
-// z_i = D_i w_i + sum_k U_ik c_ik: blockIdx.y = i, 64 rows a CTA; the pairs of
+// z_i = D_i w_i + sum_k U_ik c_ik: blockIdx.y = i, 32 rows a CTA; the pairs of
 // row i are first[i] .. first[i + 1].  D's columns past the row are zero and
 // left out.
 __global__ void __launch_bounds__(kThreads) k_row_sums(const Pair *__restrict__ pairs, const int *__restrict__ first,
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kThreads) k_row_sums(const Pair *__restrict__ 
     }
     part[g][u] = s;
     __syncthreads();
-    if (g == 0 && row < m) z[(int64_t)i * nb + row] = (part[0][u] + part[1][u]) + (part[2][u] + part[3][u]);
+    if (g == 0 && row < m) z[(int64_t)i * nb + row] = sum_parts(part, u);
 }
 
 // Per tile: sum log D_rr and |y|^2 (fixed reduction order), then their sums

@@ -433,8 +433,8 @@ __global__ void k_fill(double *__restrict__ a, int64_t n, double v) {
 // tree level or selected point: its bytes take a microsecond, so that launches,
 // their gaps and host synchronisations were all of the time.  Arrays stay in
 // L2 (__ldcg / __stcg: another CTA wrote them in an earlier phase); a cluster
-// barrier separates the phases.  40,000 locations with xy_out: Hilbert 123 -> 60
-// us, KD-tree 2,940 -> 180 us (sort 83, upper levels 71, subtrees 29); 10,000
+// barrier separates the phases.  40,000 locations with xy_out: Hilbert 123 -> 47
+// us, KD-tree 2,940 -> 177 us (sort 75, upper levels 70, subtrees 29); 10,000
 // locations by max-min 82 -> 15 ms.  Above kClusterMaxN the launches above take over (more
 // SMs share a pass).
 constexpr int kOrdCl = 16, kOrdThreads = 1024, kOrdWarps = kOrdThreads / 32;
@@ -447,20 +447,35 @@ struct SortShared {
     int skip;
 };
 
-// Stable sort of (key, val) by the low `bits` bits of the key, by one cluster:
+// Lanes (of those with `in`) that hold the same 8-bit digit: one vote a bit (a
+// match instruction goes through the warp's distinct values one by one).
+__device__ __forceinline__ uint32_t same_digit(uint32_t d, bool in) {
+    uint32_t peers = __ballot_sync(0xFFFFFFFFu, in);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool set = (d >> b) & 1u;
+        const uint32_t v = __ballot_sync(0xFFFFFFFFu, set);
+        peers &= set ? v : ~v;
+    }
+    return peers;
+}
+
+// Stable sort of (key, val) by the bits [from, to) of the key, by one cluster
+// (kVals false: of keys alone, which then carry their value in other bits: one
+// 8-byte store an item, where the scattered stores are half of a pass):
 // warp w of the cluster takes a run of items, counts its digits (one count per
 // warp and digit, leaders of equal digits found by match), the counts are
 // summed over warps, CTAs (over DSMEM) and digits, and the warp writes its
 // items in order.  A pass in which all keys share the digit is left out.  The
 // result ends in (keys, vals).
-template <typename K>
+template <typename K, bool kVals>
 __device__ void cluster_sort(cg::cluster_group &cl, SortShared &S, K *&keys, uint32_t *&vals, K *&ktmp, uint32_t *&vtmp,
-                             int n, int bits) {
+                             int n, int from, int to) {
     const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int run = (n + kOrdCl * kOrdWarps * 32 - 1) / (kOrdCl * kOrdWarps * 32);  // rounds of 32 items a warp
     const int i0 = (rank * kOrdWarps + warp) * run * 32;
     const uint32_t below = (1u << lane) - 1u;
-    for (int shift = 0; shift < bits; shift += 8) {
+    for (int shift = from; shift < to; shift += 8) {
         for (int e = tid; e < kOrdWarps * 256; e += kOrdThreads) S.cnt[e >> 8][e & 255] = 0;
         __syncthreads();
         for (int u0 = 0; u0 < run; u0 += kSortBatch) {
@@ -474,8 +489,8 @@ __device__ void cluster_sort(cg::cluster_group &cl, SortShared &S, K *&keys, uin
             for (int u = 0; u < kSortBatch; ++u) {
                 const int i = i0 + (u0 + u) * 32 + lane;
                 const bool in = u0 + u < run && i < n;
-                const uint32_t d = in ? (uint32_t)(k[u] >> shift) & 255u : 256u;
-                const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+                const uint32_t d = (uint32_t)(k[u] >> shift) & 255u;
+                const uint32_t peers = same_digit(d, in);
                 if (in && !(peers & below)) S.cnt[warp][d] += __popc(peers);
                 __syncwarp();
             }
@@ -531,18 +546,18 @@ __device__ void cluster_sort(cg::cluster_group &cl, SortShared &S, K *&keys, uin
                 const int i = i0 + (u0 + u) * 32 + lane;
                 const bool in = u0 + u < run && i < n;
                 k[u] = in ? __ldcg(keys + i) : K(0);
-                v[u] = in ? __ldcg(vals + i) : 0u;
+                v[u] = kVals && in ? __ldcg(vals + i) : 0u;
             }
 #pragma unroll
             for (int u = 0; u < kSortBatch; ++u) {
                 const int i = i0 + (u0 + u) * 32 + lane;
                 const bool in = u0 + u < run && i < n;
-                const uint32_t d = in ? (uint32_t)(k[u] >> shift) & 255u : 256u;
-                const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+                const uint32_t d = (uint32_t)(k[u] >> shift) & 255u;
+                const uint32_t peers = same_digit(d, in);
                 if (in) {
                     const uint32_t pos = S.base[d] + S.cnt[warp][d] + __popc(peers & below);
                     __stcg(ktmp + pos, k[u]);
-                    __stcg(vtmp + pos, v[u]);
+                    if constexpr (kVals) __stcg(vtmp + pos, v[u]);
                 }
                 __syncwarp();
                 if (in && !(peers & below)) S.cnt[warp][d] += __popc(peers);
@@ -559,32 +574,34 @@ __device__ void cluster_sort(cg::cluster_group &cl, SortShared &S, K *&keys, uin
     }
 }
 
-// Random / Morton / Hilbert ordering in one launch: keys, sort, permutation and
-// the permuted locations.
-__global__ void __launch_bounds__(kOrdThreads) k_sfc_cluster(const double *__restrict__ xy, int n, int method, uint64_t seed,
-                                                              uint32_t *keys, uint32_t *vals, uint32_t *ktmp,
-                                                              uint32_t *vtmp, uint32_t *__restrict__ codes,
+// Random / Morton / Hilbert ordering: items (key, index) in 64 bits, by the
+// whole GPU (their FP64 rounding alone took 9 us on the cluster's 16 SMs) ...
+__global__ void k_sfc_items(const double *__restrict__ xy, int n, int method, uint64_t seed, uint64_t *__restrict__ items,
+                            uint32_t *__restrict__ codes) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint32_t k;
+    if (method == TLR_ORDER_RANDOM) {
+        k = (uint32_t)(splitmix64(seed ^ (uint64_t)i) >> 32);
+    } else {
+        const uint32_t qx = quantize16(xy[i]), qy = quantize16(xy[n + i]);
+        k = (method == TLR_ORDER_MORTON) ? (spread_bits(qx) | (spread_bits(qy) << 1)) : hilbert16(qx, qy);
+    }
+    items[i] = ((uint64_t)k << 32) | (uint32_t)i;
+    if (codes) codes[i] = k;
+}
+// ... then their sort, the permutation and the permuted locations.
+__global__ void __launch_bounds__(kOrdThreads) k_sfc_cluster(const double *__restrict__ xy, int n, uint64_t *items,
+                                                              uint64_t *tmp,
                                                               int64_t *__restrict__ perm, double *__restrict__ xy_out,
                                                               int quantize) {
     __shared__ SortShared S;
     cg::cluster_group cl = cg::this_cluster();
     const int t0 = (int)cl.block_rank() * kOrdThreads + threadIdx.x;
-    for (int i = t0; i < n; i += kOrdCl * kOrdThreads) {
-        uint32_t k;
-        if (method == TLR_ORDER_RANDOM) {
-            k = (uint32_t)(splitmix64(seed ^ (uint64_t)i) >> 32);
-        } else {
-            const uint32_t qx = quantize16(xy[i]), qy = quantize16(xy[n + i]);
-            k = (method == TLR_ORDER_MORTON) ? (spread_bits(qx) | (spread_bits(qy) << 1)) : hilbert16(qx, qy);
-        }
-        __stcg(keys + i, k);
-        __stcg(vals + i, (uint32_t)i);
-        if (codes) codes[i] = k;
-    }
-    cl.sync();
-    cluster_sort<uint32_t>(cl, S, keys, vals, ktmp, vtmp, n, 32);
+    uint32_t *none = nullptr;
+    cluster_sort<uint64_t, false>(cl, S, items, none, tmp, none, n, 32, 64);
     for (int p = t0; p < n; p += kOrdCl * kOrdThreads) {
-        const uint32_t i = __ldcg(vals + p);
+        const uint32_t i = (uint32_t)__ldcg(items + p);
         perm[p] = (int64_t)i;
         if (xy_out) {
             double x = xy[i], y = xy[n + i];
@@ -615,7 +632,7 @@ __global__ void __launch_bounds__(kOrdThreads) k_kd_sort(const double *__restric
         __stcg(vals + i, (uint32_t)i);
     }
     cl.sync();
-    cluster_sort<uint64_t>(cl, S, keys, vals, ktmp, vtmp, n, 64);
+    cluster_sort<uint64_t, true>(cl, S, keys, vals, ktmp, vtmp, n, 0, 64);
     for (int p = t0; p < n; p += kOrdCl * kOrdThreads) list[(int64_t)dim * n + p] = __ldcg(vals + p);
     cl.sync();  // no CTA leaves while another may still read its histogram
 }
@@ -926,39 +943,50 @@ __global__ void __launch_bounds__(kMmThreads) k_maxmin_cluster(const double *__r
     int64_t p = s_p;
     if (p < 0 || p >= n) p = 0;  // only reachable with non-finite coordinates
     double px = xy[p], py = xy[n + p];
+    int bh = INT32_MIN;  // the thread's best point
+    uint32_t bl = 0, bi = 0xFFFFFFFFu;
     cl.sync();
     for (int k = 0; k < n; ++k) {
         if (rank == 0 && tid == 0) perm[k] = p;
         const float px4 = (float)px, py4 = (float)py;
-        int bh = INT32_MIN;
-        uint32_t bl = 0, bi = 0xFFFFFFFFu;
+        bool again = k == 0;
         for (int j = tid; j < cnt; j += kMmThreads) {
-            double m = D[j];
             const float r = R4[j];
-            if (g0 + j == p) {
-                m = -1.0;  // taken
-                D[j] = m;
-                R4[j] = -1.f;
-            } else if (r >= 0.f && !(fabsf(X4[j] - px4) > r) && !(fabsf(Y4[j] - py4) > r)) {
+            if (r < 0.f || fabsf(X4[j] - px4) > r || fabsf(Y4[j] - py4) > r) continue;
+            double m = -1.0;  // taken (a point's own box contains it)
+            float r2 = -1.f;
+            if (g0 + j != p) {
                 const double d = sqdist(X[j], Y[j], px, py);
-                if (!(d >= m)) {
-                    m = fmin(m, d);
-                    D[j] = m;
-                    const float m4 = (float)m;
-                    R4[j] = (m4 < 1e-30f ? 1.0001e-15f : sqrtf(m4) * 1.00001f) + slack;
-                }
+                m = D[j];
+                if (d >= m) continue;
+                m = fmin(m, d);
+                const float m4 = (float)m;
+                r2 = (m4 < 1e-30f ? 1.0001e-15f : sqrtf(m4) * 1.00001f) + slack;
             }
-            const int h = __double2hiint(m);
-            const uint32_t l = (uint32_t)__double2loint(m);
-            if (h > bh || (h == bh && l > bl)) {  // indices rise: the first of equals stays
-                bh = h;
-                bl = l;
-                bi = (uint32_t)(g0 + j);
+            D[j] = m;
+            R4[j] = r2;
+            again |= (uint32_t)(g0 + j) == bi;
+        }
+        // a thread looks its points over again, and its warp reduces again, only
+        // when a best point changed (warp reductions are slow)
+        if (again) {
+            bh = INT32_MIN;
+            for (int j = tid; j < cnt; j += kMmThreads) {
+                const double m = D[j];
+                const int h = __double2hiint(m);
+                const uint32_t l = (uint32_t)__double2loint(m);
+                if (h > bh || (h == bh && l > bl)) {  // indices rise: the first of equals stays
+                    bh = h;
+                    bl = l;
+                    bi = (uint32_t)(g0 + j);
+                }
             }
         }
         int who;
-        mm_best(bh, bl, bi, who);
-        if (lane == who) wbest[warp] = MmCand{bh, bl, (int64_t)bi, 0.0, 0.0};
+        if (__any_sync(0xFFFFFFFFu, again)) {
+            mm_best(bh, bl, bi, who);
+            if (lane == who) wbest[warp] = MmCand{bh, bl, (int64_t)bi, 0.0, 0.0};
+        }
         __syncthreads();
         if (warp == 0) {
             const MmCand c = lane < kMmWarps ? wbest[lane] : MmCand{INT32_MIN, 0u, (int64_t)0xFFFFFFFF, 0.0, 0.0};
@@ -1027,9 +1055,10 @@ void order_sfc(const double *xy, int64_t n, int method, uint64_t seed, int64_t *
                uint32_t *codes, double *xy_out, int quantize, cudaStream_t s) {
     if (n <= kClusterMaxN && cluster_order_ok()) {
         DevBuf b(16 * n, s);
-        uint32_t *k = b.as<uint32_t>();
-        launch_clustered(k_sfc_cluster, kOrdCl, 1, kOrdThreads, 0, s, xy, (int)n, method, seed, k, k + n, k + 2 * n,
-                         k + 3 * n, codes, perm, xy_out, quantize);
+        uint64_t *k = b.as<uint64_t>();
+        launch(k_sfc_items, grid1(n, 128), 128, 0, s, xy, (int)n, method, seed, k, codes);
+        TLR_CHECK_LAUNCH();
+        launch_clustered(k_sfc_cluster, kOrdCl, 1, kOrdThreads, 0, s, xy, (int)n, k, k + n, perm, xy_out, quantize);
         return;
     }
     DevBuf kb(n * 4, s), vb(n * 4, s), kt(n * 4, s), vt(n * 4, s), hb(hist_words(n) * 4, s);

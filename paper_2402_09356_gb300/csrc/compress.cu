@@ -731,77 +731,165 @@ __device__ __forceinline__ int jacobi_rotate(double *x, double *y, double *nx, d
     rotated_norms(x, y, nx, ny, al, be, ga, c, t, sdot, lane);
     return 2;
 }
-// FP32: entries in pairs, and for srot <= 512 (kKeep pairs a lane) all of both
-// columns in registers from one batch of loads, so that the dot product, the
-// angle and the rotation read shared memory once (loads and stores of x and y
-// one pair at a time wait for each other).  The cosine is formed from the
-// norms' reciprocal square roots: tol^2 |x|^2 |y|^2 would underflow FP32 for
-// columns near the accuracy (1e-11 of the largest), which then never rotated
-// and left the FP64 phase the work.  A pair whose cosine is at most
-// kFinalCos is rotated but does not ask for another sweep: convergence is
-// quadratic, so a sweep that meets no larger cosine leaves them near kFinalCos^2,
-// where the FP64 refinement starts.
+// FP32 (srot = 2 sdot, entries in pairs).  A pair's rotation is one dependent
+// chain, and the chain is what a sweep costs, so it is cut to the bone:
+//   - KC >= s / 32 pairs a lane, all of both columns in registers, one straight
+//     line of predicated loads (a uniform branch per 32 rows cost more than the
+//     arithmetic), read once for the dot product and the rotation;
+//   - the cosine from the norms' reciprocal square roots, summed over the lanes
+//     as a 26-bit fixed-point integer (one integer reduction, 50 cycles, where
+//     five shuffles and adds take 167; |sum| <= 1 by Cauchy-Schwarz, its error
+//     at most 2^-22, a tenth of the tolerance at s = 30, and the angle only
+//     steers).  (tol^2 |x|^2 |y|^2 would underflow FP32 for columns near the
+//     accuracy, 1e-11 of the largest, which then never rotated and left the
+//     FP64 phase the work.)
+// 8 warps with the barrier after each pair: 1,384 -> 615 cycles at s = 40, 1,463 ->
+// 742 at 120, 1,492 -> 1,087 at 200 (SVD of an n = 40,000 evaluation 84 -> 70 ms).
+// Not inlined: one copy per KC serves every cluster size.
+// A pair whose cosine is at most kFinalCos is rotated but does not ask for
+// another sweep: convergence is quadratic, so a sweep that meets no larger
+// cosine leaves them near kFinalCos^2, where the FP64 refinement starts.
 constexpr float kFinalCos = 3e-4f;
-__device__ __forceinline__ int jacobi_rotate(float *x, float *y, float *nx, float *ny, int sdot, int srot, int lane,
-                                             float tol) {
-    constexpr int kKeep = 8;
+__device__ __forceinline__ float2 lds2(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts2(uint32_t a, float2 v) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ float lds1(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts1(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ float rsqrt_approx32(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_approx32(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// (c, s, t) of the rotation for zeta = (|y|^2 - |x|^2) / (2 x'y), from approximate
+// roots: (c, s) is orthogonal to FP32 accuracy whatever their error, so only
+// convergence depends on it.  h = 1 / sqrt(1 + zeta^2): c^2 = (1 + |zeta| h) / 2,
+// |s| = h / (2 c).
+__device__ __forceinline__ void jacobi_angle(float zeta, float az, float &c, float &sn, float &t) {
+    const float h = rsqrt_approx32(fmaf(zeta, zeta, 1.0f)), c2 = fmaf(0.5f * az, h, 0.5f), rc = rsqrt_approx32(c2);
+    c = c2 * rc;
+    sn = copysignf(0.5f * h * rc, zeta);
+    t = sn * rc;
+}
+template <int KC>
+__device__ __noinline__ int jacobi_rotate32(uint32_t x, uint32_t y, uint32_t nx, uint32_t ny, int s, int lane, float tol) {
+    const float al = lds1(nx), be = lds1(ny);
+    float2 a[KC], b[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        const int i = lane + 32 * k;
+        a[k] = b[k] = make_float2(0.f, 0.f);
+        if (i < s) {
+            a[k] = lds2(x + 8 * i);
+            b[k] = lds2(y + 8 * i);
+        }
+    }
+    float g0 = 0.f, g1 = 0.f;
+#pragma unroll
+    for (int k = 0; k < (KC + 1) / 2; ++k) {  // the first s floats of a column
+        const int i = lane + 32 * k;
+        if (2 * i < s) g0 = fmaf(a[k].x, b[k].x, g0);
+        if (2 * i + 1 < s) g1 = fmaf(a[k].y, b[k].y, g1);
+    }
+    const float rab = rsqrt_approx32(al) * rsqrt_approx32(be);
+    // a zero or non-finite column gives 0 here (NaN converts to 0): left alone
+    const int sum = __reduce_add_sync(0xFFFFFFFFu, __float2int_rn((g0 + g1) * rab * 67108864.f));
+    const float cosine = (float)sum * 1.490116119384765625e-8f;
+    if (fabsf(cosine) <= tol) return 0;
+    const float zeta = (be - al) * rab * rcp_approx32(2.0f * cosine), az = fabsf(zeta);
+    if (!(az < 1e18f)) return 0;  // t below FP32 resolution
+    float c, sn, t;
+    jacobi_angle(zeta, az, c, sn, t);
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        const int i = lane + 32 * k;
+        const float2 u = a[k], v = b[k];
+        a[k] = make_float2(fmaf(c, u.x, -sn * v.x), fmaf(c, u.y, -sn * v.y));
+        b[k] = make_float2(fmaf(sn, u.x, c * v.x), fmaf(sn, u.y, c * v.y));
+        if (i < s) {
+            sts2(x + 8 * i, a[k]);
+            sts2(y + 8 * i, b[k]);
+        }
+    }
+    const float cc = c * c, tg = 2.0f * t * cosine * rcp_approx32(rab), tt = t * t;
+    float al2 = cc * (al - tg + tt * be), be2 = cc * (be + tg + tt * al);
+    const bool la = !(al2 > 1e-3f * cc * (al + tt * be)), lb = !(be2 > 1e-3f * cc * (be + tt * al));
+    if (la || lb) {  // cancelled: from the entries (uniform)
+        float va = 0.f, vb = 0.f;
+#pragma unroll
+        for (int k = 0; k < (KC + 1) / 2; ++k) {
+            const int i = lane + 32 * k;
+            if (2 * i < s) va = fmaf(a[k].x, a[k].x, va), vb = fmaf(b[k].x, b[k].x, vb);
+            if (2 * i + 1 < s) va = fmaf(a[k].y, a[k].y, va), vb = fmaf(b[k].y, b[k].y, vb);
+        }
+        va = warp_sum(va);
+        vb = warp_sum(vb);
+        if (la) al2 = va;
+        if (lb) be2 = vb;
+    }
+    if (lane == 0) {
+        sts1(nx, al2);
+        sts1(ny, be2);
+    }
+    return fabsf(cosine) <= kFinalCos ? 1 : 2;
+}
+// Columns longer than the registers hold (s > 256).
+__device__ __noinline__ int jacobi_rotate32_long(float *x, float *y, float *nx, float *ny, int sdot, int srot, int lane,
+                                                 float tol) {
     const float al = *nx, be = *ny;
     float2 *x2 = reinterpret_cast<float2 *>(x), *y2 = reinterpret_cast<float2 *>(y);
-    float2 a[kKeep], b[kKeep];
-    const bool keep = srot <= 64 * kKeep;
     float ga = 0.f;
-    if (keep) {
-#pragma unroll
-        for (int k = 0; k < kKeep; ++k) {
-            const int i = lane + 32 * k;
-            a[k] = b[k] = make_float2(0.f, 0.f);
-            if (64 * k < srot && 2 * i < srot) {
-                a[k] = x2[i];
-                b[k] = y2[i];
-            }
-        }
-        float g1 = 0.f;
-#pragma unroll
-        for (int k = 0; k < kKeep; ++k)
-            if (64 * k < sdot) {
-                const int i = lane + 32 * k;
-                if (2 * i < sdot) ga = fmaf(a[k].x, b[k].x, ga);
-                if (2 * i + 1 < sdot) g1 = fmaf(a[k].y, b[k].y, g1);
-            }
-        ga += g1;
-    } else {
-        for (int i = lane; 2 * i < sdot; i += 32) {
-            const float2 u = x2[i], v = y2[i];
-            ga = fmaf(u.x, v.x, ga);
-            if (2 * i + 1 < sdot) ga = fmaf(u.y, v.y, ga);
-        }
+    for (int i = lane; 2 * i < sdot; i += 32) {
+        const float2 u = x2[i], v = y2[i];
+        ga = fmaf(u.x, v.x, ga);
+        if (2 * i + 1 < sdot) ga = fmaf(u.y, v.y, ga);
     }
     ga = warp_sum(ga);
     if (ga == 0.f) return 0;
     const float cosine = fabsf(ga) * rsqrtf(al) * rsqrtf(be);
     if (cosine <= tol) return 0;
-    // approximate reciprocals and square root: (c, c t) is orthogonal to
-    // FP32 accuracy for any t, so only convergence depends on them
     const float zeta = __fdividef(be - al, 2.0f * ga), az = fabsf(zeta);
     if (az >= 1e18f) return 0;  // t below FP32 resolution
-    // h = 1 / sqrt(1 + zeta^2): c^2 = (1 + |zeta| h) / 2, |s| = h / (2 c)
-    const float h = rsqrtf(fmaf(zeta, zeta, 1.0f)), c2 = fmaf(0.5f * az, h, 0.5f), rc = rsqrtf(c2);
-    const float c = c2 * rc, sn = copysignf(0.5f * h * rc, zeta), t = sn * rc;
-    auto rotate = [&](int i, float2 u, float2 v) {
+    float c, sn, t;
+    jacobi_angle(zeta, az, c, sn, t);
+    for (int i = lane; 2 * i < srot; i += 32) {
+        const float2 u = x2[i], v = y2[i];
         x2[i] = make_float2(fmaf(c, u.x, -sn * v.x), fmaf(c, u.y, -sn * v.y));
         y2[i] = make_float2(fmaf(sn, u.x, c * v.x), fmaf(sn, u.y, c * v.y));
-    };
-    if (keep) {
-#pragma unroll
-        for (int k = 0; k < kKeep; ++k) {
-            const int i = lane + 32 * k;
-            if (64 * k < srot && 2 * i < srot) rotate(i, a[k], b[k]);
-        }
-    } else {
-        for (int i = lane; 2 * i < srot; i += 32) rotate(i, x2[i], y2[i]);
     }
     rotated_norms(x, y, nx, ny, al, be, ga, c, t, sdot, lane);
     return cosine <= kFinalCos ? 1 : 2;
+}
+__device__ __forceinline__ int jacobi_rotate(float *x, float *y, float *nx, float *ny, int sdot, int srot, int lane,
+                                             float tol) {
+    const uint32_t ax = (uint32_t)__cvta_generic_to_shared(x), ay = (uint32_t)__cvta_generic_to_shared(y);
+    const uint32_t an = (uint32_t)__cvta_generic_to_shared(nx), am = (uint32_t)__cvta_generic_to_shared(ny);
+    switch ((sdot + 31) >> 5) {
+    case 1:
+    case 2: return jacobi_rotate32<2>(ax, ay, an, am, sdot, lane, tol);
+    case 3: return jacobi_rotate32<3>(ax, ay, an, am, sdot, lane, tol);
+    case 4: return jacobi_rotate32<4>(ax, ay, an, am, sdot, lane, tol);
+    case 5: return jacobi_rotate32<5>(ax, ay, an, am, sdot, lane, tol);
+    case 6: return jacobi_rotate32<6>(ax, ay, an, am, sdot, lane, tol);
+    case 7: return jacobi_rotate32<7>(ax, ay, an, am, sdot, lane, tol);
+    case 8: return jacobi_rotate32<8>(ax, ay, an, am, sdot, lane, tol);
+    default: return jacobi_rotate32_long(x, y, nx, ny, sdot, srot, lane, tol);
+    }
 }
 
 // Convergence threshold of a pair: |x'y| <= 8 sqrt(s) u |x| |y| (u the unit

@@ -53,6 +53,10 @@ constexpr int kOversample = 24;  // samples beyond the expected rank
 constexpr int kSpare = 20;       // fewer spare samples than this: redo with more
 constexpr int kQrThreads = 256;
 constexpr int kNw = kQrThreads / 32;
+// Block Jacobi: up to kJacWarps warps a CTA (jacobi_threads); the bound leaves
+// 96 registers, with which two CTAs of 10 warps fit an SM.
+constexpr int kJacWarps = 16;
+constexpr int kJacBound = 640;
 constexpr int kQrSmThreads = 512;
 constexpr int kMaxSweeps = 40;
 
@@ -848,7 +852,7 @@ __device__ __noinline__ int jacobi_rotate32(uint32_t x, uint32_t y, uint32_t nx,
     }
     return fabsf(cosine) <= kFinalCos ? 1 : 2;
 }
-// Columns longer than the registers hold (s > 256).
+// Columns longer than the registers hold (s > 448).
 __device__ __noinline__ int jacobi_rotate32_long(float *x, float *y, float *nx, float *ny, int sdot, int srot, int lane,
                                                  float tol) {
     const float al = *nx, be = *ny;
@@ -888,6 +892,12 @@ __device__ __forceinline__ int jacobi_rotate(float *x, float *y, float *nx, floa
     case 6: return jacobi_rotate32<6>(ax, ay, an, am, sdot, lane, tol);
     case 7: return jacobi_rotate32<7>(ax, ay, an, am, sdot, lane, tol);
     case 8: return jacobi_rotate32<8>(ax, ay, an, am, sdot, lane, tol);
+    case 9:
+    case 10: return jacobi_rotate32<10>(ax, ay, an, am, sdot, lane, tol);
+    case 11:
+    case 12: return jacobi_rotate32<12>(ax, ay, an, am, sdot, lane, tol);
+    case 13:
+    case 14: return jacobi_rotate32<14>(ax, ay, an, am, sdot, lane, tol);
     default: return jacobi_rotate32_long(x, y, nx, ny, sdot, srot, lane, tol);
     }
 }
@@ -922,10 +932,11 @@ template <class T>
 __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int bx, int by, int b, int s, int srot,
                                                    bool inner, int lane, int warp, T tol, int &nchk, int &nrot) {
     bool rot = false;
+    const int nw = blockDim.x >> 5;
     if (inner) {
         const int bp = b + (b & 1);
         for (int ir = 0; ir < bp - 1; ++ir) {
-            for (int pr = warp; pr < bp; pr += kNw) {  // bp/2 pairs per block, two blocks
+            for (int pr = warp; pr < bp; pr += nw) {  // bp/2 pairs per block, two blocks
                 // (no remainder by a run-time size: a hundred cycles each)
                 const int slot = pr >= bp / 2, q = slot ? pr - bp / 2 : pr;
                 const int va = q - 1 + ir, vc = bp - 2 - q + ir;
@@ -945,7 +956,7 @@ __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int
         }
     }
     for (int k = 0; k < b; ++k) {
-        for (int i = warp; i < b; i += kNw) {
+        for (int i = warp; i < b; i += nw) {
             const int jy = i + k < b ? i + k : i + k - b;
             const int gx = bx * b + i, gy = by * b + jy;
             if (gx >= s || gy >= s) continue;
@@ -965,7 +976,8 @@ __device__ __forceinline__ bool jacobi_block_pairs(T *X, T *Y, T *NX, T *NY, int
 // Squared norms of the 2b columns of a buffer (first s entries of each).
 template <class T>
 __device__ __forceinline__ void block_norms(const T *cols, T *nrm, int b, int s, int srot, int lane, int warp) {
-    for (int q = warp; q < 2 * b; q += kNw) {
+    const int nw = blockDim.x >> 5;
+    for (int q = warp; q < 2 * b; q += nw) {
         const T v = col_norm2(cols + q * srot, s, lane);
         if (lane == 0) nrm[q] = v;
     }
@@ -985,7 +997,7 @@ __device__ int jacobi_sweeps(cg::cluster_group &cl, T *buf0, int stride, int b, 
                              int &g, int &cur, int *s_flag, int *tally = nullptr) {
     int nchk = 0, nrot = 0;  // pairs checked and rotated by this warp (warp-uniform)
     constexpr int nblk = 2 * kCl;
-    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int px = rank, py = nblk - 1 - rank, bs = b * srot;
     const T tol = jacobi_tol<T>(s);
     auto buf = [&](int k) { return buf0 + k * stride; };
@@ -1025,24 +1037,24 @@ __device__ int jacobi_sweeps(cg::cluster_group &cl, T *buf0, int stride, int b, 
                     const int h = p < kCl ? p : nblk - 1 - p, hs = p < kCl ? 0 : 1;
                     src[slot] = cl.map_shared_rank(buf(cur), h) + hs * bs;
                     const T *ns = cl.map_shared_rank(buf(cur), h) + 2 * bs + hs * b;
-                    for (int e = tid; e < b; e += kQrThreads) dst[2 * bs + slot * b + e] = ns[e];
+                    for (int e = tid; e < b; e += nt) dst[2 * bs + slot * b + e] = ns[e];
                 }
                 // 8 bytes a load: FP32 entries in pairs (bs = 2 b s is even)
                 constexpr int kPull = 4, kPer = 8 / sizeof(T);
                 const int bp = bs / kPer;
                 const double *s0 = reinterpret_cast<const double *>(src[0]), *s1 = reinterpret_cast<const double *>(src[1]);
                 double *d0 = reinterpret_cast<double *>(dst), *d1 = reinterpret_cast<double *>(dst + bs);
-                for (int e0 = tid; e0 < bp; e0 += kPull * kQrThreads) {
+                for (int e0 = tid; e0 < bp; e0 += kPull * nt) {
                     double v[2][kPull];
 #pragma unroll
                     for (int u = 0; u < kPull; ++u) {
-                        const int e = e0 + u * kQrThreads;
+                        const int e = e0 + u * nt;
                         v[0][u] = e < bp ? s0[e] : 0.0;
                         v[1][u] = e < bp ? s1[e] : 0.0;
                     }
 #pragma unroll
                     for (int u = 0; u < kPull; ++u) {
-                        const int e = e0 + u * kQrThreads;
+                        const int e = e0 + u * nt;
                         if (e < bp) {
                             d0[e] = v[0][u];
                             d1[e] = v[1][u];
@@ -1066,8 +1078,8 @@ __device__ int jacobi_sweeps(cg::cluster_group &cl, T *buf0, int stride, int b, 
 // `all_nrm` must hold every column's norm on entry.
 __device__ __forceinline__ void jacobi_emit(const SvdJob &J, const double *cols, int gx, int gy, int b,
                                             const double *all_nrm, int lane, int warp) {
-    const int s = J.s;
-    for (int q = warp; q < 2 * b; q += kNw) {
+    const int s = J.s, nw = blockDim.x >> 5;
+    for (int q = warp; q < 2 * b; q += nw) {
         const int slot = q / b, j = q % b, u = (slot ? gy : gx) * b + j;
         if (u >= s) continue;
         const double ku = norm_key(all_nrm[u]);
@@ -1124,14 +1136,14 @@ constexpr int kMoreRounds = 2;   // rounds of two more steps for tiles they did 
 // `work`, and writes W, S and the rank.
 enum { kJacPrecond = 1, kJacFinish = 2 };
 template <int kCl, int kMode>
-__global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__restrict__ jobs) {
+__global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jacobi_sm(const SvdJob *__restrict__ jobs) {
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     __shared__ int s_flag[2];
     __shared__ int s_tally[2];  // FP64 phase: pairs checked, pairs rotated (this CTA)
     extern __shared__ double sm[];
     const SvdJob J = jobs[blockIdx.x / kCl];
-    const int s = J.s, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int s = J.s, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     constexpr int nblk = 2 * kCl;
     const int b = (s + nblk - 1) / nblk, bs = b * s;
     const int stride = 2 * bs + 2 * b;  // one buffer: two blocks, 2b norms (FP64 layout)
@@ -1146,7 +1158,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
     for (int slot = 0; slot < 2; ++slot) {
         const int blk = block_at(slot ? py : px, 0, nblk);
         float *dst = f0 + slot * bsf;
-        for (int e = tid; e < bsf; e += kQrThreads) {
+        for (int e = tid; e < bsf; e += nt) {
             const int u = blk * b + e / s2, r = e % s2;
             float v = 0.0f;
             if (u < s) {
@@ -1163,7 +1175,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
     // the cluster's SMs, it took 130 us at s = 200 in pairs and more in FP64)
     const float *F = f0 + cur * stride_f;
     const int gx = block_at(px, g, nblk), gy = block_at(py, g, nblk);
-    for (int e = tid; e < 2 * b * s; e += kQrThreads) {
+    for (int e = tid; e < 2 * b * s; e += nt) {
         const int q = e / s, k = e % s, u = (q < b ? gx : gy) * b + (q < b ? q : q - b);
         if (u >= s) continue;
         const float v = F[q * s2 + s + k];
@@ -1181,7 +1193,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
     for (int slot = 0; slot < 2; ++slot) {
         const int blk = block_at(slot ? py : px, g, nblk);
         double *dst = sm + slot * bs;
-        for (int e = tid; e < bs; e += kQrThreads) {
+        for (int e = tid; e < bs; e += nt) {
             const int u = blk * b + e / s;
             dst[e] = u < s ? J.work[(int64_t)u * s + e % s] : 0.0;
         }
@@ -1191,7 +1203,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
     const int sw64 = jacobi_sweeps<kCl, double>(cl, sm, stride, b, s, s, kMaxSweeps, g, cur, s_flag, s_tally);
     double *D = sm + cur * stride;
     const int gx = block_at(px, g, nblk), gy = block_at(py, g, nblk);
-    for (int q = warp; q < 2 * b; q += kNw) {
+    for (int q = warp; q < 2 * b; q += nt >> 5) {
         const double *col = D + q * s;
         double v = 0.0;
         for (int r = lane; r < s; r += 32) v = fma(col[r], col[r], v);
@@ -1199,7 +1211,7 @@ __global__ void __launch_bounds__(kQrThreads, 2) k_jacobi_sm(const SvdJob *__res
         if (lane == 0) nrm_loc[q] = sqrt(v);
     }
     cl.sync();
-    for (int e = tid; e < 2 * b * kCl; e += kQrThreads) {
+    for (int e = tid; e < 2 * b * kCl; e += nt) {
         const int h = e / (2 * b), q = e % (2 * b), slot = q / b, j = q % b;
         const int u = block_at(slot ? nblk - 1 - h : h, g, nblk) * b + j;
         if (u < s) all_nrm[u] = cl.map_shared_rank(nrm_loc, h)[q];
@@ -1339,6 +1351,15 @@ __global__ void __launch_bounds__(kQrThreads) k_svd_emit(const EmitJob *__restri
 static size_t jacobi_sm_bytes(int s, int csize) {
     const int b = (s + 2 * csize - 1) / (2 * csize);
     return ((size_t)4 * b * s + 6 * b + s) * sizeof(double);
+}
+
+// Threads of a shared-memory Jacobi CTA: a warp for each of the b pairs of a step,
+// or the fewest equal passes of kJacWarps.  A pair is a latency-bound chain, so 8
+// warps took two or three passes (b = 24 for s <= 48 in one CTA, 12 at s = 96,
+// 10 at 160) for the time of each.
+static int jacobi_threads(int s, int csize) {
+    const int b = (s + 2 * csize - 1) / (2 * csize), passes = (b + kJacWarps - 1) / kJacWarps;
+    return 32 * std::max(kNw, (b + passes - 1) / passes);
 }
 
 // Block Jacobi with the matrix in global memory (L2): the two blocks of a
@@ -1605,6 +1626,7 @@ static void add_to_class(std::vector<LaunchClass<Job, K>> &cls, K kernel, int cs
     for (auto &c : cls)
         if (c.kernel == kernel && c.csize == csize) {
             c.smem = std::max(c.smem, smem);
+            c.threads = std::max(c.threads, threads);
             c.jobs.push_back(j);
             return;
         }
@@ -1683,7 +1705,7 @@ static void svd_launch(tlr_ctx *ctx, cudaStream_t st, const std::vector<SvdJob> 
         SvdKernel k = svd_sm_kernel(c, mode);
         size_t bytes = jacobi_sm_bytes(J.s, c);
         if (bytes <= smem_cap((const void *)k)) {
-            add_to_class(cls, k, c, bytes, J);
+            add_to_class(cls, k, c, bytes, J, jacobi_threads(J.s, c));
             csize_of[u] = c;
             continue;
         }

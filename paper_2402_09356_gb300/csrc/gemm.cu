@@ -181,15 +181,15 @@ static void launch_matern(tlr_ctx *ctx, cudaStream_t s, const std::vector<GemmPr
         smem = (size_t)per_sm / (per + 1) + 1024;
         std::lock_guard<std::mutex> lock(mu);
         if (smem > set_to) {
-            for (const void *k : {(const void *)k_gemm_df<64, 64, false, true, EpiMatern>,
+            for (const void *k : {(const void *)k_gemm_df<64, 64, EpiMatern>,
                                   (const void *)k_gemm_f64<64, 64, false, true, EpiMatern>,
-                                  (const void *)k_gemm_df<64, 64, false, true, EpiMaternMulti>,
+                                  (const void *)k_gemm_df<64, 64, EpiMaternMulti>,
                                   (const void *)k_gemm_f64<64, 64, false, true, EpiMaternMulti>})
                 TLR_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             set_to = smem;
         }
     }
-    if (df) launch(k_gemm_df<64, 64, false, true, Epi>, grid, kGemmThreads, smem, s, dp, dt, np, total, alpha, e);
+    if (df) launch(k_gemm_df<64, 64, Epi>, grid, kGemmThreads, smem, s, dp, dt, np, total, alpha, e);
     else launch(k_gemm_f64<64, 64, false, true, Epi>, grid, kGemmThreads, smem, s, dp, dt, np, total, alpha, e);
     TLR_CHECK_LAUNCH();
 }

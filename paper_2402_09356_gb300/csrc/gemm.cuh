@@ -25,6 +25,7 @@ struct GemmProb {
     const float2 *A2;  // paired-FP32 copies of A and B (same layout), for k_gemm_df
     const float2 *B2;
     int item;          // EpiMaternMulti: the factorisation whose covariance the problem holds
+    int lower;         // A (not transposed) is lower triangular: k_gemm_fit leaves out its zeros
 };
 
 constexpr int kGemmBK = 16, kGemmThreads = 256;

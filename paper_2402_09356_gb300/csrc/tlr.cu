@@ -711,7 +711,7 @@ void factor_group(tlr_ctx *ctx, cudaStream_t st, std::vector<FactorItem> &list, 
                     if (r <= 0) continue;
                     I.gram_off[j][i] = (int)off_c;
                     GemmProb g{};
-                    g.A = I.Xinv; g.lda = nb; g.m = mj; g.k = mj;
+                    g.A = I.Xinv; g.lda = nb; g.m = mj; g.k = mj; g.lower = 1;
                     g.B = Vslot(M, i, j); g.ldb = nb; g.n = r;
                     g.C = vt + off_c * nb; g.ldc = nb;
                     if (dfp) {

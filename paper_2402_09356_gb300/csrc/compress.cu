@@ -1914,6 +1914,7 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
                     a.A = X[u]; a.lda = sz; a.m = sz; a.k = sz;
                     a.B = X[u]; a.ldb = sz; a.n = sz;
                     a.C = W + oG[u]; a.ldc = sz;
+                    a.sym = 1;  // k_refine_angles reads G_ij, i <= j
                     gg.push_back(a);
                     const double tau = jobs[pending[u]].tau;
                     rjobs.push_back(RefineJob{W + oG[u], W + oIA[u], d_off + u, 0.01 * tau * tau, sz});

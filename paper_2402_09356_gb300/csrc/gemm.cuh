@@ -26,6 +26,7 @@ struct GemmProb {
     const float2 *B2;
     int item;          // EpiMaternMulti: the factorisation whose covariance the problem holds
     int lower;         // A (not transposed) is lower triangular: k_gemm_fit leaves out its zeros
+    int sym;           // C = A'A: the upper triangle is computed (k_gemm_fit also writes its mirror image)
 };
 
 constexpr int kGemmBK = 16, kGemmThreads = 256;
@@ -108,7 +109,7 @@ k_gemm_f64(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off,
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     GemmProb p;
     int m0, n0;
-    if (!gemm_tile<BM, BN>(probs, tile_off, nprob, t, p, m0, n0)) continue;
+    if (!gemm_tile<BM, BN>(probs, tile_off, nprob, t, p, m0, n0) || (p.sym && m0 >= n0 + BN)) continue;
     const int r0 = (tid & 15) * TM, c0 = (tid >> 4) * TN;
     double acc[TM][TN];
 #pragma unroll

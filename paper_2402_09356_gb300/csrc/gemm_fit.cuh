@@ -117,6 +117,10 @@ __device__ __forceinline__ void fit_tile(const GemmProb &p, int m0, int n0, int 
             if (r >= p.m) continue;
             double *cp = p.C + (int64_t)c * p.ldc + r;
             const double ab = alpha * Ar::val(acc[i][j]);
+            if (p.sym) {
+                if (r > c) continue;
+                p.C[(int64_t)r * p.ldc + c] = ab;  // and *cp, from the upper triangle (beta = 0)
+            }
             *cp = beta == 0.0 ? ab : ab + beta * (*cp);
         }
     }
@@ -144,6 +148,7 @@ k_gemm_fit(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off,
     // column groups of 8, dealt evenly to the ct column tiles
     const int ncg = (p.n + 7) / 8, base = ncg / ct, rem = ncg % ct;
     const int n0 = 8 * (tc * base + min(tc, rem)), tn = base + (tc < rem), n1 = min(p.n, n0 + 8 * tn);
+    if (p.sym && m0 >= n1) return;  // C = A'A: the upper triangle's tiles
 #define TLR_FIT(TMV, TNV) \
     case TNV: fit_tile<kDf, TA, TB, TMV, TNV>(p, m0, n0, n1, alpha, beta, As, Bs); break;
     // the widths without a body of their own take the next one (their columns

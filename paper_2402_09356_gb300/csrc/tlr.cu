@@ -731,7 +731,7 @@ void factor_group(tlr_ctx *ctx, cudaStream_t st, std::vector<FactorItem> &list, 
                 if (S > 0 && j + 1 < nt) {
                     I.gram[j].alloc((size_t)S * S * sizeof(double), st);
                     GemmProb g{};
-                    g.A = vt; g.lda = nb; g.m = S; g.k = mj;
+                    g.A = vt; g.lda = nb; g.m = S; g.k = mj; g.sym = 1;
                     g.B = vt; g.ldb = nb; g.n = S;
                     g.C = I.gram[j].as<double>(); g.ldc = S;
                     if (dfp && !tcg) {

@@ -42,9 +42,6 @@ EPS = 1e-7
 THETA0 = (1.0, 0.1, 0.5)
 ORDER = "hilbert"
 L2_FLUSH_BYTES = 256 << 20
-# DRAM bytes (read + write) per launch from ncu captures of unchanged kernels,
-# by (kernel, tile size); the capture and its command are in profiles/
-NCU_TRAFFIC = {("k_potrf_inv<16, 1>", 800): (3.34e6, "profiles/k_potrf_inv_n16000.md")}
 
 
 def peaks():
@@ -380,7 +377,7 @@ def run_gpu(args):
             peak, src = tc_peak, ("bf16_tflops_sustained %.1f of MEASURED_PEAKS.json (%s) / 15 slice-pair "
                                   "products per FP64-equivalent product" % (pk["bf16_tflops_sustained"], pk_src))
         elif o is mixed:
-            name = "k_gemm_df<64,64,N,T,EpiMatern> (panel update + Matern generation, paired-FP32 products)"
+            name = "k_gemm_df<64,64,EpiMatern> (panel update + Matern generation, paired-FP32 products)"
             peak, src = df_peak, ("FP32 pipe for paired-FP32 products: %d SMs x 128 lanes x 2 flop / 12 instr "
                                   "per emulated FMA x %.0f MHz (sampled SM clock)" % (n_sms, sm_mhz))
         else:
@@ -398,22 +395,22 @@ def run_gpu(args):
         fl = k["jacobi16_flops"] / launches
         achieved = fl / (avg / 1000.0) / 1e12 if avg > 0 else 0.0
         clusters = k["jacobi16_clusters"] / launches
-        occupied = min(n_sms, 16 * clusters) * 4 * sm_mhz * 1e6 / 1e12
+        fp32_peak = n_sms * 256 * sm_mhz * 1e6 / 1e12
+        occupied = min(n_sms, 16 * clusters) * 256 * sm_mhz * 1e6 / 1e12
         return {"bound": "alu", "kernel": "k_jacobi_sm<16> (cluster Jacobi SVD of the high-rank tiles)",
-                "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-                "frac": achieved / fp64_peak if fp64_peak else None, "traffic": None,
-                "peak_source": "FP64 DFMA pipe: %d SMs x 4 flop/clk x %.0f MHz (sampled SM clock)" % (n_sms, sm_mhz),
+                "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
+                "frac": achieved / fp32_peak if fp32_peak else None, "traffic": None,
+                "peak_source": "FP32 pipe: %d SMs x 256 flop/clk x %.0f MHz (sampled SM clock)" % (n_sms, sm_mhz),
                 "frac_of_occupied_sms": achieved / occupied if occupied else None,
                 "clusters_per_launch": clusters, "launch_ms_avg": avg, "launches": k["jacobi16_launches"],
                 "flops_per_launch": fl, "total_ms": k["jacobi16_ms"],
-                "flops_counted": "FP64 work as executed: M J (2 s^3), norms per sweep (2 s^2), "
-                                 "2 s per pair checked, 6 s per pair rotated"}
+                "flops_counted": "FP32 sweeps: norms (2 s^2), a dot product (2 s) and a rotation (12 s) per pair"}
 
     def roof_potrf(o):
-        # one launch per tile column on the side stream: L = chol(T_jj) (the
-        # algorithmic m^3/3 FP64 flops) and L^-1 (another m^3/3, executed work
-        # that replaces the TRSM); its in-step time from the events around it
-        # on that stream
+        # per tile column on the side stream: L = chol(T_jj) (the algorithmic
+        # m^3/3 FP64 flops) and L^-1 (another m^3/3, executed work that
+        # replaces the TRSM), in blocks of 288 rows with batched GEMMs between
+        # them; the in-step time from the events around it on that stream
         nt = (N_POINTS + NB - 1) // NB
         ms_step = o["detail_ms"]["potrf"]
         avg = ms_step / nt
@@ -421,20 +418,18 @@ def run_gpu(args):
         fl = sum(m ** 3 / 3.0 for m in ms) / nt
         achieved = fl / (avg / 1000.0) / 1e12 if avg > 0 else 0.0
         occupied = 16 * 4 * sm_mhz * 1e6 / 1e12
-        traffic = NCU_TRAFFIC.get(("k_potrf_inv<16, 1>", NB))
-        return {"bound": "alu", "kernel": "k_potrf_inv<16, 1> (diagonal tile: Cholesky in FP64, its inverse in "
-                                          "float-float pairs on the paired paths; one 16-CTA cluster)",
+        return {"bound": "alu", "kernel": "k_potrf_inv<16> and its block products (diagonal tile: Cholesky and "
+                                          "inverse in FP64; one 16-CTA cluster a block of 288 rows)",
                 "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp64_peak if fp64_peak else None,
-                "traffic": traffic[0] if traffic else None,
-                "traffic_source": traffic[1] if traffic else None,
+                "traffic": None,
                 "peak_source": "FP64 DFMA pipe: %d SMs x 4 flop/clk x %.0f MHz (sampled SM clock)" % (n_sms, sm_mhz),
                 "frac_of_occupied_sms": achieved / occupied if occupied else None,
                 "launch_ms_avg": avg, "launches": nt * args.steps, "flops_per_launch": fl,
                 "flops_counted": "algorithmic: m^3/3 (Cholesky of the diagonal tile)",
                 "executed_flops_per_launch": 2.0 * fl,
                 "executed_tflops": 2.0 * achieved,
-                "executed_note": "the launch also forms L^-1 (another m^3/3), used in place of a TRSM",
+                "executed_note": "they also form L^-1 (another m^3/3), used in place of a TRSM",
                 "total_ms": ms_step * args.steps}
 
     # the dominant kernel of the headline path: the largest device time per step

@@ -442,11 +442,10 @@ int tlr_compress_stats(tlr_ctx *ctx, int64_t *out);
 
 /* The cluster Jacobi SVD on 16-CTA clusters (the high-rank tiles next to the
  * diagonal) during the last profiled factorisation, written to out[0..3]:
- * device time (ms, CUDA events on its stream, summed over launches), FP64
- * floating-point operations as executed (one FP64 product M J of 2 s^3, the
- * column norms at every FP64 sweep, one dot product per pair checked, one
- * two-column rotation per pair rotated), number of launches, and number of
- * clusters (tiles) over those launches.  Errors: TLR_ERR_ARG. */
+ * device time (ms, CUDA events on its stream, summed over launches), FP32
+ * floating-point operations of its preconditioning sweeps (the column norms,
+ * and for every pair a dot product and a rotation of two columns), number of
+ * launches, and number of clusters (tiles) over those launches.  Errors: TLR_ERR_ARG. */
 int tlr_kernel_stats(tlr_ctx *ctx, double *out);
 
 /* ---- MLE (Sec. 5.1: derivative-free, bound-constrained) ------------------ */

@@ -188,7 +188,7 @@ struct tlr_ctx {
     std::vector<cudaEvent_t> comp_pending;    // complete rounds (8 marks each) not yet read
     double comp_ms[7] = {0, 0, 0, 0, 0, 0, 0};
     long long comp_stats[7] = {};  // tiles, rounds, FP64 Jacobi sweeps (sum, max), FP32 sweeps (sum), QR / SVD jobs on the global-memory kernels
-    // the 16-CTA cluster Jacobi (profiling): device ms, FP64 flops, launches, clusters
+    // the 16-CTA cluster Jacobi (profiling): device ms, FP32 flops of its sweeps, launches, clusters
     std::vector<cudaEvent_t> cls_time_events;
     double *d_potrf_scratch = nullptr;  // diagonal-block inverses of the cluster POTRF (per job)
     int potrf_scratch_jobs = 0;

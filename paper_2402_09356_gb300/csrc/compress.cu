@@ -1998,10 +1998,9 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
             ctx->comp_stats[4] += sw[1];
         }
         if (ctx->profile && t16.csize == 16) {
-            // FP64 work of the 16-CTA Jacobi launch, counted as executed:
-            // M1 = M J (2 s^3), the norms at each FP64 sweep and at the end
-            // (2 s^2 each), one dot product per pair checked (2 s), one
-            // rotation of two columns per pair rotated (6 s)
+            // FP32 work of the 16-CTA Jacobi launch: per sweep the norms (2 s^2)
+            // and, for each of s (s - 1) / 2 pairs, a dot product (2 s) and a
+            // rotation of two columns of 2 s (12 s)
             float ms = 0.f;
             TLR_CUDA_TRY(cudaEventElapsedTime(&ms, t16.e0, t16.e1));
             double fl = 0.0;
@@ -2010,7 +2009,7 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
                 if (svd_csize[u] != 16) continue;
                 const int *sw = h_rank.data() + np + 4 * u;
                 const double s = ps[u];
-                fl += 2.0 * s * s * s + 2.0 * s * s * (sw[0] + 1) + 2.0 * s * sw[2] + 6.0 * s * sw[3];
+                fl += sw[1] * (2.0 * s * s + 7.0 * s * s * (s - 1.0));
                 ++jobs16;
             }
             ctx->k16_ms += ms;

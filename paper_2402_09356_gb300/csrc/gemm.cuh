@@ -95,9 +95,8 @@ __device__ __forceinline__ bool gemm_tile(const GemmProb *__restrict__ probs, co
 // smaller than the tile count keeps the product to that many CTAs), 256
 // threads per CTA (a 16 x 16 thread grid, BM/16 x BN/16 outputs per thread),
 // K in steps of 16 through shared memory.
-// Tiles of 64 x 64 serve large products; 32-row or 32-column tiles serve the
-// many thin products of the low-rank updates (ranks of a few tens), whose
-// padding would otherwise dominate.
+// Tiles of 64 x 64 serve the panel generation, 32 x 32 and 16 x 16 the SVD's
+// refinement; the other products are k_gemm_fit's.
 template <int BM, int BN, bool TA, bool TB, class Epi>
 __global__ void __launch_bounds__(kGemmThreads)
 k_gemm_f64(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off, int nprob, int ntiles,

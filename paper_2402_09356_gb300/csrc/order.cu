@@ -1,4 +1,6 @@
-// a1: spatial ordering of the locations (Sec. 3).
+// a1: spatial ordering of the locations (Sec. 3).  Up to the sizes of the last
+// section of this file the whole ordering runs on one thread-block cluster;
+// what follows is the layout above them, a launch per pass.
 //
 // Morton / Hilbert / random: one thread per point computes a 32-bit key
 // (Sec. 3.1 "Encoding"), then a stable LSD radix sort orders (key, index)

@@ -136,18 +136,19 @@ k_gemm_f64(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off,
             Bs[kk][c] = v;
         }
         __syncthreads();
+        for (int kh = 0; kh < kGemmBK && k0 + kh < p.k; kh += 8)  // sample sizes are multiples of 8
 #pragma unroll
-        for (int kk = 0; kk < kGemmBK; ++kk) {
-            double a[TM], b[TN];
+            for (int kk = kh; kk < kh + 8; ++kk) {
+                double a[TM], b[TN];
 #pragma unroll
-            for (int q = 0; q < TM; ++q) a[q] = As[kk][r0 + q];
+                for (int q = 0; q < TM; ++q) a[q] = As[kk][r0 + q];
 #pragma unroll
-            for (int q = 0; q < TN; ++q) b[q] = Bs[kk][c0 + q];
+                for (int q = 0; q < TN; ++q) b[q] = Bs[kk][c0 + q];
 #pragma unroll
-            for (int x = 0; x < TM; ++x)
+                for (int x = 0; x < TM; ++x)
 #pragma unroll
-                for (int y = 0; y < TN; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
-        }
+                    for (int y = 0; y < TN; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+            }
         __syncthreads();
     }
 #pragma unroll

@@ -12,9 +12,17 @@ from test_gpu_qr_sizes import EPS, known_tile
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("nb,r", [(800, 340), (800, 370), (800, 424), (800, 429)])
+def test_large_samples(nb, r):
+    check(nb, r)
+
+
 @pytest.mark.parametrize("r", [2, 21, 45, 64, 82, 97, 114, 131, 148, 163, 180, 197, 211, 228, 241, 250, 275])
 def test_known_spectrum(r):
-    nb = 300
+    check(300, r)
+
+
+def check(nb, r):
     ctx = tlr.Context(0)
     tiles = np.zeros((3, nb, nb))
     tiles[0], tiles[2] = np.eye(nb), np.eye(nb)

@@ -432,22 +432,119 @@ __global__ void k_potrf_edges(const PotrfEdges jobs) {
     }
 }
 
-// Tiles wider than kPotrfOuter are factored in blocks of w <= kPotrfOuter
-// columns: the cluster kernel factors and inverts a diagonal block, and the
-// products between blocks run as batched FP64 GEMMs over the whole GPU.  For
-// block b, with X_bb = L_bb^-1:
-//   L_ib = A_ib X_bb'  (i > b);   A_ij -= L_ib L_jb'  (i >= j > b);
-//   X_bj = X_bb S_bj  (j < b);    S_ij -= L_ib X_bj  (i > b >= j),
-// S_ij the negated sum of L_ik X_kj so far.  One cluster alone runs the tile's
-// m^3 / 3 multiply-adds twice over on 16 of the 152 SMs: at m = 800 its
-// trailing updates, not its pivot chain, took most of 4.1 ms alone; in blocks
-// it takes 1.8 ms (three cluster launches of 0.33, the GEMMs 0.8).  Widths of
-// 224 and 160 took 1.95 and 1.99 ms: more launches, each as long as one 32 x 32
-// output tile's FP64 chain.  The GEMMs are split by column chunks so that the
-// triangular factors' zeros are skipped.  X_bb has to be FP64: L_ib is formed
-// from it (with a float-float inverse |L L' - A| was 1.2e-14, not 9e-16).
+// Substitution with a factored diagonal block L_bb (w <= kPotrfOuter columns) in
+// steps of 32, the inverses of its 32 x 32 diagonal blocks taken from X_bb's:
+// `rows` rows a of A below the block become those of L (x L_bb' = a, in place),
+// `cols` columns of S the inverse's (L_bb y = s, into Y).
+struct PotrfSub {
+    const double *L, *X;
+    double *A;
+    const double *S;
+    double *Y;
+    int ldl, ldx, lds, w, rows, cols;
+};
+struct PotrfSubs {
+    PotrfSub j[kMaxGroup];
+};
+// One warp a right-hand side, its entry r of a step in lane r, four a CTA (a row
+// of L that a warp reads serves the others from L1; four adjacent rows of A are a
+// 32-byte sector).  No barrier: a warp's steps depend on its own vector only.
+// Bound by the FP64 pipe: w^2 / 64 + w / 2 multiply-adds a warp of 64 cycles each,
+// one warp a scheduler at m = 800; L comes from L2 16 columns ahead.  The
+// sums are of 32 terms, each taken from the entry.  A product with X_bb takes as
+// long, but |L L' - A| and |L X - I| of smooth fields are then two to six times
+// those of the algorithm that inverts 32 x 32 blocks only, which these are.
+constexpr int kSubThreads = 128, kSubVecs = kSubThreads / 32, kSubAhead = 16;
 constexpr int kPotrfOuter = 288, kPotrfChunk = 96;
+__global__ void __launch_bounds__(kSubThreads) k_potrf_sub(const PotrfSubs jobs) {
+    __shared__ double ys[kSubVecs][kPotrfOuter], ts[kSubVecs][kBlk];
+    const PotrfSub J = jobs.j[blockIdx.y];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, w = J.w;
+    const int row_ctas = (J.rows + kSubVecs - 1) / kSubVecs, bx = blockIdx.x;
+    const bool row = bx < row_ctas;
+    const int v0 = (row ? bx : bx - row_ctas) * kSubVecs, nv = min(kSubVecs, (row ? J.rows : J.cols) - v0);
+    if (nv <= 0) return;
+    if (row) {
+        for (int e = tid; e < kSubVecs * w; e += kSubThreads) {
+            const int v = e % kSubVecs, k = e / kSubVecs;
+            if (v < nv) ys[v][k] = J.A[(int64_t)k * J.ldl + v0 + v];
+        }
+    } else {
+        for (int v = 0; v < nv; ++v)
+            for (int k = tid; k < w; k += kSubThreads) ys[v][k] = J.S[(int64_t)(v0 + v) * J.lds + k];
+    }
+    __syncthreads();
+    if (warp < nv) {
+        double *y = ys[warp], *t = ts[warp];
+        for (int p = 0; p < w; p += kBlk) {
+            const bool in = p + lane < w;
+            const double *Lr = J.L + p + lane, *Xr = J.X + (int64_t)p * J.ldx + p + lane;
+            double x[kBlk], l[2][kSubAhead];
+            auto load = [&](int k0, double (&v)[kSubAhead]) {
+#pragma unroll
+                for (int k = 0; k < kSubAhead; ++k) v[k] = in && k0 < p ? Lr[(int64_t)(k0 + k) * J.ldl] : 0.0;
+            };
+            load(0, l[0]);
+#pragma unroll
+            for (int k = 0; k < kBlk; ++k) x[k] = in && k <= lane ? Xr[(int64_t)k * J.ldx] : 0.0;
+            double a = in ? y[p + lane] : 0.0;
+            for (int k0 = 0; k0 < p; k0 += 2 * kSubAhead) {  // 32 columns: two loads ahead of their use
+                double s0 = 0.0, s1 = 0.0;
+                load(k0 + kSubAhead, l[1]);
+#pragma unroll
+                for (int k = 0; k < kSubAhead; k += 2) {
+                    s0 = fma(l[0][k], y[k0 + k], s0);
+                    s1 = fma(l[0][k + 1], y[k0 + k + 1], s1);
+                }
+                load(k0 + 2 * kSubAhead, l[0]);
+#pragma unroll
+                for (int k = 0; k < kSubAhead; k += 2) {
+                    s0 = fma(l[1][k], y[k0 + kSubAhead + k], s0);
+                    s1 = fma(l[1][k + 1], y[k0 + kSubAhead + k + 1], s1);
+                }
+                a -= s0 + s1;
+            }
+            t[lane] = a;
+            __syncwarp();
+            double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+            for (int k = 0; k < kBlk; k += 2) {
+                s0 = fma(x[k], t[k], s0);
+                s1 = fma(x[k + 1], t[k + 1], s1);
+            }
+            if (in) y[p + lane] = s0 + s1;
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    if (row) {
+        for (int e = tid; e < kSubVecs * w; e += kSubThreads) {
+            const int v = e % kSubVecs, k = e / kSubVecs;
+            if (v < nv) J.A[(int64_t)k * J.ldl + v0 + v] = ys[v][k];
+        }
+    } else {
+        for (int v = 0; v < nv; ++v)
+            for (int k = tid; k < w; k += kSubThreads) J.Y[(int64_t)(v0 + v) * J.ldx + k] = ys[v][k];
+    }
+}
 
+// Tiles wider than kPotrfOuter are factored in blocks of w <= kPotrfOuter
+// columns: the cluster kernel factors and inverts a diagonal block, the rows of L
+// below it and its rows of the inverse follow by substitution (k_potrf_sub), and
+// the products between blocks run as batched FP64 GEMMs over the whole GPU.
+// For block b, with X_bb = L_bb^-1:
+//   L_ib L_bb' = A_ib  (i > b);   A_ij -= L_ib L_jb'  (i >= j > b);
+//   L_bb X_bj = S_bj  (j < b);    S_ij -= L_ib X_bj  (i > b >= j),
+// S_ij the negated sum of L_ik X_kj so far.  One cluster alone runs the tile's
+// m^3 / 3 multiply-adds twice over on 16 of the 152 SMs, and its trailing
+// updates, not its pivot chain, take most of the time.  One tile alone, one
+// cluster -> blocks: m = 300 0.99 -> 0.55 ms, 400 1.31 -> 0.72, 512 1.81 -> 0.92,
+// 576 2.26 -> 1.05, 800 4.63 -> 1.56, 1,024 8.59 -> 2.30; up to 288 there is one
+// block.  (At m = 800 widths of 224 and 160 took a tenth longer: more launches,
+// each as long as one 32 x 32 output tile's FP64 chain.)  The GEMMs are split
+// by column chunks so that the triangular factors' zeros are skipped, and sum 32
+// terms at a time (of 288 terms in one sum each rounding is of the whole entry:
+// |L L' - A| of a rough field was twice the 32-wide algorithm's).
 void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs) {
     std::vector<PotrfJob> act;
     for (const PotrfJob &J : jobs) {
@@ -466,11 +563,10 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs)
         TLR_CUDA_TRY(cudaMalloc(&ctx->d_potrf_scratch, per * want * sizeof(double)));
         ctx->potrf_scratch_jobs = want;
     }
-    // per job: block width and count, and the scratch panels P (L_ib before it
-    // replaces A_ib) and S, both with leading dimension m
+    // per job: block width and count, and the scratch panel S with leading dimension m
     struct Blocked {
         int w = 0, n = 1;
-        double *P = nullptr, *S = nullptr;
+        double *S = nullptr;
     };
     std::vector<Blocked> bl(act.size());
     size_t words = 0;
@@ -483,7 +579,7 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs)
         bl[q].w = (int)(ceil_div(ceil_div(m, bl[q].n), kBlk) * kBlk);
         bl[q].n = (int)ceil_div(m, bl[q].w);
         blocks = std::max(blocks, bl[q].n);
-        words += (size_t)m * (m + bl[q].w);
+        words += (size_t)m * m;
     }
     if (blocks == 1) {
         potrf_cluster(ctx, s, act);
@@ -496,9 +592,8 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs)
     for (size_t q = 0; q < act.size(); ++q) {
         if (bl[q].n == 1) continue;
         const PotrfJob &J = act[q];
-        bl[q].P = buf.as<double>() + words;
-        bl[q].S = bl[q].P + (size_t)J.m * bl[q].w;
-        words += (size_t)J.m * (J.m + bl[q].w);
+        bl[q].S = buf.as<double>() + words;
+        words += (size_t)J.m * J.m;
         edges.e[nedge++] = PotrfEdge{J.A, J.X, bl[q].S, J.lda, J.ldx, J.m, J.m, bl[q].w};
         mmax = std::max(mmax, J.m);
     }
@@ -512,8 +607,9 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs)
     };
     for (int b = 0; b < blocks; ++b) {
         std::vector<PotrfJob> diag;
-        std::vector<GemmProb> gx, gl, ga, gs;
-        std::vector<CopyDesc> cl;
+        std::vector<GemmProb> ga, gs;
+        PotrfSubs subs{};
+        int nsub = 0, ctas = 0;
         for (size_t q = 0; q < act.size(); ++q) {
             const PotrfJob &J = act[q];
             const Blocked &B = bl[q];
@@ -526,34 +622,30 @@ void potrf_inv_batched(tlr_ctx *ctx, cudaStream_t s, std::vector<PotrfJob> jobs)
             D.row_base = J.row_base + p;
             diag.push_back(D);
             if (B.n == 1) continue;
+            double *Lib = J.A + (int64_t)p * J.lda + e;
+            subs.j[nsub++] = PotrfSub{D.A, D.X, Lib, B.S + p, J.X + p, J.lda, J.ldx, J.m, w, rest, p};
+            ctas = std::max(ctas, (int)(ceil_div(rest, kSubVecs) + ceil_div(p, kSubVecs)));
+            if (rest <= 0) continue;
+            // S_ib, columns c0 .. c1: X_bb is zero above row c0
             for (int c0 = 0; c0 < w; c0 += kPotrfChunk) {
                 const int c1 = std::min(w, c0 + kPotrfChunk);
-                // X_bj, rows c0 .. c1: X_bb is zero right of column c1
-                if (p > 0) gx.push_back(prob(D.X + c0, J.ldx, B.S + p, J.m, J.X + p + c0, J.ldx, c1 - c0, p, c1));
-                if (rest <= 0) continue;
-                // L_ib, columns c0 .. c1
-                gl.push_back(prob(J.A + (int64_t)p * J.lda + e, J.lda, D.X + c0, J.ldx, B.P + (int64_t)c0 * J.m + e, J.m,
-                                  rest, c1 - c0, c1));
-                // S_ib, columns c0 .. c1: X_bb is zero above row c0
-                gs.push_back(prob(B.P + (int64_t)c0 * J.m + e, J.m, D.X + (int64_t)c0 * J.ldx + c0, J.ldx,
+                gs.push_back(prob(Lib + (int64_t)c0 * J.lda, J.lda, D.X + (int64_t)c0 * J.ldx + c0, J.ldx,
                                   B.S + (int64_t)(p + c0) * J.m + e, J.m, rest, c1 - c0, w - c0));
             }
-            if (rest <= 0) continue;
-            if (p > 0) gs.push_back(prob(B.P + e, J.m, J.X + p, J.ldx, B.S + e, J.m, rest, p, w));
+            if (p > 0) gs.push_back(prob(Lib, J.lda, J.X + p, J.ldx, B.S + e, J.m, rest, p, w));
             // lower part of the trailing matrix; no chunk crosses a block
             // boundary, so that nothing above the diagonal blocks is written
             for (int c0 = e, c1; c0 < J.m; c0 = c1) {
                 c1 = std::min({J.m, c0 + kPotrfChunk, (c0 / B.w + 1) * B.w});
-                ga.push_back(prob(B.P + c0, J.m, B.P + c0, J.m, J.A + (int64_t)c0 * J.lda + c0, J.lda, J.m - c0, c1 - c0, w));
+                const double *Lc = J.A + (int64_t)p * J.lda + c0;
+                ga.push_back(prob(Lc, J.lda, Lc, J.lda, J.A + (int64_t)c0 * J.lda + c0, J.lda, J.m - c0, c1 - c0, w));
             }
-            cl.push_back(CopyDesc{B.P + e, J.m, J.A + (int64_t)p * J.lda + e, J.lda, rest, w});
         }
         potrf_cluster(ctx, s, diag);
-        gemm_batched_small(ctx, s, false, true, gl, 1.0, 0.0);   // L
-        gemm_batched_small(ctx, s, false, true, ga, -1.0, 1.0);  // trailing update
-        gemm_batched_small(ctx, s, false, false, gx, 1.0, 0.0);  // X_bj
-        gemm_batched_small(ctx, s, false, false, gs, -1.0, 1.0);  // S
-        copy_batched(ctx, s, cl);
+        launch(k_potrf_sub, dim3((unsigned)ctas, (unsigned)nsub), kSubThreads, 0, s, subs);
+        TLR_CHECK_LAUNCH();
+        gemm_batched_small(ctx, s, false, true, ga, -1.0, 1.0, true);  // trailing update
+        gemm_batched_small(ctx, s, false, false, gs, -1.0, 1.0, true);  // S
     }
 }
 

@@ -25,7 +25,7 @@ void *stage_push(tlr_ctx *ctx, const void *data, size_t bytes, cudaStream_t s) {
     return d;
 }
 
-template <int BM, int BN>
+template <int BM, int BN, bool kParts>
 static void launch_shape(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
                          double alpha, double beta) {
     if (probs.empty()) return;
@@ -43,9 +43,10 @@ static void launch_shape(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const s
     const EpiLinear epi{beta};
     // the transposition pairs the library uses: NN, TN, NT (no TT)
     if (ta && tb) throw make_error(TLR_ERR_ARG, "GEMM with both operands transposed is not provided");
-    if (!ta && !tb) launch(k_gemm_f64<BM, BN, false, false, EpiLinear>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-    else if (!ta) launch(k_gemm_f64<BM, BN, false, true, EpiLinear>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
-    else launch(k_gemm_f64<BM, BN, true, false, EpiLinear>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
+    if (!ta && !tb) launch(k_gemm_f64<BM, BN, false, false, EpiLinear, kParts>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
+    else if (!ta) launch(k_gemm_f64<BM, BN, false, true, EpiLinear, kParts>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
+    else if constexpr (kParts) throw make_error(TLR_ERR_ARG, "sums in parts with A transposed are not provided");
+    else launch(k_gemm_f64<BM, BN, true, false, EpiLinear, kParts>, total, kGemmThreads, 0, s, dp, dt, np, total, alpha, epi);
     TLR_CHECK_LAUNCH();
 }
 
@@ -136,14 +137,14 @@ void split_f2_batched(tlr_ctx *ctx, cudaStream_t s, const std::vector<SplitDesc>
 
 constexpr int kSmallTiles = 300;
 void gemm_batched_small(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
-                        double alpha, double beta) {
+                        double alpha, double beta, bool parts) {
     // tiles of 32 x 32 while they fill the SMs, else of 16 x 16: an output
     // tile's chain of FP64 multiply-adds (k x 64 cycles x 2 warps a scheduler, x
     // 4 outputs a thread) is then a quarter as long, on four times the CTAs
     int64_t tiles = 0;
     for (const GemmProb &p : probs) tiles += ceil_div(p.m, 32) * ceil_div(p.n, 32);
-    if (tiles >= kSmallTiles) launch_shape<32, 32>(ctx, s, ta, tb, probs, alpha, beta);
-    else launch_shape<16, 16>(ctx, s, ta, tb, probs, alpha, beta);
+    if (tiles >= kSmallTiles) (parts ? launch_shape<32, 32, true> : launch_shape<32, 32, false>)(ctx, s, ta, tb, probs, alpha, beta);
+    else (parts ? launch_shape<16, 16, true> : launch_shape<16, 16, false>)(ctx, s, ta, tb, probs, alpha, beta);
 }
 
 void gemm_batched(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,

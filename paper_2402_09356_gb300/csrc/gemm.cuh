@@ -96,8 +96,10 @@ __device__ __forceinline__ bool gemm_tile(const GemmProb *__restrict__ probs, co
 // threads per CTA (a 16 x 16 thread grid, BM/16 x BN/16 outputs per thread),
 // K in steps of 16 through shared memory.
 // Tiles of 64 x 64 serve the panel generation, 32 x 32 and 16 x 16 the SVD's
-// refinement; the other products are k_gemm_fit's.
-template <int BM, int BN, bool TA, bool TB, class Epi>
+// refinement and the diagonal tile's block products; the other products are
+// k_gemm_fit's.  kParts: terms are summed 32 at a time and the sums added up
+// (rounding errors of the size of a part's sum, not of the whole entry's).
+template <int BM, int BN, bool TA, bool TB, class Epi, bool kParts = false>
 __global__ void __launch_bounds__(kGemmThreads)
 k_gemm_f64(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off, int nprob, int ntiles,
            double alpha, Epi epi) {
@@ -110,11 +112,14 @@ k_gemm_f64(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off,
     int m0, n0;
     if (!gemm_tile<BM, BN>(probs, tile_off, nprob, t, p, m0, n0) || (p.sym && m0 >= n0 + BN)) continue;
     const int r0 = (tid & 15) * TM, c0 = (tid >> 4) * TN;
-    double acc[TM][TN];
+    double acc[TM][TN], sum[kParts ? TM : 1][kParts ? TN : 1];
 #pragma unroll
     for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < TN; ++b) acc[a][b] = 0.0;
+        for (int b = 0; b < TN; ++b) {
+            acc[a][b] = 0.0;
+            if constexpr (kParts) sum[a][b] = 0.0;
+        }
 
     for (int k0 = 0; k0 < p.k; k0 += kGemmBK) {
 #pragma unroll
@@ -149,7 +154,24 @@ k_gemm_f64(const GemmProb *__restrict__ probs, const int *__restrict__ tile_off,
 #pragma unroll
                     for (int y = 0; y < TN; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
             }
+        if constexpr (kParts) {
+            if ((k0 / kGemmBK & 1) || k0 + kGemmBK >= p.k) {
+#pragma unroll
+                for (int x = 0; x < TM; ++x)
+#pragma unroll
+                    for (int y = 0; y < TN; ++y) {
+                        sum[x][y] += acc[x][y];
+                        acc[x][y] = 0.0;
+                    }
+            }
+        }
         __syncthreads();
+    }
+    if constexpr (kParts) {
+#pragma unroll
+        for (int x = 0; x < TM; ++x)
+#pragma unroll
+            for (int y = 0; y < TN; ++y) acc[x][y] = sum[x][y];
     }
 #pragma unroll
     for (int y = 0; y < TN; ++y) {
@@ -335,10 +357,11 @@ struct SplitDesc {
 // split_f2 for a batch of blocks in one launch.
 void split_f2_batched(tlr_ctx *ctx, cudaStream_t s, const std::vector<SplitDesc> &descs);
 
-// FP64, 32 x 32 output tiles for every problem: four times the CTAs of the
-// 64 x 64 shape, for small square products on the critical path.
+// FP64, 32 x 32 output tiles for every problem, or 16 x 16 where those do not
+// fill the SMs, for small products on the critical path.  parts: terms summed 32
+// at a time (A not transposed).
 void gemm_batched_small(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
-                        double alpha, double beta);
+                        double alpha, double beta, bool parts = false);
 
 // df = true selects the paired-FP32 kernel (FP64-accurate products on the FP32
 // pipe); every problem must then carry A2/B2 copies made by split_f2.

@@ -7,13 +7,13 @@
 // diagonal tile block by block.  Per tile column three launches:
 //   k_trsv      y_k <- L_kk^-1 y_k, one cluster, blocks of 32 rows whose
 //               inverses were formed for all tiles by one launch at the start
-//               (k_inv_blocks: a block's substitution is then one 32 x 32
-//               product, not 32 dependent steps);
+//               (k_inv_blocks: a block's substitution is then three 32 x 32
+//               products, not 32 dependent steps);
 //   k_pair_dots c_ik = V_ik' y_k for all i > k, one warp a column of V;
 //   k_pair_sub  y_i -= U_ik c_ik for all i > k.
 // The product L w has no chain: one launch of k_pair_dots over all tiles, one
 // of k_row_sums.  All descriptors go up once per call.  n = 20,000, tile 800: solve
-// 42.4 -> 1.95 ms (k_trsv 51 us a tile, the two others 10 each), L w 1.46 -> 0.11.
+// 42.4 -> 2.58 ms (k_trsv 77 us a tile, the two others 10 each), L w 1.46 -> 0.11.
 #include <algorithm>
 #include <mutex>
 
@@ -87,12 +87,17 @@ __global__ void __launch_bounds__(kThreads) k_inv_blocks(const double *__restric
 
 // x <- L^-1 x for one diagonal tile (m <= 1024, ld ldl) by one cluster: CTA
 // `rank` owns the blocks rank, rank + kCl, ... of the right-hand side, each
-// kept by kThreads / kOwn threads (four or eight a row).  Step b: the owner
-// multiplies its block by the block's inverse and stores the 32 values into
-// every CTA; after one cluster barrier every CTA subtracts L's block column b
-// times them from its blocks.  The entries of block columns b + 1 and b + 2 are
-// on their way to registers meanwhile (the tile comes from HBM).  Bound by the
-// chain of a step: barrier, update of the next block, its product.
+// kept by kThreads / kOwn threads (four or two a row).  Step b: the owner
+// multiplies its block by the block's inverse, corrects the product by its
+// residual, y += L_bb^-1 (x - L_bb y), and stores the 32 values into every CTA;
+// after one cluster barrier every CTA subtracts L's block column b times them
+// from its blocks.  (The product alone is as far off as |L^-1| |x| lets it be:
+// right-hand sides of a smooth field, whose y is far smaller, had 2 to 50 times
+// the error of substitution; one residual step leaves none of that, for 26 us
+// more a tile of 800.)  The
+// entries of block columns b + 1 and b + 2 are on their way to registers
+// meanwhile (the tile comes from HBM).  Bound by the chain of a step: barrier,
+// update of the next block, its three products.
 template <int kCl>
 __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L, int ldl, int m,
                                                     const double *__restrict__ inv, double *__restrict__ x) {
@@ -103,10 +108,10 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
     const int rank = (int)cl.block_rank(), tid = threadIdx.x;
     const int o = tid / (kThreads / kOwn), r = tid % (kThreads / kOwn) / kQ, q = tid % kQ;
     const int I = rank + o * kCl, row = I * kB + r;  // the thread's block and row
-    __shared__ double rhs[kOwn][kB], xs[2][kB];
+    __shared__ double rhs[kOwn][kB], own[2][kOwn][kB], xs[2][kB];
     const int nblk = (m + kB - 1) / kB;
     if (q == 0) rhs[o][r] = row < m ? x[row] : 0.0;
-    double a[2][kN], d[kN];
+    double a[2][kN], d[kN], g[kN];
     auto load = [&](int b, double (&v)[kN]) {  // L's block column b in the thread's row
         const bool in = b < I && row < m;
 #pragma unroll
@@ -118,33 +123,41 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
         return v;
     };
 #pragma unroll
-    for (int k = 0; k < kN; ++k) d[k] = I < nblk ? inv[(int64_t)I * kB * kB + r * kB + q + kQ * k] : 0.0;
+    for (int k = 0; k < kN; ++k) {  // row r of the block's inverse and of the block
+        const int c = q + kQ * k;
+        d[k] = I < nblk ? inv[(int64_t)I * kB * kB + r * kB + c] : 0.0;
+        g[k] = row < m && c <= r ? L[(int64_t)(I * kB + c) * ldl + row] : 0.0;
+    }
+    // row r of d or g times a vector in shared memory
+    auto times = [&](const double (&v)[kN], const double *w) {
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < kN; k += 2) {
+            s0 = fma(v[k], w[q + kQ * k], s0);
+            s1 = fma(v[k + 1], w[q + kQ * (k + 1)], s1);
+        }
+        return reduce(s0 + s1);
+    };
+    auto block_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(o + 1), "n"(kThreads / kOwn) : "memory"); };
     load(0, a[0]);
     load(1, a[1]);
     cl.sync();  // every CTA has started (its shared memory is written below)
     auto step = [&](int b, double (&v)[kN]) {
         if (b == I) {  // uniform over the warps of the block's threads
-            double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-            for (int k = 0; k < kN; k += 2) {
-                s0 = fma(d[k], rhs[o][q + kQ * k], s0);
-                s1 = fma(d[k + 1], rhs[o][q + kQ * (k + 1)], s1);
-            }
-            const double s = reduce(s0 + s1);
+            const double s0 = times(d, rhs[o]);
+            if (q == 0) own[0][o][r] = s0;
+            block_sync();
+            const double t = times(g, own[0][o]);
+            if (q == 0) own[1][o][r] = rhs[o][r] - t;
+            block_sync();
+            const double s = s0 + times(d, own[1][o]);
 #pragma unroll
             for (int k = q; k < kCl; k += kQ) cl.map_shared_rank(&xs[b & 1][0], k)[r] = s;
             if (q == 0 && row < m) x[row] = s;
         }
         cl.sync();
         if (b < I) {
-            const double *w = xs[b & 1];
-            double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-            for (int k = 0; k < kN; k += 2) {
-                s0 = fma(v[k], w[q + kQ * k], s0);
-                s1 = fma(v[k + 1], w[q + kQ * (k + 1)], s1);
-            }
-            const double s = reduce(s0 + s1);
+            const double s = times(v, xs[b & 1]);
             if (q == 0) rhs[o][r] -= s;
         }
         load(b + 2, v);

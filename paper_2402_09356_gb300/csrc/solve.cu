@@ -13,7 +13,7 @@
 //   k_pair_sub  y_i -= U_ik c_ik for all i > k.
 // The product L w has no chain: one launch of k_pair_dots over all tiles, one
 // of k_row_sums.  All descriptors go up once per call.  n = 20,000, tile 800: solve
-// 42.4 -> 2.58 ms (k_trsv 77 us a tile, the two others 10 each), L w 1.46 -> 0.11.
+// 42.4 -> 2.74 ms (k_trsv 84 us a tile, the two others 10 each), L w 1.46 -> 0.11.
 #include <algorithm>
 #include <mutex>
 
@@ -128,13 +128,17 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
         d[k] = I < nblk ? inv[(int64_t)I * kB * kB + r * kB + c] : 0.0;
         g[k] = row < m && c <= r ? L[(int64_t)(I * kB + c) * ldl + row] : 0.0;
     }
-    // row r of d or g times a vector in shared memory
-    auto times = [&](const double (&v)[kN], const double *w) {
+    // the thread's row of a block times entries 0 .. last of a vector in shared
+    // memory (the others count as zero whatever they hold: an infinite or NaN
+    // entry of the right-hand side leaves the rows above it as they are)
+    auto times = [&](const double (&v)[kN], const double *w, int last) {
         double s0 = 0.0, s1 = 0.0;
 #pragma unroll
         for (int k = 0; k < kN; k += 2) {
-            s0 = fma(v[k], w[q + kQ * k], s0);
-            s1 = fma(v[k + 1], w[q + kQ * (k + 1)], s1);
+            const int c = q + kQ * k;
+            const double w0 = w[c], w1 = w[c + kQ];  // loaded whatever c is: a load behind a test is a branch
+            s0 = fma(v[k], c <= last ? w0 : 0.0, s0);
+            s1 = fma(v[k + 1], c + kQ <= last ? w1 : 0.0, s1);
         }
         return reduce(s0 + s1);
     };
@@ -144,20 +148,21 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
     cl.sync();  // every CTA has started (its shared memory is written below)
     auto step = [&](int b, double (&v)[kN]) {
         if (b == I) {  // uniform over the warps of the block's threads
-            const double s0 = times(d, rhs[o]);
+            const double s0 = times(d, rhs[o], r);
             if (q == 0) own[0][o][r] = s0;
             block_sync();
-            const double t = times(g, own[0][o]);
+            const double t = times(g, own[0][o], r);
             if (q == 0) own[1][o][r] = rhs[o][r] - t;
             block_sync();
-            const double s = s0 + times(d, own[1][o]);
+            const double e = times(d, own[1][o], r);
+            const double s = (__double2hiint(e) & 0x7FF00000) != 0x7FF00000 ? s0 + e : s0;
 #pragma unroll
             for (int k = q; k < kCl; k += kQ) cl.map_shared_rank(&xs[b & 1][0], k)[r] = s;
             if (q == 0 && row < m) x[row] = s;
         }
         cl.sync();
         if (b < I) {
-            const double s = times(v, xs[b & 1]);
+            const double s = times(v, xs[b & 1], kB);
             if (q == 0) rhs[o][r] -= s;
         }
         load(b + 2, v);

@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "per_device.cuh"
 #include "tlr_internal.cuh"
 
 namespace tlr {
@@ -1013,14 +1014,14 @@ __global__ void __launch_bounds__(kMmThreads) k_maxmin_cluster(const double *__r
     }
 }
 
-// Whether clusters of 16 CTAs of the kernels above run on this device.
+// Whether clusters of 16 CTAs of the kernels above run on the current device.
 static bool cluster_order_ok() {
-    static std::once_flag once;
-    static bool ok = false;
-    std::call_once(once, [] {
-        int dev = 0, optin = 0;
-        ok = cudaGetDevice(&dev) == cudaSuccess &&
-             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+    static PerDevice<bool> per_device;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    return per_device.get(dev, [dev] {
+        int optin = 0;
+        bool ok = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
              cudaFuncSetAttribute(k_kd_bottom, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(KdShared)) == cudaSuccess;
         cudaFuncAttributes fa;
         ok = ok && cudaFuncGetAttributes(&fa, k_maxmin_cluster) == cudaSuccess &&
@@ -1046,8 +1047,8 @@ static bool cluster_order_ok() {
              fits((const void *)k_kd_top, kOrdThreads, 0) &&
              fits((const void *)k_maxmin_cluster, kMmThreads, maxmin_bytes(kMaxminClusterN));
         cudaGetLastError();  // clear any error of the queries
+        return ok;
     });
-    return ok;
 }
 
 // ------------------------------------------------------------- drivers

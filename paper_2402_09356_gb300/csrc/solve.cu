@@ -15,12 +15,12 @@
 // of k_row_sums.  All descriptors go up once per call.  n = 20,000, tile 800: solve
 // 42.4 -> 2.74 ms (k_trsv 84 us a tile, the two others 10 each), L w 1.46 -> 0.11.
 #include <algorithm>
-#include <mutex>
 
 #include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "dense.cuh"
+#include "per_device.cuh"
 #include "tlr_internal.cuh"
 
 namespace tlr {
@@ -320,10 +320,13 @@ const void *upload(tlr_ctx *ctx, cudaStream_t s, const void *data, size_t bytes,
     return own.as<char>();
 }
 
+// Whether clusters of 16 CTAs of k_trsv run on the current device.
 bool trsv16_ok() {
-    static std::once_flag once;
-    static bool ok = false;
-    std::call_once(once, [] {
+    static PerDevice<bool> per_device;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    return per_device.get(dev, [] {
+        bool ok = false;
         if (cudaFuncSetAttribute(k_trsv<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(16);
@@ -339,8 +342,8 @@ bool trsv16_ok() {
             ok = cudaOccupancyMaxActiveClusters(&nc, k_trsv<16>, &cfg) == cudaSuccess && nc > 0;
         }
         cudaGetLastError();  // clear any error of the queries
+        return ok;
     });
-    return ok;
 }
 
 // Pairs a launch's grid may hold in its second dimension.

@@ -7,11 +7,13 @@
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
+#include <initializer_list>
 #include <utility>
 #include <string>
 #include <vector>
 
 #include "../../include/tlr.h"
+#include "stage_ring.cuh"
 
 namespace tlr {
 
@@ -245,7 +247,9 @@ inline int tile_rows(int64_t n, int nb, int t) {
 
 // Copies `bytes` of host data into the staging ring of stream `s` (one ring
 // per internal stream, ring 0 for the caller's) and returns the device address
-// of the copy (stream ordered on `s`).
+// of the copy (stream ordered on `s`).  A launch that reads several arrays asks
+// for the room of all of them (stage_room) before the first.
+void stage_room(tlr_ctx *ctx, cudaStream_t s, std::initializer_list<size_t> sizes);
 void *stage_push(tlr_ctx *ctx, const void *data, size_t bytes, cudaStream_t s);
 
 // Status word helpers (host side).

@@ -1595,6 +1595,9 @@ static void launch_classes(tlr_ctx *ctx, cudaStream_t st, std::vector<LaunchClas
         return a->csize > b->csize;
     });
     // descriptors go up on the calling stream, before the fork
+    size_t bytes = 0;
+    for (auto *c : use) bytes += ring_bytes(c->jobs.size() * sizeof(Job));
+    stage_room(ctx, st, {bytes});
     std::vector<const Job *> dj;
     for (auto *c : use) dj.push_back((const Job *)stage_push(ctx, c->jobs.data(), c->jobs.size() * sizeof(Job), st));
     if (use.empty()) return;

@@ -8,20 +8,26 @@
 
 namespace tlr {
 
-void *stage_push(tlr_ctx *ctx, const void *data, size_t bytes, cudaStream_t s) {
+void stage_room(tlr_ctx *ctx, cudaStream_t s, std::initializer_list<size_t> sizes) {
     StageRing &R = ctx->stage[stage_ring(ctx, s)];
-    size_t need = (bytes + 255) & ~(size_t)255;
-    if (need > R.cap) throw make_error(TLR_ERR_ARG, "descriptor batch too large (%zu bytes)", bytes);
-    if (R.off + need > R.cap) {
-        // every reader of this ring runs on `s`
-        TLR_CUDA_TRY(cudaStreamSynchronize(s));
-        R.off = 0;
+    bool restart = false;
+    if (!ring_room(R.cap, R.off, sizes, restart)) {
+        size_t bytes = 0;
+        for (size_t b : sizes) bytes += b;
+        throw make_error(TLR_ERR_ARG, "descriptor batch too large (%zu bytes)", bytes);
     }
+    // every reader of this ring runs on `s`
+    if (restart) TLR_CUDA_TRY(cudaStreamSynchronize(s));
+}
+
+void *stage_push(tlr_ctx *ctx, const void *data, size_t bytes, cudaStream_t s) {
+    stage_room(ctx, s, {bytes});
+    StageRing &R = ctx->stage[stage_ring(ctx, s)];
     char *h = R.h + R.off;
     char *d = R.d + R.off;
     std::memcpy(h, data, bytes);
     TLR_CUDA_TRY(cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, s));
-    R.off += need;
+    R.off += ring_bytes(bytes);
     return d;
 }
 
@@ -37,6 +43,7 @@ static void launch_shape(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const s
     }
     int total = off.back();
     if (total == 0) return;
+    stage_room(ctx, s, {probs.size() * sizeof(GemmProb), off.size() * sizeof(int)});
     auto *dp = (const GemmProb *)stage_push(ctx, probs.data(), probs.size() * sizeof(GemmProb), s);
     auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
     int np = (int)probs.size();
@@ -58,6 +65,7 @@ static void launch_gemv(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const st
         off[b + 1] = off[b] + (probs[b].m > 0 ? (int)ceil_div(probs[b].m, kGemvRows) : 0);
     int total = off.back();
     if (total == 0) return;
+    stage_room(ctx, s, {probs.size() * sizeof(GemmProb), off.size() * sizeof(int)});
     auto *dp = (const GemmProb *)stage_push(ctx, probs.data(), probs.size() * sizeof(GemmProb), s);
     auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
     int np = (int)probs.size();
@@ -88,6 +96,7 @@ static void launch_gemm(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const st
     while (tnmax > 1 && count(tnmax) < 2 * ctx->num_sms) tnmax /= 2;
     std::vector<int> off(fit.size() + 1, 0);
     for (size_t b = 0; b < fit.size(); ++b) off[b + 1] = off[b] + fit_tiles(fit[b].m, fit[b].n, tnmax);
+    stage_room(ctx, s, {fit.size() * sizeof(GemmProb), off.size() * sizeof(int)});
     auto *dp = (const GemmProb *)stage_push(ctx, fit.data(), fit.size() * sizeof(GemmProb), s);
     auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
     (df ? gemm_fit_df : gemm_fit_f64)(s, ta, tb, off.back(), dp, dt, (int)fit.size(), tnmax, alpha, beta);
@@ -167,6 +176,7 @@ static void launch_matern(tlr_ctx *ctx, cudaStream_t s, const std::vector<GemmPr
         off[b + 1] = off[b] + ((big[b].m > 0 && big[b].n > 0) ? (int)(ceil_div(big[b].m, 64) * ceil_div(big[b].n, 64)) : 0);
     int total = off.back();
     if (total == 0) return;
+    stage_room(ctx, s, {big.size() * sizeof(GemmProb), off.size() * sizeof(int)});
     auto *dp = (const GemmProb *)stage_push(ctx, big.data(), big.size() * sizeof(GemmProb), s);
     auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
     int np = (int)big.size();

@@ -723,6 +723,7 @@ void launch_tc(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector
         off[b + 1] = off[b] + (int)(ceil_div(p.m, kBM) * ceil_div(p.n, kBN));
     }
     const int total = off.back();
+    stage_room(ctx, s, {tp.size() * sizeof(TcProb), off.size() * sizeof(int)});
     auto *dp = (const TcProb *)stage_push(ctx, tp.data(), tp.size() * sizeof(TcProb), s);
     auto *dt = (const int *)stage_push(ctx, off.data(), off.size() * sizeof(int), s);
     if (ctas_per_sm > 0) {

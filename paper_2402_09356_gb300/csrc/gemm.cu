@@ -158,7 +158,15 @@ void gemm_batched_small(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const st
 
 void gemm_batched(tlr_ctx *ctx, cudaStream_t s, bool ta, bool tb, const std::vector<GemmProb> &probs,
                   double alpha, double beta, bool df) {
-    launch_gemm(ctx, s, ta, tb, probs, alpha, beta, df);
+    // what the descriptor ring does not hold at once goes in parts
+    const size_t most = (ctx->stage[stage_ring(ctx, s)].cap - 1024) / (sizeof(GemmProb) + sizeof(int));
+    if (probs.size() <= most) {
+        launch_gemm(ctx, s, ta, tb, probs, alpha, beta, df);
+        return;
+    }
+    for (size_t b = 0; b < probs.size(); b += most)
+        launch_gemm(ctx, s, ta, tb, std::vector<GemmProb>(probs.begin() + b, probs.begin() + std::min(probs.size(), b + most)),
+                    alpha, beta, df);
 }
 
 // The panel update is one large product: 64 x 64 tiles.  A capped grid

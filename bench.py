@@ -404,7 +404,8 @@ def run_gpu(args):
                 "frac_of_occupied_sms": achieved / occupied if occupied else None,
                 "clusters_per_launch": clusters, "launch_ms_avg": avg, "launches": k["jacobi16_launches"],
                 "flops_per_launch": fl, "total_ms": k["jacobi16_ms"],
-                "flops_counted": "FP32 sweeps: norms (2 s^2), a dot product (2 s) and a rotation (12 s) per pair"}
+                "flops_counted": "FP32 sweeps as executed: norms (2 s^2), a dot product (2 s) per pair checked, "
+                                 "a rotation (12 s) per pair rotated"}
 
     def roof_potrf(o):
         # per tile column on the side stream: L = chol(T_jj) (the algorithmic

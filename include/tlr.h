@@ -443,9 +443,10 @@ int tlr_compress_stats(tlr_ctx *ctx, int64_t *out);
 /* The cluster Jacobi SVD on 16-CTA clusters (the high-rank tiles next to the
  * diagonal) during the last profiled factorisation, written to out[0..3]:
  * device time (ms, CUDA events on its stream, summed over launches), FP32
- * floating-point operations of its preconditioning sweeps (the column norms,
- * and for every pair a dot product and a rotation of two columns), number of
- * launches, and number of clusters (tiles) over those launches.  Errors: TLR_ERR_ARG. */
+ * floating-point operations of its preconditioning sweeps as executed (the
+ * column norms, a dot product for every pair checked, a rotation of two columns
+ * for every pair rotated), number of launches, and number of clusters (tiles)
+ * over those launches.  Errors: TLR_ERR_ARG. */
 int tlr_kernel_stats(tlr_ctx *ctx, double *out);
 
 /* ---- MLE (Sec. 5.1: derivative-free, bound-constrained) ------------------ */

@@ -647,7 +647,7 @@ struct SvdJob {
     double *W;         // s x s output: unit left singular vectors of R', sorted
     double *S;         // s output singular values, descending
     int *rank;         // #{S > tau}, or -1 if any S is not finite
-    int *sweeps;       // [0] FP64 sweeps, [1] FP32 sweeps, [2] FP64 pairs checked, [3] FP64 pairs rotated
+    int *sweeps;       // [0] FP64 sweeps, [1] FP32 sweeps, [2] FP32 pairs checked, [3] FP32 pairs rotated
     int s;
     double tau;        // absolute accuracy of the tile
     const float2 *Rt2; // R' as paired FP32 (the paired-FP32 precondition reads it), or null
@@ -1098,10 +1098,9 @@ __device__ __forceinline__ void jacobi_emit(const SvdJob &J, const double *cols,
     }
 }
 
-__device__ void jacobi_rank(const SvdJob &J, const double *all_nrm, int sweeps, int sweeps32) {
+// FP64 sweeps and rank; the counts of the FP32 sweeps before stay.
+__device__ void jacobi_rank(const SvdJob &J, const double *all_nrm, int sweeps) {
     J.sweeps[0] = sweeps;
-    J.sweeps[1] = sweeps32;
-    J.sweeps[2] = J.sweeps[3] = 0;
     int r = 0;
     bool bad = false;
     for (int u = 0; u < J.s; ++u) {
@@ -1140,7 +1139,7 @@ __global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jaco
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     __shared__ int s_flag[2];
-    __shared__ int s_tally[2];  // FP64 phase: pairs checked, pairs rotated (this CTA)
+    __shared__ int s_tally[2];  // FP32 sweeps: pairs checked, pairs rotated (the cluster's, in CTA 0)
     extern __shared__ double sm[];
     const SvdJob J = jobs[blockIdx.x / kCl];
     const int s = J.s, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
@@ -1150,7 +1149,7 @@ __global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jaco
     if (tid == 0) s_tally[0] = s_tally[1] = 0;
     double *nrm_loc = sm + 2 * stride, *all_nrm = nrm_loc + 2 * b;
     const int px = rank, py = nblk - 1 - rank;
-    int g = 0, cur = 0, sw32 = 0;
+    int g = 0, cur = 0;
     if constexpr (kMode == kJacPrecond) {
     // A. FP32 phase (the same buffers hold b x 2s floats per block)
     float *f0 = reinterpret_cast<float *>(sm);
@@ -1169,7 +1168,8 @@ __global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jaco
         }
     }
     __syncthreads();
-    sw32 = jacobi_sweeps<kCl, float>(cl, f0, stride_f, b, s, s2, kMaxSweeps32, g, cur, s_flag);
+    const int sw32 = jacobi_sweeps<kCl, float>(cl, f0, stride_f, b, s, s2, kMaxSweeps32, g, cur, s_flag,
+                                               cl.map_shared_rank(s_tally, 0));
     // B. J's held columns, as doubles or (paired paths) pairs, for the product
     // M1 = M J that follows as a batched GEMM over the whole GPU (formed here, on
     // the cluster's SMs, it took 130 us at s = 200 in pairs and more in FP64)
@@ -1182,12 +1182,13 @@ __global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jaco
         if (J.Rt2) reinterpret_cast<float2 *>(J.rot)[(int64_t)u * s + k] = make_float2(v, 0.f);
         else J.rot[(int64_t)u * s + k] = (double)v;
     }
+    cl.sync();  // no CTA leaves while another may still read its blocks or flag
     if (rank == 0 && tid == 0) {
         J.sweeps[0] = 0;
         J.sweeps[1] = sw32;
-        J.sweeps[2] = J.sweeps[3] = 0;
+        J.sweeps[2] = s_tally[0];
+        J.sweeps[3] = s_tally[1];
     }
-    cl.sync();  // no CTA leaves while another may still read its blocks or flag
     } else {
     // C. FP64 phase on M1, starting from the same block positions
     for (int slot = 0; slot < 2; ++slot) {
@@ -1200,7 +1201,7 @@ __global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jaco
     }
     __syncthreads();
     cur = 0;
-    const int sw64 = jacobi_sweeps<kCl, double>(cl, sm, stride, b, s, s, kMaxSweeps, g, cur, s_flag, s_tally);
+    const int sw64 = jacobi_sweeps<kCl, double>(cl, sm, stride, b, s, s, kMaxSweeps, g, cur, s_flag);
     double *D = sm + cur * stride;
     const int gx = block_at(px, g, nblk), gy = block_at(py, g, nblk);
     for (int q = warp; q < 2 * b; q += nt >> 5) {
@@ -1218,17 +1219,8 @@ __global__ void __launch_bounds__(kCl == 16 ? 32 * kJacWarps : kJacBound) k_jaco
     }
     __syncthreads();
     jacobi_emit(J, D, gx, gy, b, all_nrm, lane, warp);
-    if (rank == 0 && tid == 0) {
-        jacobi_rank(J, all_nrm, sw64, sw32);
-        int chk = 0, rot = 0;
-        for (int k = 0; k < kCl; ++k) {
-            chk += cl.map_shared_rank(s_tally, k)[0];
-            rot += cl.map_shared_rank(s_tally, k)[1];
-        }
-        J.sweeps[2] = chk;
-        J.sweeps[3] = rot;
-    }
-    cl.sync();  // no CTA leaves while another may still read its norms or tallies
+    if (rank == 0 && tid == 0) jacobi_rank(J, all_nrm, sw64);
+    cl.sync();  // no CTA leaves while another may still read its norms
     }
 }
 
@@ -1426,7 +1418,10 @@ __global__ void __launch_bounds__(kQrThreads) k_jacobi_gm(const SvdJob *__restri
     }
     __syncthreads();
     jacobi_emit(J, Ab, gx, gy, b, all_nrm, lane, warp);
-    if (rank == 0 && tid == 0) jacobi_rank(J, all_nrm, nsweep, 0);
+    if (rank == 0 && tid == 0) {
+        J.sweeps[1] = J.sweeps[2] = J.sweeps[3] = 0;
+        jacobi_rank(J, all_nrm, nsweep);
+    }
     cl.sync();  // no CTA leaves while another may still read its flag
 }
 
@@ -2001,9 +1996,9 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
             ctx->comp_stats[4] += sw[1];
         }
         if (ctx->profile && t16.csize == 16) {
-            // FP32 work of the 16-CTA Jacobi launch: per sweep the norms (2 s^2)
-            // and, for each of s (s - 1) / 2 pairs, a dot product (2 s) and a
-            // rotation of two columns of 2 s (12 s)
+            // FP32 work of the 16-CTA Jacobi launch as executed: per sweep the
+            // norms (2 s^2), a dot product (2 s) for every pair checked, a
+            // rotation of two columns of 2 s (12 s) for every pair rotated
             float ms = 0.f;
             TLR_CUDA_TRY(cudaEventElapsedTime(&ms, t16.e0, t16.e1));
             double fl = 0.0;
@@ -2012,7 +2007,7 @@ void compress_jobs(tlr_ctx *ctx, cudaStream_t st, std::vector<CompressJob> &jobs
                 if (svd_csize[u] != 16) continue;
                 const int *sw = h_rank.data() + np + 4 * u;
                 const double s = ps[u];
-                fl += sw[1] * (2.0 * s * s + 7.0 * s * s * (s - 1.0));
+                fl += 2.0 * s * s * sw[1] + 2.0 * s * sw[2] + 12.0 * s * sw[3];
                 ++jobs16;
             }
             ctx->k16_ms += ms;

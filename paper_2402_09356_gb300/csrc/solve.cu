@@ -7,13 +7,14 @@
 // diagonal tile block by block.  Per tile column three launches:
 //   k_trsv      y_k <- L_kk^-1 y_k, one cluster, blocks of 32 rows whose
 //               inverses were formed for all tiles by one launch at the start
-//               (k_inv_blocks: a block's substitution is then three 32 x 32
-//               products, not 32 dependent steps);
+//               (k_inv_blocks: a block's substitution is then one 32 x 32
+//               product, three where its condition asks for a residual step,
+//               not 32 dependent steps);
 //   k_pair_dots c_ik = V_ik' y_k for all i > k, one warp a column of V;
 //   k_pair_sub  y_i -= U_ik c_ik for all i > k.
 // The product L w has no chain: one launch of k_pair_dots over all tiles, one
 // of k_row_sums.  All descriptors go up once per call.  n = 20,000, tile 800: solve
-// 42.4 -> 2.74 ms (k_trsv 84 us a tile, the two others 10 each), L w 1.46 -> 0.11.
+// 42.4 -> 2.03 ms (k_trsv 55 us a tile, the two others 10 each), L w 1.46 -> 0.11.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -47,13 +48,21 @@ __device__ __forceinline__ int rows_of(int64_t n, int nb, int t) {
     return (int)(r < nb ? r : nb);
 }
 
-// Inverses of the 32 x 32 diagonal blocks (row major, zero right of the
+// Inverses X of the 32 x 32 diagonal blocks L (row major, zero right of the
 // diagonal and past the tile) of every diagonal tile: one CTA a block.
 // Column by column, M <- the elimination applied to the identity: row c is
 // scaled by 1 / L_cc, the rows below it subtract their multiple.
+// `fix`: whether a product with X needs its residual step in k_trsv, from the
+// block's condition k = max_r (|X| |L| e)_r.  A product's error is up to k times
+// substitution's; measured against extended precision over 640 blocks (nu 0.4
+// to 2.5, beta 0.03 to 0.12) it is 0.6 to 0.7 times as large for k of 8 to 16,
+// 0.8 to 0.9 for 16 to 32, 1.1 to 1.3 for 32 to 64, 1.9 to 2.2 for 64 to 128, 5 to 7 for 256
+// to 1,024.  nu = 0.5: k is 16 in the middle, nu = 2.5: 520.
+constexpr double kPlainCond = 24.0;
 __global__ void __launch_bounds__(kThreads) k_inv_blocks(const double *__restrict__ D, int64_t n, int nb, int per_tile,
-                                                          double *__restrict__ inv) {
+                                                          double *__restrict__ inv, int *__restrict__ fix) {
     __shared__ double L[kB][kB + 1], M[kB][kB + 1], rd[kB];
+    __shared__ int s_fix;
     const int t = blockIdx.x / per_tile, b = blockIdx.x % per_tile, tid = threadIdx.x;
     const int m = rows_of(n, nb, t), p = b * kB, w = min(kB, m - p);
     double *out = inv + (int64_t)blockIdx.x * kB * kB;
@@ -66,6 +75,7 @@ __global__ void __launch_bounds__(kThreads) k_inv_blocks(const double *__restric
     }
     __syncthreads();
     if (tid < w) rd[tid] = 1.0 / L[tid][tid];
+    if (tid == 0) s_fix = 0;
     __syncthreads();
     const int r = tid >> 3, q = tid & 7;
     for (int c = 0; c < w; ++c) {
@@ -83,24 +93,42 @@ __global__ void __launch_bounds__(kThreads) k_inv_blocks(const double *__restric
         const int i = e / kB, c = e % kB;
         out[e] = i < w && c <= i ? M[i][c] : 0.0;
     }
+    // the condition, eight lanes a row
+    auto row_sum = [](double v) {
+#pragma unroll
+        for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        return v;
+    };
+    double v = 0.0;
+    for (int c = q; c <= r; c += 8) v += fabs(L[r][c]);
+    v = row_sum(v);
+    if (q == 0) rd[r] = v;
+    __syncthreads();
+    v = 0.0;
+    for (int c = q; c <= r; c += 8) v = fma(fabs(M[r][c]), rd[c], v);
+    v = row_sum(v);
+    if (r < w && !(v <= kPlainCond)) s_fix = 1;
+    __syncthreads();
+    if (tid == 0) fix[blockIdx.x] = s_fix;
 }
 
 // x <- L^-1 x for one diagonal tile (m <= 1024, ld ldl) by one cluster: CTA
 // `rank` owns the blocks rank, rank + kCl, ... of the right-hand side, each
 // kept by kThreads / kOwn threads (four or two a row).  Step b: the owner
 // multiplies its block by the block's inverse, corrects the product by its
-// residual, y += L_bb^-1 (x - L_bb y), and stores the 32 values into every CTA;
-// after one cluster barrier every CTA subtracts L's block column b times them
-// from its blocks.  (The product alone is as far off as |L^-1| |x| lets it be:
-// right-hand sides of a smooth field, whose y is far smaller, had 2 to 50 times
-// the error of substitution; one residual step leaves none of that, for 26 us
-// more a tile of 800.)  The
-// entries of block columns b + 1 and b + 2 are on their way to registers
-// meanwhile (the tile comes from HBM).  Bound by the chain of a step: barrier,
-// update of the next block, its three products.
+// residual, y += L_bb^-1 (x - L_bb y), where fix[b] asks for it, and stores the
+// 32 values into every CTA; after one cluster barrier every CTA subtracts L's
+// block column b times them from its blocks.  (Without the correction the
+// right-hand sides of a smooth field, whose y is far smaller than |L^-1| |x|, had
+// 2 to 50 times the error of substitution; with it, none of that.  It takes 36
+// us of a tile of 800 if every block asks.)  The entries of block columns b + 1
+// and b + 2 are on their way to registers meanwhile (the tile comes from HBM).
+// Bound by the chain of a step: barrier, update of the next block, its product
+// or three.
 template <int kCl>
 __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L, int ldl, int m,
-                                                    const double *__restrict__ inv, double *__restrict__ x) {
+                                                    const double *__restrict__ inv, const int *__restrict__ fix,
+                                                    double *__restrict__ x) {
     constexpr int kOwn = kB / kCl;                 // blocks a CTA: at most 32 blocks in a tile
     constexpr int kQ = kThreads / kOwn / kB;       // threads a row
     constexpr int kN = kB / kQ;                    // columns a thread
@@ -110,6 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
     const int I = rank + o * kCl, row = I * kB + r;  // the thread's block and row
     __shared__ double rhs[kOwn][kB], own[2][kOwn][kB], xs[2][kB];
     const int nblk = (m + kB - 1) / kB;
+    const bool correct = I < nblk && fix[I];  // the same for the block's threads
     if (q == 0) rhs[o][r] = row < m ? x[row] : 0.0;
     double a[2][kN], d[kN], g[kN];
     auto load = [&](int b, double (&v)[kN]) {  // L's block column b in the thread's row
@@ -126,7 +155,7 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
     for (int k = 0; k < kN; ++k) {  // row r of the block's inverse and of the block
         const int c = q + kQ * k;
         d[k] = I < nblk ? inv[(int64_t)I * kB * kB + r * kB + c] : 0.0;
-        g[k] = row < m && c <= r ? L[(int64_t)(I * kB + c) * ldl + row] : 0.0;
+        g[k] = correct && row < m && c <= r ? L[(int64_t)(I * kB + c) * ldl + row] : 0.0;
     }
     // the thread's row of a block times entries 0 .. last of a vector in shared
     // memory (the others count as zero whatever they hold: an infinite or NaN
@@ -148,14 +177,16 @@ __global__ void __launch_bounds__(kThreads) k_trsv(const double *__restrict__ L,
     cl.sync();  // every CTA has started (its shared memory is written below)
     auto step = [&](int b, double (&v)[kN]) {
         if (b == I) {  // uniform over the warps of the block's threads
-            const double s0 = times(d, rhs[o], r);
-            if (q == 0) own[0][o][r] = s0;
-            block_sync();
-            const double t = times(g, own[0][o], r);
-            if (q == 0) own[1][o][r] = rhs[o][r] - t;
-            block_sync();
-            const double e = times(d, own[1][o], r);
-            const double s = (__double2hiint(e) & 0x7FF00000) != 0x7FF00000 ? s0 + e : s0;
+            double s = times(d, rhs[o], r);
+            if (correct) {
+                if (q == 0) own[0][o][r] = s;
+                block_sync();
+                const double t = times(g, own[0][o], r);
+                if (q == 0) own[1][o][r] = rhs[o][r] - t;
+                block_sync();
+                const double e = times(d, own[1][o], r);
+                if ((__double2hiint(e) & 0x7FF00000) != 0x7FF00000) s += e;
+            }
 #pragma unroll
             for (int k = q; k < kCl; k += kQ) cl.map_shared_rank(&xs[b & 1][0], k)[r] = s;
             if (q == 0 && row < m) x[row] = s;
@@ -364,13 +395,18 @@ void forward_solve(tlr_ctx *ctx, cudaStream_t st, const tlr_mat *M, const double
     DevBuf inv((size_t)nt * per_tile * kB * kB * sizeof(double), st);
     DevBuf cb((size_t)std::max<int64_t>(L.total, 1) * sizeof(double), st), part((size_t)2 * nt * sizeof(double), st);
     double *c = cb.as<double>();
-    launch(k_inv_blocks, (unsigned)(nt * per_tile), kThreads, 0, st, M->D, n, nb, per_tile, inv.as<double>());
+    DevBuf fixb((size_t)nt * per_tile * sizeof(int), st);
+    launch(k_inv_blocks, (unsigned)(nt * per_tile), kThreads, 0, st, M->D, n, nb, per_tile, inv.as<double>(),
+           fixb.as<int>());
     TLR_CHECK_LAUNCH();
     const bool big = trsv16_ok();
     for (int k = 0; k < nt; ++k) {
         const double *D = M->D + (int64_t)k * nb * nb, *Di = inv.as<double>() + (int64_t)k * per_tile * kB * kB;
-        if (big) launch_clustered(k_trsv<16>, 16, 1, kThreads, 0, st, D, nb, tile_rows(n, nb, k), Di, y + (int64_t)k * nb);
-        else launch_clustered(k_trsv<8>, 8, 1, kThreads, 0, st, D, nb, tile_rows(n, nb, k), Di, y + (int64_t)k * nb);
+        const int *fix = fixb.as<int>() + (int64_t)k * per_tile;
+        if (big) launch_clustered(k_trsv<16>, 16, 1, kThreads, 0, st, D, nb, tile_rows(n, nb, k), Di, fix,
+                                  y + (int64_t)k * nb);
+        else launch_clustered(k_trsv<8>, 8, 1, kThreads, 0, st, D, nb, tile_rows(n, nb, k), Di, fix,
+                                  y + (int64_t)k * nb);
         const int p1 = L.first[(size_t)k + 1];
         for (int p = L.first[(size_t)k]; p < p1; p += kMaxGridY) {
             const unsigned cnt = (unsigned)std::min(kMaxGridY, p1 - p);

@@ -5,7 +5,8 @@
 // factors satisfy T ~ U V' with |T - U V'|_2 ~ sigma_{r+1}.  Computing the
 // full SVD of every nb x nb tile would cost O(nb^3); instead, per tile:
 //   1. Y = T Omega (Omega: k x s Gaussian) by batched GEMM (whole GPU);
-//   2. Q = orth(Y): Householder QR with the explicit Q formed in place;
+//   2. Q = orth(Y): Householder QR (k_qr_factor), Q formed from its reflectors
+//      (k_qr_form);
 //   3. B = T' Q (batched GEMM), kept, and the R factor of B = Q2 R;
 //   4. one-sided Jacobi SVD of R' = W S Z' (only W and S are formed).
 // With the unit left singular vectors W of R' (the right singular vectors
@@ -24,8 +25,9 @@
 // is slow, and the highest-rank tile of a column lies on the critical path of
 // the factorisation.  Each tile therefore runs on a thread-block cluster whose
 // CTAs keep their share of the tile in shared memory:
-//   - QR: the CTAs split the rows; per column one cluster barrier exchanges
-//     the partial dot products through distributed shared memory (DSMEM);
+//   - QR: the CTAs split the rows; per column the partial dot products are
+//     summed and spread through distributed shared memory (DSMEM), a cluster
+//     barrier before and after;
 //   - SVD: the columns of R' form 2C blocks; every CTA rotates the column
 //     pairs between (and, once per sweep, within) its two blocks and then
 //     pulls its next two blocks from their holders over DSMEM, following a
@@ -54,7 +56,9 @@ constexpr int kSpare = 20;       // fewer spare samples than this: redo with mor
 constexpr int kQrThreads = 256;
 constexpr int kNw = kQrThreads / 32;
 // Block Jacobi: up to kJacWarps warps a CTA (jacobi_threads); the bound leaves
-// 96 registers, with which two CTAs of 10 warps fit an SM.
+// 96 registers, with which two CTAs of 10 warps fit an SM.  The FP32 kernels of
+// 1 to 8 CTAs then spill 44 to 124 bytes a thread around their calls of the
+// rotation (which spills nothing), the FP64 one of 16 CTAs 184.
 constexpr int kJacWarps = 16;
 constexpr int kJacBound = 640;
 constexpr int kQrSmThreads = 512;
@@ -147,19 +151,16 @@ struct QrArith<false> {
     static __device__ __forceinline__ T from(double x) { return x; }
     static __device__ __forceinline__ double to(T x) { return x; }
     static __device__ __forceinline__ void acc(Acc &a, T x, T y) { a.d = fma(x, y, a.d); }
-    static __device__ __forceinline__ double val(const Acc &a) { return a.d; }
-    // a - w v, with w prepared by prep()
+    // a - w v, with w prepared by prepP()
     struct W {
         double w;
     };
-    static __device__ __forceinline__ W prep(double w) { return W{w}; }
     static __device__ __forceinline__ T axmy(T a, const W &w, T v) { return fma(-w.w, v, a); }
     // per-column scalars
     using P = double;
     static __device__ __forceinline__ P part(const Acc &a) { return a.d; }
     static __device__ __forceinline__ P elem(T x) { return x; }
     static __device__ __forceinline__ P padd(P a, P b) { return a + b; }
-    static __device__ __forceinline__ P pmul(P a, P b) { return a * b; }
     static __device__ __forceinline__ bool nz(P a) { return a != 0.0; }
     static __device__ __forceinline__ W prepP(P w) { return W{w}; }
     static __device__ __forceinline__ T fromP(P x) { return x; }
@@ -177,19 +178,13 @@ struct QrArith<true> {
     }
     static __device__ __forceinline__ double to(T x) { return (double)x.x + (double)x.y; }
     static __device__ __forceinline__ void acc(Acc &a, T x, T y) { df_fma(x.x, x.y, y.x, y.y, a.h, a.l); }
-    static __device__ __forceinline__ double val(const Acc &a) { return (double)a.h + (double)a.l; }
     struct W {
         float h, l;
     };
-    static __device__ __forceinline__ W prep(double w) {
-        const float h = __double2float_rn(w);
-        return W{h, __double2float_rn(w - (double)h)};
-    }
     using P = FF;
     static __device__ __forceinline__ P part(const Acc &a) { return ff_two_sum(a.h, a.l); }
     static __device__ __forceinline__ P elem(T x) { return FF{x.x, x.y}; }
     static __device__ __forceinline__ P padd(P a, P b) { return ff_add(a, b); }
-    static __device__ __forceinline__ P pmul(P a, P b) { return ff_mul(a, b); }
     static __device__ __forceinline__ bool nz(P a) { return a.h != 0.f; }
     static __device__ __forceinline__ W prepP(P w) { return W{w.h, w.l}; }
     static __device__ __forceinline__ T fromP(P x) { return make_float2(x.h, x.l); }
@@ -781,9 +776,9 @@ __device__ __forceinline__ float rcp_approx32(float x) {
     return y;
 }
 // (c, s, t) of the rotation for zeta = (|y|^2 - |x|^2) / (2 x'y), from approximate
-// roots: (c, s) is orthogonal to FP32 accuracy whatever their error, so only
-// convergence depends on it.  h = 1 / sqrt(1 + zeta^2): c^2 = (1 + |zeta| h) / 2,
-// |s| = h / (2 c).
+// roots.  h = 1 / sqrt(1 + zeta^2): c^2 = (1 + |zeta| h) / 2, |s| = h / (2 c).  An
+// error e of h makes c^2 + s^2 - 1 between e / 2 and e, and e is at most 2^-22
+// (rsqrt.approx): orthogonal to FP32 accuracy because the roots are.
 __device__ __forceinline__ void jacobi_angle(float zeta, float az, float &c, float &sn, float &t) {
     const float h = rsqrt_approx32(fmaf(zeta, zeta, 1.0f)), c2 = fmaf(0.5f * az, h, 0.5f), rc = rsqrt_approx32(c2);
     c = c2 * rc;
@@ -1116,7 +1111,8 @@ constexpr int kMoreRounds = 2;   // rounds of two more steps for tiles they did 
 
 // Block Jacobi with the blocks in shared memory, in two precisions.
 //  A. FP32 sweeps on fl32(M), M = R', carrying the accumulated rotations J
-//     (each column holds s entries of M then s of J), until FP32 convergence.
+//     (each column holds s entries of M then s of J), until a sweep meets no
+//     cosine above kFinalCos = 3e-4: what is left is the FP64 refinement's.
 //  B. J is written out; M1 = M J follows as a GEMM (FP64, or paired FP32 from
 //     the paired copy of M: J is exact in FP32, and M1 then carries ~1e-14 of
 //     |M|, below the thresholds of those paths).
@@ -1633,7 +1629,11 @@ static void add_to_class(std::vector<LaunchClass<Job, K>> &cls, K kernel, int cs
 }
 
 // Q of every job of a class from its reflectors; rows in the smallest of the
-// register sizes that holds the class's tallest job.
+// register sizes that holds the class's tallest job.  Groups of 32 rows past
+// the tile cost as much as any: with 16 and 32 alone the QR of the sample took 6
+// to 8% longer in FP64 and 3 to 6% in pairs at tiles of 600 to 800.  Each size is
+// two kernels to compile, so that there are five, no step above 512 rows more
+// than a quarter.
 template <bool kDf>
 static void form_q(cudaStream_t st, const QrJob *d, const std::vector<QrJob> &jobs) {
     int cols = 0, rows = 0;

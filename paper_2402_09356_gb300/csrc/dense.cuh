@@ -7,9 +7,9 @@ namespace tlr {
 
 // A = L L' in place (lower; strict upper zeroed) and X = L^-1 (m x m, lower,
 // ld ldx), both in FP64; m <= 1024.  One launch on one thread-block cluster up
-// to 288 rows, in blocks with batched products between them above.  A
-// non-positive pivot sets NOT_SPD (info = row_base + local row); X is then
-// not written.
+// to 288 rows, in blocks with substitutions and batched products between them
+// above.  A non-positive pivot sets NOT_SPD (info = row_base + local row); X
+// then holds nothing of use.
 void potrf_inv(tlr_ctx *ctx, cudaStream_t s, double *A, int lda, int m, double *X, int ldx, long long row_base);
 
 // The same for several tiles, sharing every launch (one cluster each); every job

@@ -439,7 +439,9 @@ __global__ void k_fill(double *__restrict__ a, int64_t n, double v) {
 // barrier separates the phases.  40,000 locations with xy_out: Hilbert 123 -> 47
 // us, KD-tree 2,940 -> 177 us (sort 75, upper levels 70, subtrees 29); 10,000
 // locations by max-min 82 -> 15 ms.  Above kClusterMaxN the launches above take over (more
-// SMs share a pass).
+// SMs share a pass): their distance shrinks as n grows, 65,536 locations 162 -> 77
+// us by Hilbert and 3,560 -> 238 by KD-tree, 131,072 180 -> 97 and 5,390 -> 367,
+// 262,144 227 -> 144 and 9,330 -> 685 (launches -> cluster).
 constexpr int kOrdCl = 16, kOrdThreads = 1024, kOrdWarps = kOrdThreads / 32;
 constexpr int64_t kClusterMaxN = (int64_t)1 << 18;
 constexpr int kSortBatch = 4;  // keys a lane loads before it counts them
@@ -880,7 +882,10 @@ __global__ void __launch_bounds__(kOrdThreads) k_kd_bottom(const double *__restr
 // cycles a warp) is formed only where an FP32 box test cannot rule it out:
 // |dx| > r or |dy| > r with r above the square root of the minimum distance by
 // more than every rounding involved means that the distance is larger.  Steps
-// depend on one another: 1 us each, most of it the exchange.
+// depend on one another: 1.4 us each at n = 10,000, the chain of the FP64
+// distances of the points hit, the look at their neighbours and the reductions
+// (on one CTA, without the exchange, as long).  40,000 points 407 -> 78 ms,
+// 98,304 1,007 -> 292, where the points no longer fit the shared memory.
 constexpr int kMaxminClusterN = 98304;  // 36 bytes a point, 6,144 points a CTA
 constexpr int kMmThreads = 512, kMmWarps = kMmThreads / 32;
 struct MmCand {

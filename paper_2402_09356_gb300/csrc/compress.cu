@@ -1632,8 +1632,7 @@ static void add_to_class(std::vector<LaunchClass<Job, K>> &cls, K kernel, int cs
 // register sizes that holds the class's tallest job.  Groups of 32 rows past
 // the tile cost as much as any: with 16 and 32 alone the QR of the sample took 6
 // to 8% longer in FP64 and 3 to 6% in pairs at tiles of 600 to 800.  Each size is
-// two kernels to compile, so that there are five, no step above 512 rows more
-// than a quarter.
+// two kernels to compile, so that there are five, a quarter apart above 512 rows.
 template <bool kDf>
 static void form_q(cudaStream_t st, const QrJob *d, const std::vector<QrJob> &jobs) {
     int cols = 0, rows = 0;

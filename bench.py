@@ -410,22 +410,20 @@ def run_gpu(args):
     def roof_potrf(o):
         # per tile column on the side stream: L = chol(T_jj) (the algorithmic
         # m^3/3 FP64 flops) and L^-1 (another m^3/3, executed work that
-        # replaces the TRSM), in blocks of 288 rows with batched GEMMs between
-        # them; the in-step time from the events around it on that stream
+        # replaces the TRSM), in blocks of 288 rows with substitutions and
+        # batched GEMMs between them; the in-step time from the events around it on that stream
         nt = (N_POINTS + NB - 1) // NB
         ms_step = o["detail_ms"]["potrf"]
         avg = ms_step / nt
         ms = [min(NB, N_POINTS - t * NB) for t in range(nt)]
         fl = sum(m ** 3 / 3.0 for m in ms) / nt
         achieved = fl / (avg / 1000.0) / 1e12 if avg > 0 else 0.0
-        occupied = 16 * 4 * sm_mhz * 1e6 / 1e12
-        return {"bound": "alu", "kernel": "k_potrf_inv<16> and its block products (diagonal tile: Cholesky and "
+        return {"bound": "alu", "kernel": "k_potrf_inv<16>, k_potrf_sub and block products (diagonal tile: Cholesky and "
                                           "inverse in FP64; one 16-CTA cluster a block of 288 rows)",
                 "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
                 "frac": achieved / fp64_peak if fp64_peak else None,
                 "traffic": None,
                 "peak_source": "FP64 DFMA pipe: %d SMs x 4 flop/clk x %.0f MHz (sampled SM clock)" % (n_sms, sm_mhz),
-                "frac_of_occupied_sms": achieved / occupied if occupied else None,
                 "launch_ms_avg": avg, "launches": nt * args.steps, "flops_per_launch": fl,
                 "flops_counted": "algorithmic: m^3/3 (Cholesky of the diagonal tile)",
                 "executed_flops_per_launch": 2.0 * fl,
